@@ -229,10 +229,11 @@ def work(case):
 
 def tolerance(case):
     """Everything but the scorer is whole numbers, defined to the last bit.  The scorer's cost is a dozen fp32 operations
-    (measured: 3e-8 in the 2-norm and 2.5e-7 at most against 64 bits); an argmin may differ where two instances' costs
-    are a few fp32 roundings apart (measured: 2 in 10^6 requests)."""
+    (against 64 bits over 42 inputs: 3e-8 to 7e-8 in the 2-norm, 2e-7 at most).  An argmin may differ where two
+    instances' costs are within a few fp32 roundings of each other; predicted lengths are whole numbers, so all requests
+    of one length (up to 0.3 % of them) stand at such a tie together (seen in none of the 42)."""
     if case["kind"] == "score":
-        return {"rel": 2e-7, "max": 1e-6, "differ": min(0.01, max(1e-5, 2 / case["n"]))}
+        return {"rel": 3e-7, "max": 8e-7, "differ": min(0.01, max(4e-3, 2 / case["n"]))}
     return "exact"
 
 
