@@ -200,15 +200,20 @@ size_t ctr_workspace_bytes(int32_t which, const ctr_sim_cfg* cfg, int64_t n_rows
     if (which != CTR_WS_SIMULATE || !valid_sim_cfg(cfg) || n_rows < 0) return 0;
     int64_t off_act = 0, off_wait = 0;
     int32_t cap_pr = 0;
-    const int64_t slot = sim_slot_bytes(*cfg, &off_act, &off_wait, &cap_pr);
     int wpb = 0, blocks = 0;
     const int64_t resident = sim_max_resident_warps(&wpb, &blocks);
     if (resident <= 0) return 0;
-    // one slot per persistent warp, and a warp carries 32 / width rows
-    const int64_t rows_per_warp = 32 / sim_group_width(cfg->n_prefill + cfg->n_decode);
-    const int64_t warps = (n_rows + rows_per_warp - 1) / rows_per_warp;
-    const int64_t slots = warps < resident ? (warps > 0 ? warps : 1) : resident;
-    return (size_t)(256 + slots * slot);
+    // one slot per persistent warp: with the pool's full warps (every workspace has room for one of
+    // those), and with the rows spread as ctr_simulate spreads them
+    const int width = sim_group_width(cfg->n_prefill + cfg->n_decode);
+    int64_t most = 0;
+    for (const int rpw : {32 / width, sim_rows_per_warp(width, n_rows)}) {
+        const int64_t slot = sim_slot_bytes(*cfg, width * rpw, &off_act, &off_wait, &cap_pr);
+        const int64_t warps = (n_rows + rpw - 1) / rpw;
+        const int64_t slots = warps < resident ? (warps > 0 ? warps : 1) : resident;
+        most = slots * slot > most ? slots * slot : most;
+    }
+    return (size_t)(256 + most);
 }
 
 int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t n_const_sets,
@@ -293,16 +298,26 @@ int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t 
         d.poll_recip = k.occupancy_poll_us > 0 ? ~0ull / (uint64_t)k.occupancy_poll_us : 0;
     }
 
-    p.slot_bytes = sim_slot_bytes(*cfg, &p.off_act, &p.off_wait, &p.cap_pr);
+    p.slot_bytes = sim_slot_bytes(*cfg, kWarp, &p.off_act, &p.off_wait, &p.cap_pr);
     int wpb = 0, blocks_max = 0;
     const int64_t resident = sim_max_resident_warps(&wpb, &blocks_max);
     if (resident <= 0) return CTR_ECUDA;
     if (workspace_bytes < 256 + (size_t)p.slot_bytes) return CTR_EINVAL;
-    int64_t slots = (int64_t)((workspace_bytes - 256) / (size_t)p.slot_bytes);
-    if (slots > resident) slots = resident;
-    const int64_t rows_per_warp = 32 / sim_group_width(cfg->n_prefill + cfg->n_decode);
-    const int64_t warps_needed = (n_rows + rows_per_warp - 1) / rows_per_warp;
-    if (slots > warps_needed) slots = warps_needed;
+    p.row_lanes = sim_group_width(cfg->n_prefill + cfg->n_decode);
+    const int full = 32 / p.row_lanes;
+    int64_t slots = 0;
+    // spread the rows over more warps only where the workspace holds a slot for each of them
+    for (int rpw = sim_rows_per_warp(p.row_lanes, n_rows);; rpw *= 2) {
+        p.slot_bytes = sim_slot_bytes(*cfg, p.row_lanes * rpw, &p.off_act, &p.off_wait, &p.cap_pr);
+        slots = (int64_t)((workspace_bytes - 256) / (size_t)p.slot_bytes);
+        if (slots > resident) slots = resident;
+        const int64_t warps_needed = (n_rows + rpw - 1) / rpw;
+        p.rows_per_warp = rpw;
+        if (slots >= warps_needed || rpw >= full) {
+            if (slots > warps_needed) slots = warps_needed;
+            break;
+        }
+    }
     p.n_slots = (int32_t)slots;
     p.ws = static_cast<unsigned char*>(workspace) + 256;
     p.next_row = static_cast<uint32_t*>(workspace);

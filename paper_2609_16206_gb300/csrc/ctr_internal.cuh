@@ -162,6 +162,8 @@ struct SimParams {
     int64_t off_act, off_wait;  // byte offsets of the active heap and waiting ring inside a slot
     int32_t cap_pr;             // max(cap_pend_store, cap_ring): entries of the first region
     int32_t n_slots;
+    int32_t row_lanes;          // lanes of a slot that belong to one row: sim_group_width of the pool
+    int32_t rows_per_warp;      // rows that share a warp, each 32 / rows_per_warp lanes wide
     ctr_requests trace;
     uint8_t* i_pre;
     uint8_t* i_dec;
@@ -173,9 +175,12 @@ struct SimParams {
     int64_t trace_len;          // entries of each trace array (replicas x requests)
     int64_t out_len;            // entries of each per-request output (rows x requests)
 };
-int64_t sim_slot_bytes(const ctr_sim_cfg& cfg, int64_t* off_act, int64_t* off_wait, int32_t* cap_pr);
+// workspace bytes of one warp whose slot holds `lanes` lanes' structures
+int64_t sim_slot_bytes(const ctr_sim_cfg& cfg, int lanes, int64_t* off_act, int64_t* off_wait, int32_t* cap_pr);
 int sim_max_resident_warps(int* warps_per_block, int* blocks);
-int sim_group_width(int n_instances);  // lanes per simulated row; 32 / width rows share a warp
+int sim_group_width(int n_instances);  // lanes that one simulated row needs; at most 32 / width rows share a warp
+// rows that share a warp in a launch of n_rows rows, a power of two from 1 to 32 / width
+int sim_rows_per_warp(int width, int64_t n_rows);
 cudaError_t launch_sim(const SimParams& p, int blocks, int warps_per_block, cudaStream_t stream);
 // The first-token and completion checksum terms in a pass of their own (when no
 // goodput pass adds them); kmix as for GoodputParams, or null.

@@ -66,7 +66,7 @@ int ctr_simulate_noalloc(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, 
     if (cfg->cap_pending >= 1 && cfg->cap_waiting >= 1 && cfg->cap_active >= 1 && cfg->cap_prefill_ring >= 1 &&
         cfg->cap_pending <= (1 << 20) && cfg->cap_waiting <= (1 << 20) && cfg->cap_active <= (1 << 20) &&
         cfg->cap_prefill_ring <= (1 << 20)) {
-        const int64_t slot = ctr::sim_slot_bytes(*cfg, &off_act, &off_wait, &cap_pr);
+        const int64_t slot = ctr::sim_slot_bytes(*cfg, ctr::kWarp, &off_act, &off_wait, &cap_pr);
         if (256 + slot > (int64_t)kScratchBytes) return CTR_EINVAL;  // one warp's structures do not fit
     }
     void* scratch = nullptr;

@@ -4,7 +4,8 @@
 // sec. III-A and the sec. IV-C baselines.
 //
 // Layout: a row is (replica x cost-constant set x policy); a lane group of G
-// lanes (G = the next power of two >= the pool size) simulates one row, lane
+// lanes (a power of two >= the pool size: the next one in large launches, up to
+// a whole warp in small ones, see sim_rows_per_warp) simulates one row, lane
 // i < n_pre being prefill instance i and lane n_pre + d decode instance d, and
 // a warp carries 32 / G rows side by side (the policies of one replica, which
 // share arrival times).  Warps are persistent and pull row groups from an
@@ -489,10 +490,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
     if (slot >= P.n_slots) return;
     unsigned char* sb = P.ws + slot * P.slot_bytes;
     const int64_t pr_stride = heap_stride(P.cap_pr);
-    uint64_t* pend = reinterpret_cast<uint64_t*>(sb) + lane * pr_stride;  // decode lanes: 4-ary heap
-    int64_t* ring = reinterpret_cast<int64_t*>(sb) + lane * pr_stride;    // prefill lanes: ring from 0
-    uint64_t* act = reinterpret_cast<uint64_t*>(sb + P.off_act) + lane * heap_stride(P.cap_act);
-    uint32_t* wait = reinterpret_cast<uint32_t*>(sb + P.off_wait) + lane * P.cap_wait;
+    // the lane's place in the slot, which holds row_lanes lanes a row (lanes past a row's instances use none)
+    const int sl = grp * P.row_lanes + gl;
+    uint64_t* pend = reinterpret_cast<uint64_t*>(sb) + sl * pr_stride;  // decode lanes: 4-ary heap
+    int64_t* ring = reinterpret_cast<int64_t*>(sb) + sl * pr_stride;    // prefill lanes: ring from 0
+    uint64_t* act = reinterpret_cast<uint64_t*>(sb + P.off_act) + sl * heap_stride(P.cap_act);
+    uint32_t* wait = reinterpret_cast<uint32_t*>(sb + P.off_wait) + sl * P.cap_wait;
 
     const bool is_pre = gl < P.n_pre;
     const bool is_dec = gl >= P.n_pre && gl < P.n_pre + P.n_dec;
@@ -599,7 +602,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                     if (is_dec && live) {
                         int pos = h_i;
                         for (int32_t m = 0; m < m_i; ++m) {
-                            const int64_t v = ck_ld(rings + src * pr_stride, pos, (int64_t)P.cap_ring, oob);
+                            const int64_t v = ck_ld(rings + (grp * P.row_lanes + i) * pr_stride, pos, (int64_t)P.cap_ring, oob);
                             if ((int)((v >> kRingPBits) & 31) == gl - P.n_pre) {
                                 const int64_t ready = e_i + P.xfer_tok * (v & kRingPMask);
                                 if (s.pend_n == P.cap_pend_store) {
@@ -902,13 +905,13 @@ __global__ void __launch_bounds__(kHashThreads) hash_kernel(const __grid_constan
 
 }  // namespace
 
-int64_t sim_slot_bytes(const ctr_sim_cfg& cfg, int64_t* off_act, int64_t* off_wait, int32_t* cap_pr)
+int64_t sim_slot_bytes(const ctr_sim_cfg& cfg, int lanes, int64_t* off_act, int64_t* off_wait, int32_t* cap_pr)
 {
     const int64_t pend_store = (int64_t)cfg.cap_pending + cfg.cap_waiting + 1;  // pending heap entries
     const int64_t pr = pend_store > cfg.cap_prefill_ring ? pend_store : cfg.cap_prefill_ring;
-    const int64_t a = heap_stride(pr) * 8 * kWarp;
-    const int64_t b = a + heap_stride(cfg.cap_active) * 8 * kWarp;
-    const int64_t c = b + (int64_t)cfg.cap_waiting * 4 * kWarp;
+    const int64_t a = heap_stride(pr) * 8 * lanes;
+    const int64_t b = a + heap_stride(cfg.cap_active) * 8 * lanes;
+    const int64_t c = b + (int64_t)cfg.cap_waiting * 4 * lanes;
     *off_act = a;
     *off_wait = b;
     *cap_pr = (int32_t)pr;
@@ -918,6 +921,24 @@ int64_t sim_slot_bytes(const ctr_sim_cfg& cfg, int64_t* off_act, int64_t* off_wa
 int sim_group_width(int n_instances)
 {
     return n_instances <= 4 ? 4 : n_instances <= 8 ? 8 : n_instances <= 16 ? 16 : 32;
+}
+
+// Rows of a launch are spread over more warps, fewer to a warp, while that
+// leaves at most kSpreadWarps warps an SM: a warp of one row has fewer diverged
+// event sequences to serialise (2,000 requests on 2P+6D, four policies: 6.2 ms
+// a row alone, 7.7 ms two, 8.8 ms four to a warp), and as long as few warps share an SM
+// a launch lasts as long as one warp.  With more of them the issue slots run
+// out and packing wins: rows = 2,048 take 8.5 / 8.5 / 8.9 ms with 1 / 2 / 4 to a
+// warp, 3,072 take 10.1 / 9.3 / 10.2, 4,096 take 12.3 / 10.5 / 10.3.
+constexpr int kSpreadWarps = 14;
+int sim_rows_per_warp(int width, int64_t n_rows)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 32 / width;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 32 / width;
+    int rpw = 1;
+    while (rpw < 32 / width && (n_rows + rpw - 1) / rpw > (int64_t)sms * kSpreadWarps) rpw *= 2;
+    return rpw;
 }
 
 int sim_max_resident_warps(int* warps_per_block, int* blocks)
@@ -967,7 +988,7 @@ cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
 template <int kMode>
 cudaError_t launch_mode(const SimParams& p, int blocks, cudaStream_t stream)
 {
-    switch (sim_group_width(p.n_pre + p.n_dec)) {
+    switch (32 / p.rows_per_warp) {
     case 4: return launch_width<4, kMode>(p, blocks, stream);
     case 8: return launch_width<8, kMode>(p, blocks, stream);
     case 16: return launch_width<16, kMode>(p, blocks, stream);

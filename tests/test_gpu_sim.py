@@ -116,6 +116,24 @@ def test_small_workspace_same_results(orc):
         assert np.array_equal(full[key], small[key]), key
 
 
+@pytest.mark.parametrize("sc", [W.SimCfg(), W.SimCfg(n_prefill=2, n_decode=6), W.SimCfg(n_prefill=3, n_decode=9),
+                                W.SimCfg(n_prefill=2, n_decode=6, prefill_batch_tokens=4096)],
+                         ids=["1p3d", "2p6d", "3p9d", "batched"])
+@pytest.mark.parametrize("R,deployed", [(1, 0), (5, 1), (430, 0), (859, 1), (1100, 0)])
+def test_rows_per_warp_same_results(orc, sc, R, deployed):
+    """Few rows get a warp each, more share one (2,150 rows: two to a warp, 4,295: four), and a workspace of one
+    slot packs as many as the pool allows: the same rows, and the oracle's."""
+    ctr = need_gpu()
+    sets = [W.as_deployed(W.CALIBRATED) if deployed else W.CALIBRATED]
+    pols, N = list(W.ALL_POLICIES) + [W.POLICY_LEARNED_P2], 37
+    tr = gen(ctr, W.replica_sweep().trace, R, N)
+    spread = simulate(ctr, sc, sets, pols, tr, R, N)
+    packed = simulate(ctr, sc, sets, pols, tr, R, N, ws_bytes=ctr.ctr_workspace_bytes(0, sc, 1, N))
+    for key in spread:
+        assert np.array_equal(spread[key], packed[key]), key
+    _check_rows(orc, sc, sets, pols, [host_trace(tr, r) for r in range(min(R, 3))], spread, N)
+
+
 def test_routes_optional(orc):
     ctr = need_gpu()
     wl = W.replica_sweep()
