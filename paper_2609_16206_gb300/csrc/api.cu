@@ -242,7 +242,7 @@ int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t 
     p.n_pre = cfg->n_prefill;
     p.n_dec = cfg->n_decode;
     p.kv_cap = cfg->kv_cap_tokens;
-    p.kv_cap_recip = ~0ull / (uint64_t)cfg->kv_cap_tokens;
+    p.kv_cap_magic = in_range(cfg->kv_cap_tokens, 2, (1LL << 23) - 1) ? ~0ull / (uint64_t)cfg->kv_cap_tokens + 1 : 0;
     p.pre_base = cfg->pre_base_us;
     p.pre_tok = cfg->pre_us_per_tok;
     p.xfer_tok = cfg->xfer_us_per_tok;

@@ -142,7 +142,7 @@ struct ConstsDev {
 struct SimParams {
     int32_t n_pre, n_dec;
     int64_t kv_cap;
-    uint64_t kv_cap_recip;      // floor((2^64 - 1) / kv_cap)
+    uint64_t kv_cap_magic;      // ceil(2^64 / kv_cap) for 2 <= kv_cap < 2^23, else 0 (see sim.cu's pressure)
     int64_t pre_base, pre_tok, xfer_tok;
     int64_t dec_base, dec_seq;
     int64_t kv_div;

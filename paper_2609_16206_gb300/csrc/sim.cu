@@ -52,15 +52,17 @@ constexpr int kRingPBits = 21;  // prefill ring entry: end << 21 | p (p <= 2^20)
 constexpr int64_t kRingPMask = (int64_t(1) << kRingPBits) - 1;
 constexpr int kRingKShift = 26;  // batched prefill ring entry: k << 26 | d << 21 | p
 
-// floor((2^64 - 1) / n) for n = 1..kRecipN, for the decode backlog's division
-// by the batch size (built at compile time, read through the read-only path)
+// ceil(2^64 / n) for n = 2..kRecipN, for the decode backlog's division by the
+// batch size (built at compile time, read through the read-only path):
+// floor(x / n) is the high word of x * v[n], exactly, while x < 2^54 (the
+// product exceeds x / n by x e / (n 2^64) with e = v[n] n - 2^64 < n <= 2^10)
 struct RecipTable {
     uint64_t v[kRecipN + 1];
 };
 constexpr RecipTable make_recip_table()
 {
     RecipTable t{};
-    for (int i = 1; i <= kRecipN; ++i) t.v[i] = ~0ull / (uint64_t)i;
+    for (int i = 2; i <= kRecipN; ++i) t.v[i] = ~0ull / (uint64_t)i + 1;
     return t;
 }
 __device__ const RecipTable kRecipTable = make_recip_table();
@@ -78,28 +80,12 @@ __device__ __forceinline__ uint64_t div_recip(uint64_t num, uint64_t d, uint64_t
     return q;
 }
 
-// floor(x / d) for 0 <= x < 2^56 and 0 < d < 2^37: an fp32 estimate (both
-// operands rounded to fp32, relative error of the quotient a few 2^-24), then
-// exact integer correction (the estimate is within one unit of the quotient
-// whenever the quotient is below 2^20, the only case the simulator asks for;
-// larger quotients fall back to division).
-__device__ __forceinline__ int64_t floor_div_small(int64_t x, int64_t d)
+// An estimate of x / d for 0 <= x < 2^31 and 1 <= d < 2^31 whose quotient is
+// below 2^20: both operands rounded to fp32 and a divide good to a few 2^-24,
+// so it is off by less than one unit either way.
+__device__ __forceinline__ int32_t div_estimate(int32_t x, int32_t d)
 {
-    const float xf = __ll2float_rn(x);
-    const float df = __ll2float_rn(d);
-    const float qf = __fdividef(xf, df);
-    if (!(qf < 1048576.0f)) return x / d;
-    int32_t q = __float2int_rz(qf);  // within one of the quotient, below 2^20
-    int64_t r = x - (int64_t)q * d;
-    while (r < 0) {
-        --q;
-        r += d;
-    }
-    while (r >= d) {
-        ++q;
-        r -= d;
-    }
-    return q;
+    return __float2int_rz(__fdividef(__int2float_rn(x), __int2float_rn(d)));
 }
 
 // floor(x / kv_div) for 0 <= x < 2^32 with magic = ceil(2^64 / kv_div), exact: the
@@ -251,29 +237,80 @@ __device__ __forceinline__ int warp_argmin(uint64_t v)
     return __ffs(ball) - 1;
 }
 
-// A decode lane's state.  `sum` is the one in-flight sum the row's policy
-// reads: the true remaining output tokens R for the learned router on the true
-// backlog, the predicted lengths o_hat for the length heuristic and the proxy's
-// ledger (sum_is_o_hat), nothing for the others.
+// A decode lane's state.  Its next event is the end of a step at which
+// something can change (a completion, an admission, the floor(KV / kv_div) term
+// of the step time), and the steps before it are a run of equal ones, left as
+// they are until the event: the running step ends at step_end, `run` more of
+// `step` us follow, and the event is at step_end + run * step.  An idle lane
+// (n_act = 0) has run = 0 and step_end the time of its next KV-ready request
+// (kNever without one).  run * step stays below 2^31, so a time inside the run
+// is a 32-bit offset from step_end.  step_idx, kv_res and a true-backlog sum
+// are the values before the step that ends at step_end.
+// `sum` is the one in-flight sum the row's policy reads: the true remaining
+// output tokens R for the learned router on the true backlog, the predicted
+// lengths o_hat for the length heuristic and the proxy's ledger
+// (sum_is_o_hat), nothing for the others.
 struct Decode {
     int64_t step_end, sum;
+    int32_t run, step;
     int32_t step_idx;        // steps ended; the step budget keeps it and every completion step below 2^31
     int32_t kv_res, kv_rsv;  // resident <= reserved <= C < 2^31 tokens
     uint64_t pend_top, act_top;
     int32_t n_act, q, pend_n, w_head, w_n;  // n_act is also the active heap's size
-    bool stepping;
 };
 
-// Move every pending request whose KV is ready by t into the waiting FIFO, in
-// (time, index) order; the FIFO's size is checked after each insertion.
+__device__ __forceinline__ int64_t next_event(const Decode& s) { return s.step_end + (int64_t)s.run * s.step; }
+
+// Steps of the run that have ended by t, for t before the next event: exact
+// (the quotient is below run <= 2^20).
+__device__ __forceinline__ int32_t ends_by(const Decode& s, int64_t t)
+{
+    if (s.n_act == 0 || t < s.step_end) return 0;
+    const int32_t dt = (int32_t)(t - s.step_end);
+    int32_t q = div_estimate(dt, s.step);
+    const int32_t r = dt - q * s.step;
+    q += (r >= s.step) - (r < 0);
+    return q + 1;
+}
+
+// A request becomes KV-ready at tp: the event moves up to the first step end at
+// or after tp (or, where the estimate is one low, to the end before it, an event
+// at which nothing changes).
+__device__ __forceinline__ void cut_run(Decode& s, int64_t tp)
+{
+    if (tp <= s.step_end) {
+        s.run = 0;
+    } else if (tp < next_event(s)) {
+        const int32_t rel = (int32_t)(tp - s.step_end);
+        int32_t q = div_estimate(rel, s.step);
+        q += rel > q * s.step;
+        s.run = q;
+    }
+}
+
+// A new key of the pending heap (ready at key >> 23).  While requests wait for
+// admission (w_n > 0) the next event does not depend on it: either the head
+// waits for a completion, or an event no later than this one is set already.
 template <int kArity>
-__device__ __forceinline__ int flush_ready(Decode& s, int64_t t, const SimParams& P, uint64_t* pend, uint32_t* wait,
-                                           bool& bad)
+__device__ __forceinline__ void push_pending(Decode& s, uint64_t* pend, uint64_t key, int64_t lim, bool& bad)
+{
+    hpush<kArity == 2>(pend, s.pend_n, s.pend_top, key, lim, bad);
+    if (s.n_act == 0)
+        s.step_end = (int64_t)(s.pend_top >> kKeyBits);
+    else if (s.w_n == 0)
+        cut_run(s, (int64_t)(key >> kKeyBits));
+}
+
+// Move every pending request whose KV is ready by t into the waiting FIFO, in
+// (time, index) order; room is what the FIFO can still take.
+template <int kArity>
+__device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, const SimParams& P, uint64_t* pend,
+                                           uint32_t* wait, bool& bad)
 {
     while (s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= t) {
         const uint32_t k = (uint32_t)(s.pend_top & kKeyMask);
         hpop<kArity == 2>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
-        if (s.w_n == P.cap_wait) return CTR_EOVERFLOW;
+        if (--room < 0) return CTR_EOVERFLOW;
         int pos = s.w_head + s.w_n;
         if (pos >= P.cap_wait) pos -= P.cap_wait;
         ck_st(wait, pos, P.cap_wait, k, bad);
@@ -282,133 +319,123 @@ __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, const SimParams
     return CTR_OK;
 }
 
-// Advance one decode instance through every event at times <= T.  The pending
-// heap may hold requests already KV-ready (taken at the next step end); it has
-// room for cap_pend + cap_wait + 1 entries, so a full heap means the waiting
-// FIFO has overflowed.  kSnap: when tsnap >= 0, also record in kv_snap the
-// resident KV as it is after every event at times <= tsnap (an occupancy
-// poll; tsnap <= T), then set tsnap to -1.
+// One event of a decode instance (at next_event): the run's steps end, requests
+// that finish with the last one complete, those KV-ready by then are admitted
+// strictly FCFS while the reservation fits, the next step starts and the next
+// event is set.  The pending heap may hold requests already KV-ready (a
+// KV-ready event while a step runs only matters at the step's end; while the
+// FIFO's head waits for room, at the next completion); it has room for
+// cap_pend + cap_wait + 1 entries, so a full heap means the waiting FIFO has
+// overflowed.
+template <int kArity>
+__device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimParams& P, uint64_t* pend, uint64_t* act,
+                                            uint32_t* wait, int64_t tb, int64_t ob, bool sum_is_o_hat, bool& bad)
+{
+    if (tev >= kTimeLimit) return CTR_EOVERFLOW;
+    if (s.n_act > 0) {  // (1) run + 1 steps end: as many tokens for every active request
+        const int32_t ends = s.run + 1;
+        const int32_t tokens = ends * s.n_act;  // within the reservation
+        s.step_idx += ends;
+        s.kv_res += tokens;
+        if (!sum_is_o_hat) s.sum -= tokens;
+        if (s.step_idx > (int32_t)P.max_steps) return CTR_ETIMEOUT;
+        while (s.n_act > 0 && (int32_t)(s.act_top >> kKeyBits) == s.step_idx) {
+            const int64_t k = (int64_t)(s.act_top & kKeyMask);
+            const int32_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
+            const int32_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
+            if (sum_is_o_hat) s.sum -= ck_ldg(P.trace.pred_out, tb + k, P.trace_len, bad);
+            ck_st(P.t_done, ob + k, P.out_len, tev, bad);
+            hpop<kArity == 2>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
+            s.q -= 1;
+            s.kv_res -= pk + ok;
+            s.kv_rsv -= pk + ok;
+        }
+    }
+    // (2) admission in FCFS order: the waiting FIFO, then the requests KV-ready by now in (time, index)
+    // order, which join the FIFO once its head does not fit.  Before any admission the FIFO holds all of
+    // them, so its room counts those admitted from the pending heap too.
+    int32_t room = P.cap_wait - s.w_n;
+    int32_t admitted = 0;
+    uint32_t last = 0;  // the request admitted last; the others are chained through their t_first entries
+    for (;;) {
+        const bool fifo = s.w_n > 0;
+        if (!fifo && !(s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= tev)) break;
+        const uint32_t k = fifo ? ck_ld(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
+        const int32_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
+        const int32_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
+        if ((uint32_t)s.kv_rsv + (uint32_t)(pk + ok) > (uint32_t)P.kv_cap) {  // < 2^31 + 2^21
+            const int rc = flush_ready<kArity>(s, tev, room, P, pend, wait, bad);
+            if (rc != CTR_OK) return rc;
+            break;
+        }
+        if (s.n_act == P.cap_act) return CTR_EOVERFLOW;
+        if (fifo) {
+            s.w_n -= 1;
+            s.w_head = s.w_n == 0 || s.w_head + 1 == P.cap_wait ? 0 : s.w_head + 1;  // an empty ring restarts at 0
+        } else {
+            hpop<kArity == 2>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
+            if (--room < 0) return CTR_EOVERFLOW;
+        }
+        s.kv_rsv += pk + ok;
+        s.kv_res += pk;
+        hpush<kArity == 2>(act, s.n_act, s.act_top, ((uint64_t)(uint32_t)(s.step_idx + ok) << kKeyBits) | k,
+                           heap_stride(P.cap_act), bad);
+        if (admitted > 0) ck_st(P.t_first, ob + k, P.out_len, (int64_t)last, bad);
+        last = k;
+        admitted += 1;
+    }
+    // (3) the next step and the next event
+    const int64_t tp = s.pend_n > 0 ? (int64_t)(s.pend_top >> kKeyBits) : kNever;
+    if (s.n_act == 0) {
+        s.step_end = tp;
+        s.run = 0;
+        return CTR_OK;
+    }
+    if (s.step_idx >= (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
+    const int32_t n = s.n_act;
+    const int64_t fixed = P.dec_base + (int64_t)(int32_t)P.dec_seq * n;
+    s.step_end = tev + fixed + kv_term(s.kv_res, P);
+    for (; admitted > 0; --admitted) {  // first token at the end of this step
+        const int64_t prev = admitted > 1 ? ck_ld(P.t_first, ob + last, P.out_len, bad) : 0;
+        ck_st(P.t_first, ob + last, P.out_len, s.step_end, bad);
+        last = (uint32_t)prev;
+    }
+    // after j of the run's ends the KV term is that of kv_res + j n, and it stays q1 while j n <= room1
+    // (q1 + 1 <= 2^31 and kv_div <= 2^31; the sum is below 2^32)
+    const int64_t q1 = kv_term(s.kv_res + n, P);
+    const uint32_t room1 = (uint32_t)(q1 + 1) * (uint32_t)P.kv_div - 1u - (uint32_t)s.kv_res;
+    int32_t m = (int32_t)(s.act_top >> kKeyBits) - s.step_idx - 1;  // plain ends before the next completion, <= 2^20
+    if ((uint64_t)(uint32_t)m * (uint32_t)n > room1) {  // the term changes first: at most room1 / n (one less is fine)
+        m = __float2int_rz(__fdividef(__uint2float_rn(room1), __int2float_rn(n)));
+        m -= (uint64_t)(uint32_t)m * (uint32_t)n > room1;
+    }
+    const int64_t step = fixed + q1;
+    if (((int64_t)m * step) >> 31) m = step >> 31 ? 0 : (int32_t)(0x7fffffffu / (uint32_t)step);
+    s.step = (int32_t)step;  // a step of 2^31 us or more has m = 0
+    s.run = m;
+    if (s.w_n == 0 && s.pend_n > 0) cut_run(s, tp);
+    return CTR_OK;
+}
+
+// Advance one decode instance through every event at times <= T.  kSnap: when
+// tsnap >= 0, also record in kv_snap the resident KV as it is after every event
+// at times <= tsnap (an occupancy poll; tsnap <= T).
 template <bool kSnap, int kArity>
 __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimParams& P, uint64_t* pend, uint64_t* act,
-                                              uint32_t* wait, int64_t tb, int64_t ob, int64_t& tsnap, int64_t& kv_snap,
+                                              uint32_t* wait, int64_t tb, int64_t ob, int64_t tsnap, int64_t& kv_snap,
                                               bool sum_is_o_hat, bool& bad)
 {
     for (;;) {
-        // Plain step ends first: the step ends by T, no request finishes with
-        // it, nothing has become KV-ready by then and nobody waits for
-        // admission, so the batch is unchanged and the next step starts at
-        // once.  Lanes leave this loop at their next non-plain event, which
-        // the handler below takes.
-        const int64_t tp = s.pend_n > 0 ? (int64_t)(s.pend_top >> kKeyBits) : kNever;
-        const int64_t limit = tp <= T ? tp - 1 : T;  // plain step ends lie at or before limit
-        // The run is taken in closed form: while the floor(KV / kv_div) term of
-        // the step time is unchanged every step lasts S, so the number of plain
-        // ends is the least of the steps before the next completion, the steps
-        // before that term changes, and the steps that end by the limit.
-        while (s.stepping && s.step_end <= limit && s.w_n == 0) {
-            const int32_t m_fin = (int32_t)(s.act_top >> kKeyBits) - s.step_idx - 1;  // <= 2^20
-            if (m_fin <= 0) break;
-            const int32_t n = s.n_act;
-            const int64_t q1 = kv_term(s.kv_res + n, P);  // KV term of the next step
-            const int64_t S = P.dec_base + (int64_t)(int32_t)P.dec_seq * n + q1;
-            // plain end j happens at step_end + (j - 1) S <= limit (usually the binding bound)
-            int32_t m = (int32_t)m_fin;
-            const int64_t span = limit - s.step_end;
-            if ((int64_t)(m - 1) * S > span) {  // then span < 2^20 * 2^37
-                m = (int32_t)(span < (int64_t(1) << 56) ? floor_div_small(span, S) : span / S) + 1;
-            }
-            // the term stays q1 while j n <= room; q1 + 1 <= 2^31 and kv_div <= 2^31
-            const int64_t room = (int64_t)((uint64_t)(uint32_t)(q1 + 1) * (uint32_t)P.kv_div) - 1 - s.kv_res;
-            if ((int64_t)m * n > room) {  // the KV term changes first: m = floor(room / n) >= 1
-                m = n <= kRecipN ? (int32_t)div_recip((uint64_t)room, (uint64_t)n, __ldg(&kRecipTable.v[n]))
-                                 : (int32_t)(room / n);
-            }
-            if constexpr (kSnap) {
-                // the poll instant falls before this run or inside it: the occupancy
-                // there follows from the number of the run's ends by then
-                if (tsnap >= 0) {
-                    if (tsnap < s.step_end) {
-                        kv_snap = s.kv_res;
-                        tsnap = -1;
-                    } else if (tsnap < s.step_end + (int64_t)(m - 1) * S) {
-                        const int64_t d = tsnap - s.step_end;  // < (m - 1) S < 2^57
-                        const int64_t j = (d < (int64_t(1) << 56) ? floor_div_small(d, S) : d / S) + 1;
-                        kv_snap = s.kv_res + j * (int64_t)n;
-                        tsnap = -1;
-                    }
-                }
-            }
-            const int64_t mn = (int64_t)m * n;
-            s.step_idx += m;
-            s.kv_res += (int32_t)mn;  // stays within the reservation
-            if (!sum_is_o_hat) s.sum -= mn;  // R: every active request is one token closer
-            if (s.step_idx >= (int32_t)P.max_steps) return CTR_ETIMEOUT;
-            s.step_end += (int64_t)m * S;
-            if (s.step_end >= kTimeLimit) return CTR_EOVERFLOW;
-        }
-        // A KV-ready event while a step runs only matters at the step's end (the
-        // next admission), so it is taken there, in the same pass: the next
-        // event is the running step's end, or the next KV-ready when idle.
-        const int64_t tev = s.stepping ? s.step_end : tp;
+        const int64_t tev = next_event(s);
         if constexpr (kSnap) {
-            if (tsnap >= 0 && tev > tsnap) {  // every event by the poll instant is done
-                kv_snap = s.kv_res;
+            if (tsnap >= 0 && tev > tsnap) {
+                kv_snap = s.kv_res + ends_by(s, tsnap) * s.n_act;
                 tsnap = -1;
             }
         }
         if (tev > T) return CTR_OK;
-        if (s.stepping) {  // (1) the running step ends: one token for every active request
-            s.step_idx += 1;
-            s.kv_res += s.n_act;
-            if (!sum_is_o_hat) s.sum -= s.n_act;
-            s.stepping = false;
-            while (s.n_act > 0 && (int32_t)(s.act_top >> kKeyBits) == s.step_idx) {
-                const int64_t k = (int64_t)(s.act_top & kKeyMask);
-                hpop<kArity == 2>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
-                const int64_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
-                const int64_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
-                s.q -= 1;
-                s.kv_res -= (int32_t)(pk + ok);
-                s.kv_rsv -= (int32_t)(pk + ok);
-                if (sum_is_o_hat) s.sum -= ck_ldg(P.trace.pred_out, tb + k, P.trace_len, bad);
-                ck_st(P.t_done, ob + k, P.out_len, tev, bad);
-            }
-        }
-        // (2) every request KV-ready by now joins the waiting FIFO in (time, index) order
-        const int rc = flush_ready<kArity>(s, tev, P, pend, wait, bad);
+        const int rc = decode_event<kArity>(s, tev, P, pend, act, wait, tb, ob, sum_is_o_hat, bad);
         if (rc != CTR_OK) return rc;
-        // (3) not mid-step: strict FCFS admission while the reservation fits, then start a step
-        if (!s.stepping) {
-            const int pos0 = s.w_head;
-            int admitted = 0;
-            while (s.w_n > 0) {
-                const uint32_t k = ck_ld(wait, s.w_head, P.cap_wait, bad);
-                const int64_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
-                const int64_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
-                if ((uint32_t)s.kv_rsv + (uint32_t)(pk + ok) > (uint32_t)P.kv_cap) break;  // < 2^31 + 2^21
-                if (s.n_act == P.cap_act) return CTR_EOVERFLOW;
-                s.w_head = s.w_head + 1 == P.cap_wait ? 0 : s.w_head + 1;
-                s.w_n -= 1;
-                s.kv_rsv += (int32_t)(pk + ok);
-                s.kv_res += (int32_t)pk;
-                hpush<kArity == 2>(act, s.n_act, s.act_top, ((uint64_t)(s.step_idx + ok) << kKeyBits) | k,
-                                   heap_stride(P.cap_act), bad);
-                admitted += 1;
-            }
-            if (s.n_act > 0) {
-                if (s.step_idx >= (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
-                s.step_end = tev + P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act + kv_term(s.kv_res, P);
-                if (s.step_end >= kTimeLimit) return CTR_EOVERFLOW;
-                s.stepping = true;
-                int pos = pos0;
-                for (int i = 0; i < admitted; ++i) {  // first token at the end of this step
-                    const uint32_t k = ck_ld(wait, pos, P.cap_wait, bad);
-                    ck_st(P.t_first, ob + k, P.out_len, s.step_end, bad);
-                    pos = pos + 1 == P.cap_wait ? 0 : pos + 1;
-                }
-            }
-            if (s.w_n == 0) s.w_head = 0;  // an empty ring restarts at its first entry (stays cache-resident)
-        }
     }
 }
 
@@ -534,10 +561,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         bool live = has_row && valid;
 
         Decode s;
-        s.step_end = 0; s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
+        s.step_end = is_dec ? kNever : 0; s.run = 0; s.step = 1;
+        s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
         s.pend_top = kEmpty; s.act_top = kEmpty;
         s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
-        s.stepping = false;
         // A lane simulates a prefill or a decode instance, never both, so a prefill
         // lane keeps its state in decode fields it does not use (fewer live registers).
         int64_t& busy = s.step_end;    // end of the last prefill (of the running batch, when batched)
@@ -608,9 +635,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                                 if (s.pend_n == P.cap_pend_store) {
                                     err = CTR_EOVERFLOW;  // the waiting FIFO has overflowed
                                 } else {
-                                    hpush<kArity == 2>(pend, s.pend_n, s.pend_top,
-                                              ((uint64_t)ready << kKeyBits) | (uint64_t)(v >> kRingKShift), pr_stride,
-                                              oob);
+                                    push_pending<kArity>(s, pend,
+                                                         ((uint64_t)ready << kKeyBits) | (uint64_t)(v >> kRingKShift),
+                                                         pr_stride, oob);
                                 }
                             }
                             pos = pos + 1 == P.cap_ring ? 0 : pos + 1;
@@ -644,7 +671,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                 }
                 if (live) {
                     if (is_dec) {
-                        int64_t tsnap = -1;
+                        int64_t tsnap = -1;  // >= 0: the occupancy at this time is recorded on the way
                         if (kSig && cc.poll_us > 0) {
                             // the router sees the occupancy of the last poll instant floor(T / D) D,
                             // taken after every event at that instant, on the way to T
@@ -707,25 +734,35 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                     } else if (is_dec) {
                         if (learned) {
                             const int64_t na = s.n_act;
-                            const int64_t step = P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act + kv_term(s.kv_res, P);
-                            const uint64_t hi = __umul64hi((uint64_t)s.sum, (uint64_t)step);
-                            const uint64_t lo = (uint64_t)s.sum * (uint64_t)step;
+                            const int32_t tokens = ends_by(s, T) * s.n_act;  // of the run's steps that have ended
+                            const int32_t kv_live = s.kv_res + tokens;
+                            const uint64_t R = (uint64_t)(s.sum - tokens);  // unread where sum is o_hat
+                            const int64_t step = P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act + kv_term(kv_live, P);
+                            const uint64_t lo = R * (uint64_t)step;
+                            const uint64_t nd = (uint64_t)(na > 1 ? na : 1);
                             int64_t b;
-                            if (hi != 0 || lo >= (1ull << 62)) {
+                            if (((R | ((uint64_t)step << 10)) >> 32) == 0 && nd <= (uint64_t)kRecipN) {  // lo < 2^54
+                                b = (int64_t)(nd > 1 ? __umul64hi(lo, __ldg(&kRecipTable.v[nd])) : lo);
+                            } else if (__umul64hi(R, (uint64_t)step) != 0 || lo >= (1ull << 62)) {
                                 b = kBacklogClamp;
                             } else {
-                                const uint64_t nd = (uint64_t)(na > 1 ? na : 1);
-                                b = (int64_t)(nd <= (uint64_t)kRecipN ? div_recip(lo, nd, __ldg(&kRecipTable.v[nd]))
-                                                                      : lo / nd);
-                                if (b > kBacklogClamp) b = kBacklogClamp;
+                                b = (int64_t)(lo / nd);
                             }
+                            if (b > kBacklogClamp) b = kBacklogClamp;
                             if (kSig && cc.proxy) {  // the ledger: tau_dec o_hat per request routed here and not done
                                 b = (cc.ablate & CTR_ABLATE_PREDICTED_LENGTH) ? 0 : cc.tau_dec * s.sum;
                                 if (b > kBacklogClamp) b = kBacklogClamp;
                             }
-                            const int64_t kv = kSig && cc.poll_us > 0 ? kv_seen : s.kv_res;
-                            int64_t press = (int64_t)div_recip((uint64_t)(kv + pk + oh_f) << 16,
-                                                               (uint64_t)P.kv_cap, P.kv_cap_recip);
+                            const int64_t kv = kSig && cc.poll_us > 0 ? kv_seen : (int64_t)kv_live;
+                            const uint32_t after = (uint32_t)(kv + pk + oh_f);  // < 2^31 + 2^20 + 2^17
+                            int64_t press;
+                            if (P.kv_cap_magic != 0) {
+                                const uint64_t lo = (uint64_t)after * (uint32_t)P.kv_cap_magic;
+                                const uint64_t hi = (uint64_t)after * (uint32_t)(P.kv_cap_magic >> 32);
+                                press = (int64_t)((hi + (lo >> 32)) >> 16);
+                            } else {
+                                press = (int64_t)(((uint64_t)after << 16) / (uint64_t)P.kv_cap);
+                            }
                             if (press > kPressureClamp) press = kPressureClamp;
                             if (cc.ablate & CTR_ABLATE_PRESSURE) press = 0;
                             const int64_t own = oh_f * cc.tau_dec;
@@ -818,14 +855,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                 if (live && gl == P.n_pre + id && ready < kTimeLimit) {
                     // requests routed here whose KV is not ready yet, exactly: first move
                     // those already ready (kept in the heap until the step end) if it matters
-                    if (s.q - s.w_n - s.n_act >= P.cap_pend) err = flush_ready<kArity>(s, T, P, pend, wait, oob);
+                    if (s.q - s.w_n - s.n_act >= P.cap_pend)
+                        err = flush_ready<kArity>(s, T, P.cap_wait - s.w_n, P, pend, wait, oob);
                     if (err != CTR_OK || s.q - s.w_n - s.n_act == P.cap_pend ||
                         (ready >= 0 && s.pend_n == P.cap_pend_store)) {
                         err = CTR_EOVERFLOW;
                     } else {
                         if (ready >= 0)
-                            hpush<kArity == 2>(pend, s.pend_n, s.pend_top, ((uint64_t)ready << kKeyBits) | (uint64_t)k,
-                                               pr_stride, oob);
+                            push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, pr_stride, oob);
                         s.q += 1;
                         s.sum += sum_is_o_hat ? ohk : ok;
                     }
@@ -849,8 +886,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
             }
         }
         if (live && is_dec) {
-            int64_t no_snap = -1;
-            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, tb, ob, no_snap, kv_seen, sum_is_o_hat,
+            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, tb, ob, -1, kv_seen, sum_is_o_hat,
                                                 oob);
         }
 

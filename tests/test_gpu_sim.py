@@ -134,6 +134,41 @@ def test_rows_per_warp_same_results(orc, sc, R, deployed):
     _check_rows(orc, sc, sets, pols, [host_trace(tr, r) for r in range(min(R, 3))], spread, N)
 
 
+@pytest.mark.parametrize("kv_div,o_max", [(1, 1 << 13), (3, 1 << 15), (1 << 20, 1 << 20), (1 << 31, 1 << 20)])
+@pytest.mark.parametrize("dec_base,kv_cap", [(1, (1 << 23) - 1), (3_000, 1 << 23), (3_000, (1 << 31) - 1)])
+def test_long_runs_of_steps(orc, kv_div, o_max, dec_base, kv_cap):
+    """Outputs of up to 2^20 tokens: runs of equal steps from one (the KV term grows every step) to more than 2^31 us,
+    step counts at both ends of the quotient estimates, and the pressure on both sides of its 2^23-token line."""
+    ctr = need_gpu()
+    sc = W.SimCfg(n_prefill=2, n_decode=3, kv_cap_tokens=kv_cap, pre_base_us=1, pre_us_per_tok=0, xfer_us_per_tok=1,
+                  dec_base_us=dec_base, dec_us_per_seq=1, dec_kv_tokens_per_us=kv_div)
+    rng = np.random.default_rng(kv_div % 1009 + dec_base)
+    N = 70
+    trh = {"arrival_us": np.sort(rng.integers(0, o_max * max(dec_base, 4), N)).astype(np.int64),
+           "prompt_len": rng.integers(0, 1 << 20, N).astype(np.int32),
+           "true_out": np.where(rng.random(N) < 0.5, rng.integers(1, 40, N), rng.integers(1, o_max + 1, N)).astype(np.int32),
+           "pred_out": rng.integers(0, 1 << 17, N).astype(np.int32), "slo_class": rng.integers(0, 2, N).astype(np.uint8)}
+    sets = [W.CALIBRATED, W.as_deployed(W.CALIBRATED)]
+    pols = list(W.ALL_POLICIES)
+    res = simulate(ctr, sc, sets, pols, to_dev(trh), 1, N)
+    _check_rows(orc, sc, sets, pols, [trh], res, N)
+
+
+def test_steps_longer_than_31_bits(orc):
+    """36,000 requests on one instance: steps of more than 2^31 us, which never form a run."""
+    ctr = need_gpu()
+    N, cap = 36_000, 1 << 16
+    sc = W.SimCfg(n_prefill=1, n_decode=1, kv_cap_tokens=(1 << 31) - 1, pre_base_us=1, pre_us_per_tok=0, xfer_us_per_tok=0,
+                  dec_base_us=1 << 24, dec_us_per_seq=1 << 16, dec_kv_tokens_per_us=1 << 31, cap_pending=cap,
+                  cap_waiting=cap, cap_active=cap, cap_prefill_ring=cap)
+    trh = {"arrival_us": np.zeros(N, np.int64), "prompt_len": np.full(N, 5, np.int32),
+           "true_out": (np.arange(N) % 4 + 1).astype(np.int32), "pred_out": np.full(N, 3, np.int32),
+           "slo_class": np.zeros(N, np.uint8)}
+    res = simulate(ctr, sc, [W.CALIBRATED], [W.POLICY_LEARNED], to_dev(trh), 1, N)
+    assert res["t_done_us"].max() > 1 << 32
+    _check_rows(orc, sc, [W.CALIBRATED], [W.POLICY_LEARNED], [trh], res, N)
+
+
 def test_routes_optional(orc):
     ctr = need_gpu()
     wl = W.replica_sweep()
