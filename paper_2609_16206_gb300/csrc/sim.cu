@@ -1002,19 +1002,25 @@ int sim_max_resident_warps(int* warps_per_block, int* blocks)
 
 namespace {
 
-// 7 blocks per SM (72 registers a thread, fewer spills) when all of the
-// launch's persistent warps fit on the GPU at that occupancy -- the common
-// case of one row group per warp -- else 8 (more warps to hide latency).
+// The instantiation with the most registers at which all of the launch's
+// persistent warps are resident at once (its launch bound promises that many
+// blocks an SM): 4 blocks / 128 registers for launches of up to 16 warps an SM,
+// which wait on their own chains and not for issue slots, so spills and
+// constants re-read from the parameter bank cost time (256 rows of each kind:
+// document 6.5 -> 5.7 ms, 3,120 learned rows 9.1 -> 8.4 ms against 7 blocks);
+// 7 blocks / 72 registers for one wave of up to 28; else 8 / 64, where more
+// warps hide more latency.
 template <int G, int kMode>
 cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
 {
-    int dev = 0, sms = 0, per_sm7 = 0;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm7, sim_kernel<G, kMode, 7>, kWarpsPerBlock * 32, 0);
-    if (e != cudaSuccess) return e;
-    if ((int64_t)p.n_slots <= (int64_t)sms * per_sm7 * kWarpsPerBlock)
+    const int64_t per_block = (int64_t)sms * kWarpsPerBlock;  // warps at one block an SM
+    if (p.n_slots <= 4 * per_block)
+        sim_kernel<G, kMode, 4><<<blocks, kWarpsPerBlock * 32, 0, stream>>>(p);
+    else if (p.n_slots <= 7 * per_block)
         sim_kernel<G, kMode, 7><<<blocks, kWarpsPerBlock * 32, 0, stream>>>(p);
     else
         sim_kernel<G, kMode, 8><<<blocks, kWarpsPerBlock * 32, 0, stream>>>(p);
