@@ -144,6 +144,7 @@ int ctr_gen_trace(const ctr_trace_cfg* cfg, int32_t n_replicas, int64_t replica_
     p.replica_offset = replica_offset;
     p.n_req = n_req;
     p.out = out;
+    p.minus_zeros = 0x8000000080000000ull;
     return cuda_status(launch_trace(p, (cudaStream_t)stream));
 }
 

@@ -123,6 +123,7 @@ struct TraceParams {
     uint64_t class_thr[3];
     int64_t n_replicas, replica_offset, n_req;
     ctr_requests out;
+    uint64_t minus_zeros;       // two fp32 -0 (see mul2 in trace.cu)
 };
 cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream);
 

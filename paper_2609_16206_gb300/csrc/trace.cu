@@ -1,12 +1,15 @@
 // trace.cu -- synthetic request trace on the GPU (ctr_gen_trace).
 //
-// One warp per replica; lane l owns request base + l of each 32-request
-// chunk.  Per request: two Philox4x32-10 blocks (Salmon et al., SC'11),
-// rounded lognormal prompt / output lengths (Table 1 profiles), a predicted
-// output length with multiplicative lognormal noise (sec. III-C, sec. V-G),
-// an SLO class, and an integer unit-rate exponential gap.  A warp-wide int64
-// inclusive scan turns gaps into cumulative work; Poisson arrivals divide by
-// the rate, MMPP arrivals walk the state intervals cooperatively.
+// A warp takes 32 consecutive requests of a replica (a chunk), one to a lane.
+// Per request: two Philox4x32-10 blocks (Salmon et al., SC'11), rounded
+// lognormal prompt / output lengths (Table 1 profiles), a predicted output
+// length with multiplicative lognormal noise (sec. III-C, sec. V-G), an SLO
+// class, and an integer unit-rate exponential gap.  An int64 inclusive scan
+// turns gaps into cumulative work (exact in any order); Poisson arrivals divide
+// by the rate, MMPP arrivals find their state interval among windows of 32.
+// With many replicas a warp walks one replica's chunks in order
+// (trace_kernel); with few, a cluster of blocks shares one replica
+// (trace_split_kernel).
 //
 // Bit-identity with the CPU reference construction rests on doing only IEEE
 // basic operations in a fixed order, in fp32 (the precision the integer
@@ -15,7 +18,11 @@
 // contraction into FMA; the file is also compiled with -fmad=false), and
 // log / exp / the normal quantile are written here from their published
 // methods rather than taken from CUDA's math library.
+#include <cooperative_groups.h>
+
 #include "ctr_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ctr {
 namespace {
@@ -103,23 +110,71 @@ __device__ float det_expf(float x)
     return mul(acc, __uint_as_float((uint32_t)(k + 127) << 23));
 }
 
-// Wichura (1988), algorithm AS241 PPND16 in fp32: rational approximations of
-// degree 7 in r = 0.180625 - q^2 (|q| <= 0.425, q = U - 1/2) or in
-// r = sqrt(-ln min(U, 1 - U)) shifted by 1.6 (r <= 5) or by 5.
-__device__ __forceinline__ float poly7(const float* c, float r)
+// Two fp32 operations in one instruction, each rounded to nearest on its own.
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 pack(float lo, float hi)
 {
-    float acc = c[7];
-#pragma unroll
-    for (int i = 6; i >= 0; --i) acc = add(mul(acc, r), c[i]);
-    return acc;
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack(F2 a, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+// The product as a fused multiply-add of -0, which rounds a b alone and keeps its sign.  The zeros come from
+// the kernel's parameters: where the assembler sees a plain product, or knows the zeros, it contracts it into
+// the add.rn.f32x2 that follows, and one request in 3,000 got another length.
+__device__ __forceinline__ F2 mul2(F2 a, F2 b, uint64_t minus_zeros)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(minus_zeros));
+    return r;
 }
 
-__device__ float det_ndtrif(uint32_t u)
+// Wichura (1988), algorithm AS241 PPND16 in fp32: rational approximations of
+// degree 7 in r = 0.180625 - q^2 (|q| <= 0.425, q = U - 1/2) or in
+// r = sqrt(-ln min(U, 1 - U)) shifted by 1.6 (r <= 5) or by 5.  The numerator
+// and the denominator go through Horner's scheme as one pair.
+__device__ __forceinline__ void ratio7(const float* num, const float* den, float r, uint64_t mz, float& n,
+                                       float& d)
+{
+    const F2 rr = pack(r, r);
+    F2 acc = pack(num[7], den[7]);
+#pragma unroll
+    for (int i = 6; i >= 0; --i) acc = add2(mul2(acc, rr, mz), pack(num[i], den[i]));
+    unpack(acc, n, d);
+}
+
+// 2^33 (U - 1/2) = 2 u + 1 - 2^32 (odd, below 2^32 in magnitude) as q = U - 1/2 rounded once
+__device__ __forceinline__ float centred(uint32_t u)
+{
+    const bool neg = (u & 0x80000000u) == 0;
+    const uint32_t mag = neg ? ~(u << 1) : (u << 1) + 1u;  // |2 u + 1 - 2^32|
+    const float m = __uint2float_rn(mag);
+    return mul(neg ? -m : m, 0x1p-33f);
+}
+
+constexpr float kCentre = 0x1.b33334p-2f;  // |q| up to here: the central approximation
+
+__device__ __forceinline__ float ndtri_centre(float q, uint64_t mz)
 {
     const float a[8] = {0x1.b18d92p+1f, 0x1.0a4888p+7f, 0x1.ece5d2p+10f, 0x1.ad1d8cp+13f,
                         0x1.66c3e8p+15f, 0x1.06c1c6p+16f, 0x1.052d26p+15f, 0x1.39a296p+11f};
     const float b[8] = {0x1p+0f, 0x1.5281b4p+5f, 0x1.5797fp+9f, 0x1.512322p+12f,
                         0x1.4b772ep+14f, 0x1.3317cap+15f, 0x1.c0e458p+14f, 0x1.46a7ecp+12f};
+    float n, d;
+    ratio7(a, b, sub(0x1.71eb86p-3f, mul(q, q)), mz, n, d);
+    return dvd(mul(q, n), d);
+}
+
+__device__ float ndtri_tail(uint32_t u, uint64_t mz)
+{
     const float c[8] = {0x1.6c666p+0f, 0x1.285774p+2f, 0x1.713f72p+2f, 0x1.d2ecb2p+1f,
                         0x1.453ccp+0f, 0x1.ef2abcp-3f, 0x1.744eb6p-6f, 0x1.9615acp-11f};
     const float d[8] = {0x1p+0f, 0x1.06cefcp+1f, 0x1.ad278ep+0f, 0x1.61293p-1f,
@@ -128,25 +183,47 @@ __device__ float det_ndtrif(uint32_t u)
                         0x1.b2b412p-6f, 0x1.45c19p-10f, 0x1.c6ec6cp-16f, 0x1.afb74ep-23f};
     const float f[8] = {0x1p+0f, 0x1.331d34p-1f, 0x1.186eb2p-3f, 0x1.e76f94p-7f,
                         0x1.9c8bcap-11f, 0x1.35c2c4p-16f, 0x1.31447p-23f, 0x1.269cp-49f};
-    const long long twice = 2ll * (long long)u + 1ll - 4294967296ll;  // 2^33 (U - 1/2), odd, |twice| < 2^32
-    const float mag = __uint2float_rn((uint32_t)(twice < 0 ? -twice : twice));
-    const float q = mul(twice < 0 ? -mag : mag, 0x1p-33f);
-    const float aq = q < 0.0f ? -q : q;
-    if (aq <= 0x1.b33334p-2f) {
-        const float r = sub(0x1.71eb86p-3f, mul(q, q));
-        return dvd(mul(q, poly7(a, r)), poly7(b, r));
+    const bool neg = (u & 0x80000000u) == 0;
+    const float r = __fsqrt_rn(-det_logf(u01(neg ? u : ~u)));
+    float n, m;
+    if (r <= 5.0f)
+        ratio7(c, d, sub(r, 0x1.99999ap+0f), mz, n, m);
+    else
+        ratio7(e, f, sub(r, 5.0f), mz, n, m);
+    const float v = dvd(n, m);
+    return neg ? -v : v;
+}
+
+// The normal quantiles of three words per lane, warp-collective.  15 % of the
+// words lie in the tails, so nearly every warp would run the tail path (a
+// logarithm, a square root, a rational) once for each of the three with a few
+// lanes active; instead the tail words of all lanes queue up in shared memory
+// (the warp's 96 entries at `q`) and are done together, 32 at a time: 14.4 of
+// them on average, so one pass.
+__device__ __forceinline__ void ndtri3(const uint32_t (&u)[3], float (&z)[3], uint64_t mz, uint32_t* q,
+                                       int lane)
+{
+    uint32_t m[3], pos[3];
+    uint32_t total = 0;
+    const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float c = centred(u[i]);
+        const bool tail = fabsf(c) > kCentre;
+        z[i] = ndtri_centre(c, mz);
+        const uint32_t b = __ballot_sync(0xffffffffu, tail);
+        pos[i] = total + __popc(b & below);
+        total += __popc(b);
+        m[i] = (b >> lane) & 1u;
+        if (m[i]) q[pos[i]] = u[i];
     }
-    const float tail = twice < 0 ? u01(u) : u01(~u);
-    float r = __fsqrt_rn(-det_logf(tail));
-    float v;
-    if (r <= 5.0f) {
-        r = sub(r, 0x1.99999ap+0f);
-        v = dvd(poly7(c, r), poly7(d, r));
-    } else {
-        r = sub(r, 5.0f);
-        v = dvd(poly7(e, r), poly7(f, r));
-    }
-    return twice < 0 ? -v : v;
+    __syncwarp();
+    for (uint32_t i = lane; i < total; i += 32) q[i] = __float_as_uint(ndtri_tail(q[i], mz));
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (m[i]) z[i] = __uint_as_float(q[pos[i]]);
+    __syncwarp();  // the queue is free for the next chunk
 }
 
 // clip(floor(v + 1/2), lo, hi) for v >= 0 (NaN / inf / huge -> hi); hi <= 2^20
@@ -171,90 +248,209 @@ __device__ __forceinline__ int64_t div_rate(int64_t num, int64_t d, uint64_t rec
     return (int64_t)q;
 }
 
-__device__ __forceinline__ int64_t dwell(const TraceParams& P, uint32_t k0, uint32_t k1, uint32_t sub_id,
-                                         int64_t j)
+// The replica's Philox key and sub-stream.
+struct Stream {
+    uint32_t k0, k1, sub_id;
+};
+__device__ __forceinline__ Stream stream_of(const TraceParams& P, int64_t r)
 {
-    const U32x4 x = philox((uint32_t)j, sub_id, 1u, 0u, k0, k1);
-    const float g = det_logf(u01(x.v[0]));
-    return trunc_pos(mul(-g, P.dwell_mean_f));
+    const int64_t g = P.replica_offset + r;
+    const uint64_t seed = P.seed + (uint64_t)(g % P.n_seeds);
+    return {(uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)(g / P.n_seeds)};
 }
 
-__global__ void __launch_bounds__(256) trace_kernel(const TraceParams P)
+// Request k's lengths and class, written to its place; returns its gap (0 past
+// the end).  Warp-collective.
+__device__ __forceinline__ int64_t request(const TraceParams& P, const Stream& S, int64_t row, int64_t k, uint32_t* q,
+                                           int lane)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t r = warp; r < P.n_replicas; r += n_warps) {
-        const int64_t g = P.replica_offset + r;
-        const uint64_t seed = P.seed + (uint64_t)(g % P.n_seeds);
-        const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-        const uint32_t sub_id = (uint32_t)(g / P.n_seeds);
-        const int64_t row = r * P.n_req;
+    const U32x4 x = philox((uint32_t)k, S.sub_id, 0u, 0u, S.k0, S.k1);
+    const U32x4 y = philox((uint32_t)k, S.sub_id, 0u, 1u, S.k0, S.k1);
+    const uint32_t u[3] = {x.v[0], x.v[2], x.v[3]};
+    float z[3];
+    ndtri3(u, z, P.minus_zeros, q, lane);
+    if (k >= P.n_req) return 0;
+    const bool is_short = (uint64_t)x.v[1] < P.mix_short_thr;
+    const float mu = is_short ? P.short_mu : P.long_mu;
+    const float sg = is_short ? P.short_sigma : P.long_sigma;
+    const int64_t p = round_clip(det_expf(add(P.prompt_mu, mul(P.prompt_sigma, z[0]))), P.prompt_min, P.prompt_max);
+    const int64_t o = round_clip(det_expf(add(mu, mul(sg, z[1]))), P.out_min, P.out_max);
+    const int64_t oh = round_clip(mul(__int2float_rn((int)o), det_expf(mul(P.noise_sigma, z[2]))), P.pred_min, P.pred_max);
+    int c = 0;
+    while (c < P.n_classes - 1 && (uint64_t)y.v[0] >= P.class_thr[c]) ++c;
+    P.out.prompt_len[row + k] = (int32_t)p;
+    P.out.true_out[row + k] = (int32_t)o;
+    P.out.pred_out[row + k] = (int32_t)oh;
+    P.out.slo_class[row + k] = (uint8_t)c;
+    return trunc_pos(mul(-det_logf(u01(y.v[1])), 0x1.dcd65p+29f));
+}
 
-        int64_t carry = 0;  // cumulative unit-rate work before this chunk (nano-events)
-        // MMPP interval j: [T, T + D) over which cumulative work runs from A to A_next
-        int64_t j = 0, T = 0, A = 0, D = 0, A_next = 0;
-        if (P.arrival_kind == 1) {
-            D = dwell(P, k0, k1, sub_id, 0);
-            A_next = A + P.rate[0] * D;
-        }
-        for (int64_t base = 0; base < P.n_req; base += 32) {
-            const int64_t k = base + lane;
-            const bool live = k < P.n_req;
-            int64_t p = 0, o = 0, oh = 0, c = 0, gap = 0;
-            if (live) {
-                const U32x4 x = philox((uint32_t)k, sub_id, 0u, 0u, k0, k1);
-                const U32x4 y = philox((uint32_t)k, sub_id, 0u, 1u, k0, k1);
-                const float zp = det_ndtrif(x.v[0]);
-                p = round_clip(det_expf(add(P.prompt_mu, mul(P.prompt_sigma, zp))), P.prompt_min, P.prompt_max);
-                const bool is_short = (uint64_t)x.v[1] < P.mix_short_thr;
-                const float mu = is_short ? P.short_mu : P.long_mu;
-                const float sg = is_short ? P.short_sigma : P.long_sigma;
-                const float zo = det_ndtrif(x.v[2]);
-                o = round_clip(det_expf(add(mu, mul(sg, zo))), P.out_min, P.out_max);
-                const float zn = det_ndtrif(x.v[3]);
-                oh = round_clip(mul(__int2float_rn((int)o), det_expf(mul(P.noise_sigma, zn))), P.pred_min, P.pred_max);
-                while (c < P.n_classes - 1 && (uint64_t)y.v[0] >= P.class_thr[c]) ++c;
-                gap = trunc_pos(mul(-det_logf(u01(y.v[1])), 0x1.dcd65p+29f));
-            }
-            // inclusive warp scan of the gaps (integers: exact in any order)
-            int64_t lam = gap;
+// inclusive warp scan of 64-bit integers (sums mod 2^64)
+__device__ __forceinline__ uint64_t scan32(uint64_t v, int lane)
+{
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int64_t v = __shfl_up_sync(0xffffffffu, lam, off);
-                if (lane >= off) lam += v;
-            }
-            lam += carry;
-            carry = __shfl_sync(0xffffffffu, lam, 31);
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint64_t w = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v += w;
+    }
+    return v;
+}
 
-            int64_t t = 0;
-            if (P.arrival_kind == 0) {
-                t = div_rate(lam, P.rate[0], P.rate_recip[0]);
-            } else {
-                // walk the intervals until every live lane found the last j with A_j <= lam
-                bool done = !live;
-                for (;;) {
-                    if (!done && lam < A_next) {
-                        t = T + div_rate(lam - A, P.rate[j & 1], P.rate_recip[j & 1]);
-                        done = true;
-                    }
-                    if (__all_sync(0xffffffffu, done)) break;
-                    T += D;
-                    A = A_next;
-                    j += 1;
-                    D = dwell(P, k0, k1, sub_id, j);
-                    A_next = A + P.rate[j & 1] * D;
-                }
+// Arrival times from cumulative work, for one warp whose lam never decreases.
+// MMPP: lane l holds interval j0 + l of a window of 32, its start time and the
+// work done before it; the window after starts at (t_next, a_next), and
+// (ti, ai, end, par) is the interval found last.  A dwell longer than any trace
+// counts as 2^58 of work, so no sum leaves 64 bits (lam stays below 2^23 gaps of
+// 2.3e10 < 2^58) and no later interval is looked at.
+struct Arrivals {
+    int64_t j0, t, t_next, ti;
+    uint64_t a, a_next, ai, end;
+    int par;
+
+    __device__ __forceinline__ void window(const TraceParams& P, const Stream& S, int lane)
+    {
+        const U32x4 x = philox((uint32_t)(j0 + lane), S.sub_id, 1u, 0u, S.k0, S.k1);
+        const uint64_t d = (uint64_t)trunc_pos(mul(-det_logf(u01(x.v[0])), P.dwell_mean_f));
+        uint64_t w = (uint64_t)P.rate[lane & 1] * d;  // below 2^62; j0 is even
+        if (w > (uint64_t(1) << 58)) w = uint64_t(1) << 58;
+        const uint64_t td = scan32(d, lane), aw = scan32(w, lane);
+        t = t_next + (int64_t)(td - d);
+        a = a_next + aw - w;
+        t_next += (int64_t)__shfl_sync(0xffffffffu, td, 31);
+        a_next += __shfl_sync(0xffffffffu, aw, 31);
+    }
+    __device__ __forceinline__ void start(const TraceParams& P, const Stream& S, int lane)
+    {
+        j0 = t = t_next = ti = 0;
+        a = a_next = ai = end = 0;  // an empty interval: the first call looks its own up
+        par = 0;
+        if (P.arrival_kind == 1) window(P, S, lane);
+    }
+    // each lane's arrival for its lam (unused where !live); warp-collective
+    __device__ __forceinline__ int64_t time(const TraceParams& P, const Stream& S, uint64_t lam, bool live, int lane)
+    {
+        if (P.arrival_kind == 0) return div_rate((int64_t)lam, P.rate[0], P.rate_recip[0]);
+        int64_t out = 0;
+        bool done = !live;
+        for (;;) {
+            if (!done && lam < end) {
+                out = ti + div_rate((int64_t)(lam - ai), P.rate[par], P.rate_recip[par]);
+                done = true;
             }
-            if (live) {
-                P.out.arrival_us[row + k] = t;
-                P.out.prompt_len[row + k] = (int32_t)p;
-                P.out.true_out[row + k] = (int32_t)o;
-                P.out.pred_out[row + k] = (int32_t)oh;
-                P.out.slo_class[row + k] = (uint8_t)c;
+            const uint32_t left = __ballot_sync(0xffffffffu, !done);
+            if (left == 0) return out;
+            // the interval of the first lane left: the last one that starts at or before its lam
+            const uint64_t lf = __shfl_sync(0xffffffffu, lam, __ffs(left) - 1);
+            while (lf >= a_next) {
+                j0 += 32;
+                window(P, S, lane);
             }
+            const int i = 31 - __clz(__ballot_sync(0xffffffffu, a <= lf));  // a never decreases over the lanes
+            const uint64_t up = __shfl_sync(0xffffffffu, a, (i + 1) & 31);
+            ai = __shfl_sync(0xffffffffu, a, i);
+            ti = __shfl_sync(0xffffffffu, t, i);
+            end = i < 31 ? up : a_next;
+            par = i & 1;
         }
     }
+};
+
+// One warp per replica.  Bound by instruction issue (Philox, the fp32 variates): 4,096 x 20,000 MMPP requests took
+// 2.95 ms with a tail path per variate, scalar polynomials and one dwell at a time, and take 2.43 ms; 21 B a
+// request are 0.7 TB/s of stores.  72 registers keep the 27 warps an SM of that size in one wave.
+constexpr int kWalkWarps = 4;
+__global__ void __launch_bounds__(kWalkWarps * 32, 7) trace_kernel(const TraceParams P)
+{
+    __shared__ uint32_t queue[kWalkWarps][96];
+    const int lane = threadIdx.x & 31;
+    uint32_t* q = queue[threadIdx.x >> 5];
+    const int64_t warp = (int64_t)blockIdx.x * kWalkWarps + (threadIdx.x >> 5);
+    const int64_t n_warps = (int64_t)gridDim.x * kWalkWarps;
+    for (int64_t r = warp; r < P.n_replicas; r += n_warps) {
+        const Stream S = stream_of(P, r);
+        const int64_t row = r * P.n_req;
+        uint64_t carry = 0;  // cumulative unit-rate work before this chunk (nano-events)
+        Arrivals arr;
+        arr.start(P, S, lane);
+        for (int64_t base = 0; base < P.n_req; base += 32) {
+            const int64_t k = base + lane;
+            const uint64_t lam = carry + scan32((uint64_t)request(P, S, row, k, q, lane), lane);
+            carry = __shfl_sync(0xffffffffu, lam, 31);
+            const int64_t t = arr.time(P, S, lam, k < P.n_req, lane);
+            if (k < P.n_req) P.out.arrival_us[row + k] = t;
+        }
+    }
+}
+
+// A cluster of blocks per replica, each block a contiguous range of its chunks.
+// Pass 1 writes every request's lengths, and its work within the chunk into its
+// arrival's place; a block scan of the chunks' totals and the totals of the
+// cluster's blocks before it (read from their shared memory) give each chunk
+// its start; pass 2 turns the work into arrival times, each thread reading back
+// what it wrote itself.  Bound by the chain of a chunk (Philox, quantile,
+// logarithm) and the two cluster barriers: 1 x 10,000 requests take 8.3 us
+// (Poisson) and 11.5 us (MMPP: every warp steps over the windows before its
+// chunks), 408 and 459 us with one warp.
+constexpr int kSplitWarps = 8;
+constexpr int kMaxCluster = 16;
+constexpr int64_t kMaxChunks = 16384;  // of one block: 2^23 requests over a full cluster
+__global__ void __launch_bounds__(kSplitWarps * 32) trace_split_kernel(const TraceParams P)
+{
+    __shared__ uint32_t queue[kSplitWarps][96];
+    __shared__ uint64_t warp_sum[kSplitWarps];
+    __shared__ uint64_t block_sum;
+    extern __shared__ uint64_t chunk[];  // work of each chunk, then the block's work before it
+    cg::cluster_group cluster = cg::this_cluster();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t blocks = (int64_t)cluster.num_blocks(), rank = (int64_t)cluster.block_rank();
+    const int64_t r = blockIdx.x / blocks;
+    const int64_t n_chunks = (P.n_req + 31) / 32;
+    const int64_t c0 = n_chunks * rank / blocks, c1 = n_chunks * (rank + 1) / blocks;
+    const Stream S = stream_of(P, r);
+    const int64_t row = r * P.n_req;
+
+    for (int64_t c = c0 + wid; c < c1; c += kSplitWarps) {
+        const int64_t k = c * 32 + lane;
+        const uint64_t lam = scan32((uint64_t)request(P, S, row, k, queue[wid], lane), lane);
+        if (k < P.n_req) P.out.arrival_us[row + k] = (int64_t)lam;
+        if (lane == 31) chunk[c - c0] = lam;
+    }
+    __syncthreads();
+    // exclusive scan of the chunks' work: a run of chunks per thread, then over the block's threads
+    const int64_t m = c1 - c0, per = (m + blockDim.x - 1) / blockDim.x;
+    const int64_t b = threadIdx.x * per, e = b + per < m ? b + per : m;
+    uint64_t sum = 0;
+    for (int64_t i = b; i < e; ++i) sum += chunk[i];
+    const uint64_t incl = scan32(sum, lane);
+    if (lane == 31) warp_sum[wid] = incl;
+    __syncthreads();
+    uint64_t before = incl - sum;
+    for (int w = 0; w < wid; ++w) before += warp_sum[w];
+    for (int64_t i = b; i < e; ++i) {
+        const uint64_t v = chunk[i];
+        chunk[i] = before;
+        before += v;
+    }
+    if (threadIdx.x == 0) {
+        uint64_t all = 0;
+        for (int w = 0; w < kSplitWarps; ++w) all += warp_sum[w];
+        block_sum = all;
+    }
+    cluster.sync();  // every block's sum is there (and this block's chunks)
+    uint64_t offset = lane < rank ? *cluster.map_shared_rank(&block_sum, lane) : 0;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) offset += __shfl_xor_sync(0xffffffffu, offset, off);
+
+    Arrivals arr;
+    arr.start(P, S, lane);
+    for (int64_t c = c0 + wid; c < c1; c += kSplitWarps) {
+        const int64_t k = c * 32 + lane;
+        const bool live = k < P.n_req;
+        const uint64_t lam = live ? offset + chunk[c - c0] + (uint64_t)P.out.arrival_us[row + k] : 0;
+        const int64_t t = arr.time(P, S, lam, live, lane);
+        if (live) P.out.arrival_us[row + k] = t;
+    }
+    cluster.sync();  // no block leaves while another may still read its sum
 }
 
 }  // namespace
@@ -267,13 +463,46 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream)
     if (err != cudaSuccess) return err;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
+    // Split replicas while a warp each leaves the GPU idle or waiting on one warp's chain (1.5 us a chunk
+    // against 2 us for the 8 of a block): 1 x 10,000 requests 459 -> 11.5 us, 64 x 10,000 469 -> 34,
+    // 1,024 x 5,000 271 -> 167, 3,000 x 5,000 457 -> 441.  Short traces leave a block's warps idle and stay
+    // with one warp a replica unless there are very few of them: 1,000 x 64 takes 6.3 us there, 13 us split.
+    const int64_t n_chunks = (p.n_req + 31) / 32;
+    if (p.n_replicas <= (int64_t)sms * 20 && n_chunks >= (p.n_replicas <= sms ? 4 : 16)) {
+        // blocks per replica: up to 8 blocks an SM in all, at least 2 chunks a block; clusters of 16 only for a few replicas, as they are slow to place (16 x 10,000: 19.6 us with 8
+        // blocks, 16.8 with 16; 64 x 10,000: 34 us with 4 or 8, 40 with 16)
+        int cluster = 1;
+        while (cluster < kMaxCluster &&
+               ((p.n_replicas * cluster * 2 <= (cluster < 8 ? sms * 8 : sms * 2) && n_chunks >= cluster * 4) ||
+                n_chunks > (int64_t)cluster * kMaxChunks))
+            cluster *= 2;
+        const size_t smem = (size_t)((n_chunks + cluster - 1) / cluster) * 8;
+        err = cudaFuncSetAttribute(trace_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)(kMaxChunks * sizeof(uint64_t)));
+        if (err != cudaSuccess) return err;
+        err = cudaFuncSetAttribute(trace_split_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (err != cudaSuccess) return err;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(p.n_replicas * cluster));
+        cfg.blockDim = dim3(kSplitWarps * 32);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cluster;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        err = cudaLaunchKernelEx(&cfg, trace_split_kernel, p);
+        if (err != cudaSuccess) return err;
+        return cudaGetLastError();
+    }
     // small blocks spread one warp per replica evenly over the SMs (the kernel is
     // issue-bound, so the SM holding the most warps sets its time)
-    const int warps_per_block = 4;
-    int64_t blocks = (p.n_replicas + warps_per_block - 1) / warps_per_block;
+    int64_t blocks = (p.n_replicas + kWalkWarps - 1) / kWalkWarps;
     const int64_t cap = (int64_t)sms * 16;
     if (blocks > cap) blocks = cap;
-    trace_kernel<<<(unsigned)blocks, warps_per_block * 32, 0, stream>>>(p);
+    trace_kernel<<<(unsigned)blocks, kWalkWarps * 32, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

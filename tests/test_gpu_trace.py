@@ -34,6 +34,19 @@ def test_trace_bit_identical(orc, name, tc, R, N, off):
     _compare(orc, tc, tr, R, N, off)
 
 
+@pytest.mark.parametrize("R,N", [(1, 32), (1, 63), (2, 64), (1, 65), (3, 1025), (1, 10_000), (17, 10_001), (130, 257),
+                                 (1, 700_001), (700, 40), (1215, 70), (1217, 70)])
+@pytest.mark.parametrize("tc", [W.replica_sweep().trace, W.TraceCfg(seed=11, n_classes=1, class_thr=()),
+                                W.TraceCfg(seed=3, n_seeds=2, arrival_kind=1, rate_mreq=(9_000_000, 40),
+                                           dwell_mean_us=1_000)], ids=["mmpp", "poisson", "short_dwell"])
+def test_split_replicas_bit_identical(orc, tc, R, N):
+    """Few replicas are each split over a cluster of blocks, many take a warp each: sizes around the chunk of 32,
+    block and cluster ranges of unequal length, both sides of the line between the two, many intervals to a chunk."""
+    ctr = need_gpu()
+    tr = gen(ctr, tc, R, N, 5)
+    _compare(orc, tc, tr, R, N, 5, rows=sorted({0, 1, R // 2, R - 1} & set(range(R))))
+
+
 def test_empty_sizes(orc):
     ctr = need_gpu()
     gen(ctr, W.TraceCfg(), 0, 100)
