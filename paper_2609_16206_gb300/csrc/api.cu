@@ -251,15 +251,12 @@ int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t 
     p.dec_seq = cfg->dec_us_per_seq;
     p.kv_div = cfg->dec_kv_tokens_per_us;
     p.pre_batch = cfg->prefill_batch_tokens;
-    // ceil(2^64 / kv_div) = floor((2^64 - 1) / kv_div) + 1 for kv_div >= 2 (not a power of two
-    // or otherwise: the +1 rounds up whenever kv_div does not divide 2^64 exactly)
-    if (p.kv_div >= 2) {
-        const uint64_t d = (uint64_t)p.kv_div;
-        uint64_t m = ~0ull / d;
-        if ((d & (d - 1)) != 0) m += 1;                 // d does not divide 2^64
-        else m = (uint64_t)1 << (64 - __builtin_ctzll(d)); // exact power of two
-        p.kv_div_magic = m;
-    }
+    while ((1LL << p.kv_shift) < p.kv_div) ++p.kv_shift;
+    p.kv_mul = (uint32_t)(((1ull << (31 + p.kv_shift)) + (uint64_t)p.kv_div - 1) / (uint64_t)p.kv_div);
+    // the longest step: a full batch, every token of the capacity resident
+    const int64_t longest = p.dec_base + p.dec_seq * (int64_t)cfg->cap_active + p.kv_cap / p.kv_div;
+    const int64_t run_max = ((1LL << 31) - 1) / longest - 1;
+    p.run_max = run_max < 0 ? 0 : run_max > (1 << 20) ? 1 << 20 : (int32_t)run_max;
     p.n_classes = cfg->n_classes;
     p.heur_thresh = cfg->heuristic_threshold_tokens;
     p.max_steps = cfg->max_steps_per_instance;

@@ -148,7 +148,9 @@ struct SimParams {
     int64_t dec_base, dec_seq;
     int64_t kv_div;
     int64_t pre_batch;          // prefill batch token budget, 0 = serial prefill
-    uint64_t kv_div_magic;      // ceil(2^64 / kv_div) (kv_div >= 2)
+    uint32_t kv_mul;            // ceil(2^(31 + kv_shift) / kv_div)
+    int32_t kv_shift;           // ceil(log2(kv_div))
+    int32_t run_max;            // (run_max + 1) times the longest possible step is below 2^31 us; 0 if one step is not
     int32_t n_classes, heur_thresh;
     int64_t max_steps;
     int32_t cap_pend, cap_wait, cap_act, cap_ring;

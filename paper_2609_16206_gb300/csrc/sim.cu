@@ -88,15 +88,11 @@ __device__ __forceinline__ int32_t div_estimate(int32_t x, int32_t d)
     return __float2int_rz(__fdividef(__int2float_rn(x), __int2float_rn(d)));
 }
 
-// floor(x / kv_div) for 0 <= x < 2^32 with magic = ceil(2^64 / kv_div), exact: the
-// 96-bit product x * magic shifted right by 64, from two 32 x 32-bit products
-__device__ __forceinline__ int64_t kv_term(int64_t x, const SimParams& P)
+// floor(x / kv_div) for 0 <= x < 2^31, exact: kv_mul = ceil(2^(31 + s) / kv_div) with
+// s = kv_shift the least with 2^s >= kv_div, so that x (kv_mul kv_div - 2^(31 + s)) < 2^31 2^s
+__device__ __forceinline__ int32_t kv_term(int32_t x, const SimParams& P)
 {
-    if (P.kv_div == 1) return x;
-    const uint32_t xl = (uint32_t)x;
-    const uint64_t lo = (uint64_t)xl * (uint32_t)P.kv_div_magic;
-    const uint64_t hi = (uint64_t)xl * (uint32_t)(P.kv_div_magic >> 32);
-    return (int64_t)((hi + (lo >> 32)) >> 32);  // no overflow: hi <= 2^64 - 2^33 + 1
+    return (int32_t)(__umulhi((uint32_t)x << 1, P.kv_mul) >> P.kv_shift);
 }
 
 // Entries per lane of a heap region holding up to cap keys.  The heaps are
@@ -338,8 +334,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         s.step_idx += ends;
         s.kv_res += tokens;
         if (!sum_is_o_hat) s.sum -= tokens;
-        if (s.step_idx > (int32_t)P.max_steps) return CTR_ETIMEOUT;
-        while (s.n_act > 0 && (int32_t)(s.act_top >> kKeyBits) == s.step_idx) {
+        while ((int32_t)(s.act_top >> kKeyBits) == s.step_idx) {  // never with an empty heap: its top is all ones
             const int64_t k = (int64_t)(s.act_top & kKeyMask);
             const int32_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
             const int32_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
@@ -385,13 +380,13 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         admitted += 1;
     }
     // (3) the next step and the next event
+    if (s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
     const int64_t tp = s.pend_n > 0 ? (int64_t)(s.pend_top >> kKeyBits) : kNever;
     if (s.n_act == 0) {
         s.step_end = tp;
         s.run = 0;
         return CTR_OK;
     }
-    if (s.step_idx >= (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
     const int32_t n = s.n_act;
     const int64_t fixed = P.dec_base + (int64_t)(int32_t)P.dec_seq * n;
     s.step_end = tev + fixed + kv_term(s.kv_res, P);
@@ -402,17 +397,15 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     }
     // after j of the run's ends the KV term is that of kv_res + j n, and it stays q1 while j n <= room1
     // (q1 + 1 <= 2^31 and kv_div <= 2^31; the sum is below 2^32)
-    const int64_t q1 = kv_term(s.kv_res + n, P);
+    const int32_t q1 = kv_term(s.kv_res + n, P);
     const uint32_t room1 = (uint32_t)(q1 + 1) * (uint32_t)P.kv_div - 1u - (uint32_t)s.kv_res;
     int32_t m = (int32_t)(s.act_top >> kKeyBits) - s.step_idx - 1;  // plain ends before the next completion, <= 2^20
     if ((uint64_t)(uint32_t)m * (uint32_t)n > room1) {  // the term changes first: at most room1 / n (one less is fine)
         m = __float2int_rz(__fdividef(__uint2float_rn(room1), __int2float_rn(n)));
         m -= (uint64_t)(uint32_t)m * (uint32_t)n > room1;
     }
-    const int64_t step = fixed + q1;
-    if (((int64_t)m * step) >> 31) m = step >> 31 ? 0 : (int32_t)(0x7fffffffu / (uint32_t)step);
-    s.step = (int32_t)step;  // a step of 2^31 us or more has m = 0
-    s.run = m;
+    s.step = (int32_t)fixed + q1;  // run_max = 0 where a step could reach 2^31 us
+    s.run = m < P.run_max ? m : P.run_max;
     if (s.w_n == 0 && s.pend_n > 0) cut_run(s, tp);
     return CTR_OK;
 }
