@@ -282,15 +282,18 @@ int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t 
     for (int i = 0; i < n_const_sets; ++i) {
         const ctr_cost_consts& k = consts[i];
         ConstsDev& d = p.sets[i];
-        d.tau_pre0 = k.tau_pre0_us;
-        d.tau_pre = k.tau_pre_us;
-        d.tau_dec = k.tau_dec_us;
-        d.w_q = k.w_q_us;
-        d.w_b = k.w_b_q8;
-        d.w_s = k.w_s_q8;
-        d.rho = k.rho_q8;
-        for (int c = 0; c < 4; ++c) d.sigma[c] = k.sigma_q8[c];
-        d.ablate = k.ablate;
+        d.tau_pre0 = (uint32_t)k.tau_pre0_us;
+        d.tau_pre = (uint32_t)k.tau_pre_us;
+        d.tau_dec = (uint32_t)k.tau_dec_us;
+        d.w_q16 = (uint64_t)k.w_q_us << 16;
+        d.w_b = (uint32_t)k.w_b_q8;
+        d.w_s = (uint32_t)k.w_s_q8;
+        d.rho = (uint32_t)k.rho_q8;
+        for (int c = 0; c < 4; ++c) d.sigma[c] = (k.ablate & CTR_ABLATE_SLO) ? 256u : (uint32_t)k.sigma_q8[c];
+        const bool no_length = (k.ablate & CTR_ABLATE_PREDICTED_LENGTH) != 0;
+        d.oh_mask = no_length ? 0u : ~0u;
+        d.press_mask = (k.ablate & CTR_ABLATE_PRESSURE) ? 0u : ~0u;
+        d.ledger_tau = no_length ? 0u : d.tau_dec;
         d.proxy = k.backlog_signal;
         d.poll_us = k.occupancy_poll_us;
         d.poll_recip = k.occupancy_poll_us > 0 ? ~0ull / (uint64_t)k.occupancy_poll_us : 0;

@@ -129,12 +129,15 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream);
 
 // ---------------------------------------------------------------- simulator
 struct ConstsDev {
-    int64_t tau_pre0, tau_pre, tau_dec, w_q;
-    int32_t w_b, w_s, rho, sigma[4];
-    uint32_t ablate;
-    uint32_t proxy;       // backlog from the priced in-flight ledger
-    int64_t poll_us;      // > 0: occupancy polled on this period
-    uint64_t poll_recip;  // floor((2^64 - 1) / poll_us)
+    uint64_t w_q16;                  // w_q << 16
+    uint32_t tau_pre0, tau_pre, tau_dec;
+    uint32_t w_b, w_s, rho;
+    uint32_t sigma[4];               // 256 for every class when the SLO class is ablated
+    uint32_t oh_mask, press_mask;    // 0 when the predicted length / the pressure is ablated, else all ones
+    uint32_t ledger_tau;             // tau_dec, 0 when the predicted length is ablated
+    uint32_t proxy;                  // backlog from the priced in-flight ledger
+    int64_t poll_us;                 // > 0: occupancy polled on this period
+    uint64_t poll_recip;             // floor((2^64 - 1) / poll_us)
 };
 
 // The host validates pre_tok, xfer_tok <= 2^20, dec_seq <= 2^16, kv_div <= 2^31

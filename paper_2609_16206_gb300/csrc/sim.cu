@@ -46,7 +46,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarpsPerBlock = 4;
 constexpr int64_t kNever = INT64_MAX;
 constexpr int64_t kBacklogClamp = int64_t(1) << 40;
-constexpr int64_t kPressureClamp = int64_t(1) << 18;
+constexpr uint64_t kPressureClamp = uint64_t(1) << 18;
 constexpr int kRecipN = 1024;  // batch sizes with a tabulated reciprocal
 constexpr int kRingPBits = 21;  // prefill ring entry: end << 21 | p (p <= 2^20)
 constexpr int64_t kRingPMask = (int64_t(1) << kRingPBits) - 1;
@@ -81,11 +81,12 @@ __device__ __forceinline__ uint64_t div_recip(uint64_t num, uint64_t d, uint64_t
 }
 
 // An estimate of x / d for 0 <= x < 2^31 and 1 <= d < 2^31 whose quotient is
-// below 2^20: both operands rounded to fp32 and a divide good to a few 2^-24,
-// so it is off by less than one unit either way.
-__device__ __forceinline__ int32_t div_estimate(int32_t x, int32_t d)
+// below 2^20, inv being recip_estimate(d): x and d rounded to fp32, a reciprocal
+// good to a few 2^-24 and a product, so it is off by less than one unit either way.
+__device__ __forceinline__ float recip_estimate(int32_t d) { return __fdividef(1.0f, __int2float_rn(d)); }
+__device__ __forceinline__ int32_t div_estimate(int32_t x, float inv)
 {
-    return __float2int_rz(__fdividef(__int2float_rn(x), __int2float_rn(d)));
+    return __float2int_rz(__int2float_rn(x) * inv);
 }
 
 // floor(x / kv_div) for 0 <= x < 2^31, exact: kv_mul = ceil(2^(31 + s) / kv_div) with
@@ -233,6 +234,51 @@ __device__ __forceinline__ int warp_argmin(uint64_t v)
     return __ffs(ball) - 1;
 }
 
+// The row's slice of the trace and of the outputs: four pointers where
+// registers allow (kPtr: 128 of them), else two offsets added on each access
+// (pointers in every instantiation: single replica 4.72 -> 4.65 ms, but the
+// replica sweep at 72 registers 137.0 -> 137.8).
+template <bool kPtr>
+struct RowView {
+    const SimParams& P;
+    const int32_t *p_ = nullptr, *o_ = nullptr;
+    int64_t *tf_ = nullptr, *td_ = nullptr;
+    int64_t tb, ob;
+    __device__ __forceinline__ RowView(const SimParams& P, int64_t tb, int64_t ob) : P(P), tb(tb), ob(ob)
+    {
+        if (kPtr) {
+            p_ = P.trace.prompt_len + tb;
+            o_ = P.trace.true_out + tb;
+            tf_ = P.t_first + ob;
+            td_ = P.t_done + ob;
+        }
+    }
+    __device__ __forceinline__ int32_t p(uint32_t k, bool& bad) const
+    {
+        return kPtr ? ck_ldg(p_, k, P.n_req, bad) : ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
+    }
+    __device__ __forceinline__ int32_t o(uint32_t k, bool& bad) const
+    {
+        return kPtr ? ck_ldg(o_, k, P.n_req, bad) : ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
+    }
+    __device__ __forceinline__ int32_t o_hat(uint32_t k, bool& bad) const
+    {
+        return ck_ldg(P.trace.pred_out, tb + k, P.trace_len, bad);
+    }
+    __device__ __forceinline__ int64_t first(uint32_t k, bool& bad) const
+    {
+        return kPtr ? ck_ld(tf_, k, P.n_req, bad) : ck_ld(P.t_first, ob + k, P.out_len, bad);
+    }
+    __device__ __forceinline__ void set_first(uint32_t k, int64_t v, bool& bad) const
+    {
+        kPtr ? ck_st(tf_, k, P.n_req, v, bad) : ck_st(P.t_first, ob + k, P.out_len, v, bad);
+    }
+    __device__ __forceinline__ void set_done(uint32_t k, int64_t v, bool& bad) const
+    {
+        kPtr ? ck_st(td_, k, P.n_req, v, bad) : ck_st(P.t_done, ob + k, P.out_len, v, bad);
+    }
+};
+
 // A decode lane's state.  Its next event is the end of a step at which
 // something can change (a completion, an admission, the floor(KV / kv_div) term
 // of the step time), and the steps before it are a run of equal ones, left as
@@ -249,6 +295,7 @@ __device__ __forceinline__ int warp_argmin(uint64_t v)
 struct Decode {
     int64_t step_end, sum;
     int32_t run, step;
+    float inv_step;          // about 1 / step (see div_estimate)
     int32_t step_idx;        // steps ended; the step budget keeps it and every completion step below 2^31
     int32_t kv_res, kv_rsv;  // resident <= reserved <= C < 2^31 tokens
     uint64_t pend_top, act_top;
@@ -263,7 +310,7 @@ __device__ __forceinline__ int32_t ends_by(const Decode& s, int64_t t)
 {
     if (s.n_act == 0 || t < s.step_end) return 0;
     const int32_t dt = (int32_t)(t - s.step_end);
-    int32_t q = div_estimate(dt, s.step);
+    int32_t q = div_estimate(dt, s.inv_step);
     const int32_t r = dt - q * s.step;
     q += (r >= s.step) - (r < 0);
     return q + 1;
@@ -278,7 +325,7 @@ __device__ __forceinline__ void cut_run(Decode& s, int64_t tp)
         s.run = 0;
     } else if (tp < next_event(s)) {
         const int32_t rel = (int32_t)(tp - s.step_end);
-        int32_t q = div_estimate(rel, s.step);
+        int32_t q = div_estimate(rel, s.inv_step);
         q += rel > q * s.step;
         s.run = q;
     }
@@ -323,9 +370,9 @@ __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, c
 // FIFO's head waits for room, at the next completion); it has room for
 // cap_pend + cap_wait + 1 entries, so a full heap means the waiting FIFO has
 // overflowed.
-template <int kArity>
+template <int kArity, bool kPtr>
 __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimParams& P, uint64_t* pend, uint64_t* act,
-                                            uint32_t* wait, int64_t tb, int64_t ob, bool sum_is_o_hat, bool& bad)
+                                            uint32_t* wait, const RowView<kPtr>& V, bool sum_is_o_hat, bool& bad)
 {
     if (tev >= kTimeLimit) return CTR_EOVERFLOW;
     if (s.n_act > 0) {  // (1) run + 1 steps end: as many tokens for every active request
@@ -335,11 +382,10 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         s.kv_res += tokens;
         if (!sum_is_o_hat) s.sum -= tokens;
         while ((int32_t)(s.act_top >> kKeyBits) == s.step_idx) {  // never with an empty heap: its top is all ones
-            const int64_t k = (int64_t)(s.act_top & kKeyMask);
-            const int32_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
-            const int32_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
-            if (sum_is_o_hat) s.sum -= ck_ldg(P.trace.pred_out, tb + k, P.trace_len, bad);
-            ck_st(P.t_done, ob + k, P.out_len, tev, bad);
+            const uint32_t k = (uint32_t)(s.act_top & kKeyMask);
+            const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
+            if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
+            V.set_done(k, tev, bad);
             hpop<kArity == 2>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
             s.q -= 1;
             s.kv_res -= pk + ok;
@@ -356,8 +402,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         const bool fifo = s.w_n > 0;
         if (!fifo && !(s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= tev)) break;
         const uint32_t k = fifo ? ck_ld(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
-        const int32_t pk = ck_ldg(P.trace.prompt_len, tb + k, P.trace_len, bad);
-        const int32_t ok = ck_ldg(P.trace.true_out, tb + k, P.trace_len, bad);
+        const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
         if ((uint32_t)s.kv_rsv + (uint32_t)(pk + ok) > (uint32_t)P.kv_cap) {  // < 2^31 + 2^21
             const int rc = flush_ready<kArity>(s, tev, room, P, pend, wait, bad);
             if (rc != CTR_OK) return rc;
@@ -375,7 +420,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         s.kv_res += pk;
         hpush<kArity == 2>(act, s.n_act, s.act_top, ((uint64_t)(uint32_t)(s.step_idx + ok) << kKeyBits) | k,
                            heap_stride(P.cap_act), bad);
-        if (admitted > 0) ck_st(P.t_first, ob + k, P.out_len, (int64_t)last, bad);
+        if (admitted > 0) V.set_first(k, (int64_t)last, bad);
         last = k;
         admitted += 1;
     }
@@ -391,8 +436,8 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     const int64_t fixed = P.dec_base + (int64_t)(int32_t)P.dec_seq * n;
     s.step_end = tev + fixed + kv_term(s.kv_res, P);
     for (; admitted > 0; --admitted) {  // first token at the end of this step
-        const int64_t prev = admitted > 1 ? ck_ld(P.t_first, ob + last, P.out_len, bad) : 0;
-        ck_st(P.t_first, ob + last, P.out_len, s.step_end, bad);
+        const int64_t prev = admitted > 1 ? V.first(last, bad) : 0;
+        V.set_first(last, s.step_end, bad);
         last = (uint32_t)prev;
     }
     // after j of the run's ends the KV term is that of kv_res + j n, and it stays q1 while j n <= room1
@@ -405,6 +450,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         m -= (uint64_t)(uint32_t)m * (uint32_t)n > room1;
     }
     s.step = (int32_t)fixed + q1;  // run_max = 0 where a step could reach 2^31 us
+    s.inv_step = recip_estimate(s.step);
     s.run = m < P.run_max ? m : P.run_max;
     if (s.w_n == 0 && s.pend_n > 0) cut_run(s, tp);
     return CTR_OK;
@@ -413,9 +459,9 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
 // Advance one decode instance through every event at times <= T.  kSnap: when
 // tsnap >= 0, also record in kv_snap the resident KV as it is after every event
 // at times <= tsnap (an occupancy poll; tsnap <= T).
-template <bool kSnap, int kArity>
+template <bool kSnap, int kArity, bool kPtr>
 __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimParams& P, uint64_t* pend, uint64_t* act,
-                                              uint32_t* wait, int64_t tb, int64_t ob, int64_t tsnap, int64_t& kv_snap,
+                                              uint32_t* wait, const RowView<kPtr>& V, int64_t tsnap, int64_t& kv_snap,
                                               bool sum_is_o_hat, bool& bad)
 {
     for (;;) {
@@ -427,7 +473,7 @@ __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimPar
             }
         }
         if (tev > T) return CTR_OK;
-        const int rc = decode_event<kArity>(s, tev, P, pend, act, wait, tb, ob, sum_is_o_hat, bad);
+        const int rc = decode_event<kArity>(s, tev, P, pend, act, wait, V, sum_is_o_hat, bad);
         if (rc != CTR_OK) return rc;
     }
 }
@@ -539,6 +585,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         const bool sum_is_o_hat = pol == CTR_POLICY_LENGTH_HEURISTIC || (kSig && learned_row && cc.proxy);
         const int64_t tb = rep * n;
         const int64_t ob = row * n;
+        const RowView<kBlocksPerSM <= 4> V(P, tb, ob);
 
         // per-request bounds, one row at a time with the whole warp
         bool oob = false;  // bounds-checked builds: an index of this lane fell outside its buffer
@@ -554,7 +601,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         bool live = has_row && valid;
 
         Decode s;
-        s.step_end = is_dec ? kNever : 0; s.run = 0; s.step = 1;
+        s.step_end = is_dec ? kNever : 0; s.run = 0; s.step = 1; s.inv_step = 1.0f;
         s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
         s.pend_top = kEmpty; s.act_top = kEmpty;
         s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
@@ -676,7 +723,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                             }
                         }
                         if (err == CTR_OK)
-                            err = decode_advance<kSig, kArity>(s, T, P, pend, act, wait, tb, ob, tsnap, kv_seen,
+                            err = decode_advance<kSig, kArity>(s, T, P, pend, act, wait, V, tsnap, kv_seen,
                                                                sum_is_o_hat, oob);
                     } else if (is_pre && !batched) {
                         const int64_t thr = ((T + 1) << kRingPBits) - 1;  // entries whose prefill ended by T
@@ -703,70 +750,64 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                 // 2. price the candidates and take the argmin of each pool
                 uint64_t cost = kEmpty;
                 if (live && pol != CTR_POLICY_ROUND_ROBIN) {
-                    const bool learned = pol == CTR_POLICY_LEARNED || pol == CTR_POLICY_LEARNED_P2;
-                    // feature ablation (sec. V-F): a removed feature takes its neutral value
-                    const int64_t oh_f = (cc.ablate & CTR_ABLATE_PREDICTED_LENGTH) ? 0 : ohk;
-                    const int64_t sig = (cc.ablate & CTR_ABLATE_SLO) ? 256 : cc.sigma[ck];
-                    if (is_pre) {
-                        if (learned) {
-                            int64_t b = busy > T ? busy - T : 0;
-                            if (batched) {  // the running batch's rest, then the queue's batches
-                                b = (run_n > 0 && busy > T ? busy - T : 0) + P.pre_base * (int64_t)q_batches +
-                                    P.pre_tok * (ring_sum_p - run_p);
-                                if (b > kBacklogClamp) b = kBacklogClamp;
-                            }
+                    if (learned_row) {
+                        // backlog and own work of the lane's instance, then the cost both kinds share
+                        // (feature ablation, sec. V-F, is in the constants: see ConstsDev)
+                        uint64_t b = 0, work = 0;
+                        if (is_pre) {
                             if (kSig && cc.proxy) {  // the ledger: tau_pre0 + tau_pre p per prefill not yet ended
-                                b = cc.tau_pre0 * (int64_t)ring_n + cc.tau_pre * ring_sum_p;
-                                if (b > kBacklogClamp) b = kBacklogClamp;
-                            }
-                            const int64_t load = cc.w_b * b + cc.w_s * (cc.tau_pre0 + pk * cc.tau_pre);
-                            cost = (uint64_t)(load * sig + cc.w_q * (int64_t)ring_n * 65536);
-                        } else {
-                            cost = (uint64_t)ring_n;
-                        }
-                    } else if (is_dec) {
-                        if (learned) {
-                            const int64_t na = s.n_act;
-                            const int32_t tokens = ends_by(s, T) * s.n_act;  // of the run's steps that have ended
-                            const int32_t kv_live = s.kv_res + tokens;
-                            const uint64_t R = (uint64_t)(s.sum - tokens);  // unread where sum is o_hat
-                            const int64_t step = P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act + kv_term(kv_live, P);
-                            const uint64_t lo = R * (uint64_t)step;
-                            const uint64_t nd = (uint64_t)(na > 1 ? na : 1);
-                            int64_t b;
-                            if (((R | ((uint64_t)step << 10)) >> 32) == 0 && nd <= (uint64_t)kRecipN) {  // lo < 2^54
-                                b = (int64_t)(nd > 1 ? __umul64hi(lo, __ldg(&kRecipTable.v[nd])) : lo);
-                            } else if (__umul64hi(R, (uint64_t)step) != 0 || lo >= (1ull << 62)) {
-                                b = kBacklogClamp;
+                                b = (uint64_t)cc.tau_pre0 * (uint32_t)ring_n + (uint64_t)cc.tau_pre * (uint64_t)ring_sum_p;
+                            } else if (batched) {  // the running batch's rest, then the queue's batches
+                                b = (uint64_t)((run_n > 0 && busy > T ? busy - T : 0) + P.pre_base * (int64_t)q_batches +
+                                               P.pre_tok * (ring_sum_p - run_p));
                             } else {
-                                b = (int64_t)(lo / nd);
+                                b = (uint64_t)(busy > T ? busy - T : 0);
                             }
-                            if (b > kBacklogClamp) b = kBacklogClamp;
-                            if (kSig && cc.proxy) {  // the ledger: tau_dec o_hat per request routed here and not done
-                                b = (cc.ablate & CTR_ABLATE_PREDICTED_LENGTH) ? 0 : cc.tau_dec * s.sum;
-                                if (b > kBacklogClamp) b = kBacklogClamp;
+                            work = (uint64_t)cc.tau_pre * (uint32_t)pk + cc.tau_pre0;
+                        } else if (is_dec) {
+                            const uint32_t oh_f = (uint32_t)ohk & cc.oh_mask;
+                            int32_t kv = (int32_t)kv_seen;
+                            const bool polled = kSig && cc.poll_us > 0;
+                            if (!(kSig && cc.proxy && polled)) {
+                                const int32_t tokens = ends_by(s, T) * s.n_act;  // of the run's steps that have ended
+                                const int32_t kv_live = s.kv_res + tokens;
+                                if (!polled) kv = kv_live;
+                                if (!(kSig && cc.proxy)) {
+                                    const uint64_t R = (uint64_t)(s.sum - tokens);
+                                    const uint64_t step = (uint64_t)(P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act +
+                                                                     kv_term(kv_live, P));
+                                    const uint32_t nd = (uint32_t)(s.n_act > 1 ? s.n_act : 1);
+                                    if (((R | (step << 10)) >> 32) == 0 && nd <= (uint32_t)kRecipN) {
+                                        const uint64_t lo = (uint64_t)(uint32_t)R * (uint32_t)step;  // < 2^54
+                                        b = nd > 1 ? __umul64hi(lo, __ldg(&kRecipTable.v[nd])) : lo;
+                                    } else {
+                                        const uint64_t lo = R * step;
+                                        b = __umul64hi(R, step) != 0 || lo >= (1ull << 62) ? (uint64_t)kBacklogClamp : lo / nd;
+                                    }
+                                }
                             }
-                            const int64_t kv = kSig && cc.poll_us > 0 ? kv_seen : (int64_t)kv_live;
-                            const uint32_t after = (uint32_t)(kv + pk + oh_f);  // < 2^31 + 2^20 + 2^17
-                            int64_t press;
+                            if (kSig && cc.proxy)  // the ledger: tau_dec o_hat per request routed here and not done
+                                b = (uint64_t)cc.ledger_tau * (uint64_t)s.sum;
+                            const uint32_t after = (uint32_t)kv + (uint32_t)pk + oh_f;  // < 2^31 + 2^20 + 2^17
+                            uint64_t press;
                             if (P.kv_cap_magic != 0) {
                                 const uint64_t lo = (uint64_t)after * (uint32_t)P.kv_cap_magic;
-                                const uint64_t hi = (uint64_t)after * (uint32_t)(P.kv_cap_magic >> 32);
-                                press = (int64_t)((hi + (lo >> 32)) >> 16);
+                                press = ((uint64_t)after * (uint32_t)(P.kv_cap_magic >> 32) + (lo >> 32)) >> 16;
                             } else {
-                                press = (int64_t)(((uint64_t)after << 16) / (uint64_t)P.kv_cap);
+                                press = ((uint64_t)after << 16) / (uint64_t)P.kv_cap;
                             }
-                            if (press > kPressureClamp) press = kPressureClamp;
-                            if (cc.ablate & CTR_ABLATE_PRESSURE) press = 0;
-                            const int64_t own = oh_f * cc.tau_dec;
-                            const int64_t priced = own + ((((own * press) >> 16) * cc.rho) >> 8);
-                            const int64_t load = cc.w_b * b + cc.w_s * priced;
-                            cost = (uint64_t)(load * sig + cc.w_q * (int64_t)s.q * 65536);
-                        } else if (pol == CTR_POLICY_LENGTH_HEURISTIC && ohk >= P.heur_thresh) {
-                            cost = (uint64_t)s.sum;
-                        } else {
-                            cost = (uint64_t)s.q;
+                            const uint32_t p18 = (press < kPressureClamp ? (uint32_t)press : (uint32_t)kPressureClamp) &
+                                                 cc.press_mask;
+                            const uint64_t own = (uint64_t)oh_f * cc.tau_dec;  // < 2^37
+                            work = own + ((((own * p18) >> 16) * cc.rho) >> 8);
                         }
+                        if (b > (uint64_t)kBacklogClamp) b = (uint64_t)kBacklogClamp;
+                        const uint32_t queue = (uint32_t)(is_pre ? ring_n : s.q);
+                        cost = (b * cc.w_b + work * cc.w_s) * cc.sigma[ck] + cc.w_q16 * queue;
+                    } else if (is_pre) {
+                        cost = (uint64_t)ring_n;
+                    } else {
+                        cost = pol == CTR_POLICY_LENGTH_HEURISTIC && ohk >= P.heur_thresh ? (uint64_t)s.sum : (uint64_t)s.q;
                     }
                     if (pol == CTR_POLICY_LEARNED_P2 && (is_pre || is_dec)) {
                         // power of two choices: only two sampled candidates per pool are priced
@@ -784,15 +825,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                         if (me != c0 && me != c1) cost = kEmpty;
                     }
                 }
-                const int amin_p = group_argmin<G>(is_pre ? cost : kEmpty, gl);
-                const int amin_d = group_argmin<G>(is_dec ? cost : kEmpty, gl);
-                int ip, id;
-                if (pol == CTR_POLICY_ROUND_ROBIN) {
-                    ip = rr_p;
-                    id = rr_d;
-                } else {
-                    ip = amin_p;
-                    id = amin_d - P.n_pre;
+                int ip = rr_p, id = rr_d;
+                if (G < 32 || pol != CTR_POLICY_ROUND_ROBIN) {  // a whole warp's row has one policy
+                    const int amin_p = group_argmin<G>(is_pre ? cost : kEmpty, gl);
+                    const int amin_d = group_argmin<G>(is_dec ? cost : kEmpty, gl);
+                    if (pol != CTR_POLICY_ROUND_ROBIN) {
+                        ip = amin_p;
+                        id = amin_d - P.n_pre;
+                    }
                 }
                 rr_p = rr_p + 1 == P.n_pre ? 0 : rr_p + 1;
                 rr_d = rr_d + 1 == P.n_dec ? 0 : rr_d + 1;
@@ -879,7 +919,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
             }
         }
         if (live && is_dec) {
-            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, tb, ob, -1, kv_seen, sum_is_o_hat,
+            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat,
                                                 oob);
         }
 
