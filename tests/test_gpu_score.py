@@ -129,6 +129,35 @@ def test_every_line_on_the_envelope(orc, n_inst):
     _check(orc, p, oh, cls, Q, A, kap, W.SCORE_CONSTS, am, cost)
 
 
+@pytest.mark.parametrize("n_inst", [64, 65, 95, 96, 97, 255, 256])
+@pytest.mark.parametrize("state", ["random", "twins", "every_line", "one_slope", "falling"])
+def test_wide_pool_envelopes(orc, n_inst, state):
+    """Both sides of the 64-instance line and of whole warps: random lines, pairs of equal ones, an envelope of every
+    line, parallel lines (one segment), and lines each below the one before it at every o_hat (the last one wins)."""
+    ctr = need_gpu()
+    rng = np.random.default_rng(n_inst)
+    d = np.arange(n_inst)
+    Q = rng.integers(0, 65536, n_inst).astype(np.float32)
+    A = rng.integers(0, 256, n_inst).astype(np.float32)
+    kap = rng.random(n_inst, dtype=np.float32)
+    if state == "twins":
+        Q, A, kap = (np.repeat(v[:(n_inst + 1) // 2], 2)[:n_inst] for v in (Q, A, kap))
+    elif state == "every_line":
+        Q, A = (37.0 * d * d * (64.0 / n_inst) ** 2).astype(np.float32), np.zeros(n_inst, np.float32)
+        kap = ((n_inst - d) / n_inst).astype(np.float32)
+    elif state == "one_slope":
+        kap[:] = 0.25
+    elif state == "falling":
+        Q, A = (1000.0 * (n_inst - d)).astype(np.float32), np.zeros(n_inst, np.float32)
+        kap = ((n_inst - d) / n_inst).astype(np.float32)
+    n = 6_001
+    oh = np.floor(rng.random(n) * 3300.0).astype(np.float32)
+    p = np.floor(rng.random(n) * 4000.0 + 16.0).astype(np.float32)
+    cls = rng.integers(0, 4, n).astype(np.uint8)
+    am, cost = _run(ctr, p, oh, cls, Q, A, kap, W.SCORE_CONSTS)
+    _check(orc, p, oh, cls, Q, A, kap, W.SCORE_CONSTS, am, cost)
+
+
 def test_hand_computed_exact(orc):
     ctr = need_gpu()
     with open(os.path.join(GOLDEN, "score_hand.json")) as f:
