@@ -1012,25 +1012,14 @@ int sim_rows_per_warp(int width, int64_t n_rows)
 
 int sim_max_resident_warps(int* warps_per_block, int* blocks)
 {
-    int dev = 0, sms = 0, per_sm = 0, per_sm_g = 0;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    // the smallest occupancy over the group widths and modes at 8 blocks per
+    // the launch bound of the instantiations with the fewest registers: every width and mode has 8 blocks an
     // SM, so one workspace size fits every launch
-    per_sm = 1 << 30;
-    const void* kernels[12] = {
-        (const void*)sim_kernel<4, 0, 8>, (const void*)sim_kernel<8, 0, 8>, (const void*)sim_kernel<16, 0, 8>,
-        (const void*)sim_kernel<32, 0, 8>, (const void*)sim_kernel<4, 1, 8>, (const void*)sim_kernel<8, 1, 8>,
-        (const void*)sim_kernel<16, 1, 8>, (const void*)sim_kernel<32, 1, 8>, (const void*)sim_kernel<4, 2, 8>,
-        (const void*)sim_kernel<8, 2, 8>, (const void*)sim_kernel<16, 2, 8>, (const void*)sim_kernel<32, 2, 8>};
-    for (const void* k : kernels) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_g, k, kWarpsPerBlock * 32, 0) != cudaSuccess)
-            return 0;
-        if (per_sm_g < per_sm) per_sm = per_sm_g;
-    }
     *warps_per_block = kWarpsPerBlock;
-    *blocks = sms * per_sm;
-    return sms * per_sm * kWarpsPerBlock;
+    *blocks = sms * 8;
+    return sms * 8 * kWarpsPerBlock;
 }
 
 namespace {

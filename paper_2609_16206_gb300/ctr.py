@@ -12,6 +12,7 @@ import ctypes as C
 import os
 import threading
 
+import numpy as np
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -90,7 +91,7 @@ def lib():
             vp, i32, i64 = C.c_void_p, C.c_int32, C.c_int64
             L.ctr_gen_trace.argtypes = [C.POINTER(CtrTraceCfg), i32, i64, i64, CtrRequests, vp]
             L.ctr_gen_trace.restype = C.c_int
-            L.ctr_score_batch.argtypes = [vp, vp, vp, i64, vp, vp, vp, i32, C.POINTER(C.c_float), vp, vp, vp, vp]
+            L.ctr_score_batch.argtypes = [vp, vp, vp, i64, vp, vp, vp, i32, vp, vp, vp, vp, vp]
             L.ctr_score_batch.restype = C.c_int
             L.ctr_score_stream_probe.argtypes = [vp, vp, vp, i64, vp, vp, vp]
             L.ctr_score_stream_probe.restype = C.c_int
@@ -149,9 +150,9 @@ def _ptr(t):
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    if stream is None:  # the current stream's handle, without a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 # ---------------------------------------------------------------- struct conversion
@@ -241,7 +242,11 @@ def ctr_gen_trace(trace_cfg, n_replicas: int, replica_offset: int, n_req: int, o
 
 def ctr_score_batch(prompt_len, pred_out, slo_class, q_tokens, n_active, kv_occ, consts, out_argmin, out_cost,
                     status=None, stream=None):
-    cv = (C.c_float * CTR_SCORE_N_CONST)(*[float(x) for x in consts])
+    if type(consts) is np.ndarray and consts.dtype == np.float32 and consts.shape == (CTR_SCORE_N_CONST,):
+        consts = np.ascontiguousarray(consts)  # read during the call, where it lies
+        cv = consts.__array_interface__["data"][0]
+    else:
+        cv = (C.c_float * CTR_SCORE_N_CONST)(*[float(x) for x in consts])
     _check("ctr_score_batch", lib().ctr_score_batch(
         _ptr(prompt_len), _ptr(pred_out), _ptr(slo_class), int(prompt_len.numel()), _ptr(q_tokens), _ptr(n_active),
         _ptr(kv_occ), int(q_tokens.numel()), cv, _ptr(out_argmin), _ptr(out_cost), _ptr(status), _stream(stream)))
