@@ -206,20 +206,75 @@ __device__ __forceinline__ void heap_pop_bin(uint64_t* h, int32_t& n, uint64_t& 
     top = ck_ld(h, 1, lim, bad);
 }
 
-// the heap operations of a kernel instantiation: binary with batched prefill, else 4-ary
-template <bool kBin>
+// 32-ary variants for a warp whose lanes all simulate the same instance (every
+// lane calls with the same arguments and makes the same stores): a node's
+// children, 32 consecutive entries, are one load of the warp and their minimum
+// two redux.sync, so a level costs one child's worth of instructions instead of
+// 32 and a heap of up to 33 keys has one.  Node j sits at position j + 3, its
+// children at 32 j + 4 .. 32 j + 35: the 4-ary region's size serves.
+__device__ __forceinline__ void heap_push_warp(uint64_t* h, int32_t& n, uint64_t& top, uint64_t key, int64_t lim,
+                                               bool& bad)
+{
+    int i = kHeapRoot + n++;
+    while (i > kHeapRoot) {
+        const int parent = ((i - 4) >> 5) + kHeapRoot;
+        const uint64_t pv = ck_ld(h, parent, lim, bad);
+        if (pv < key) break;
+        ck_st(h, i, lim, pv, bad);
+        i = parent;
+    }
+    ck_st(h, i, lim, key, bad);
+    if (i == kHeapRoot) top = key;
+}
+
+__device__ __forceinline__ void heap_pop_warp(uint64_t* h, int32_t& n, uint64_t& top, int64_t lim, bool& bad)
+{
+    const int m = n--;
+    if (m == 1) {
+        top = kEmpty;
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int lastp = kHeapRoot + m - 1;
+    const uint64_t last = ck_ld(h, lastp, lim, bad);
+    int i = kHeapRoot;
+    uint64_t first = last;  // what comes to the root
+    for (;;) {
+        const int c = 32 * (i - kHeapRoot) + 4;  // first child
+        if (c >= lastp) break;
+        const uint64_t v = c + lane < lastp ? ck_ld(h, c + lane, lim, bad) : kEmpty;
+        const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
+        const uint32_t mhi = __reduce_min_sync(kFull, hi);
+        const uint32_t mlo = __reduce_min_sync(kFull, hi == mhi ? lo : 0xffffffffu);
+        const uint64_t cv = ((uint64_t)mhi << 32) | mlo;
+        if (last < cv) break;
+        if (i == kHeapRoot) first = cv;
+        ck_st(h, i, lim, cv, bad);
+        i = c + __ffs(__ballot_sync(kFull, v == cv)) - 1;
+    }
+    ck_st(h, i, lim, last, bad);
+    top = first;
+}
+
+// the heap operations of a kernel instantiation: binary with batched prefill, 32-ary where a whole warp
+// simulates one instance, else 4-ary
+template <int kArity>
 __device__ __forceinline__ void hpush(uint64_t* h, int32_t& n, uint64_t& top, uint64_t key, int64_t lim, bool& bad)
 {
-    if constexpr (kBin)
+    if constexpr (kArity == 2)
         heap_push_bin(h, n, top, key, lim, bad);
+    else if constexpr (kArity == 32)
+        heap_push_warp(h, n, top, key, lim, bad);
     else
         heap_push(h, n, top, key, lim, bad);
 }
-template <bool kBin>
+template <int kArity>
 __device__ __forceinline__ void hpop(uint64_t* h, int32_t& n, uint64_t& top, int64_t lim, bool& bad)
 {
-    if constexpr (kBin)
+    if constexpr (kArity == 2)
         heap_pop_bin(h, n, top, lim, bad);
+    else if constexpr (kArity == 32)
+        heap_pop_warp(h, n, top, lim, bad);
     else
         heap_pop(h, n, top, lim, bad);
 }
@@ -337,7 +392,7 @@ __device__ __forceinline__ void cut_run(Decode& s, int64_t tp)
 template <int kArity>
 __device__ __forceinline__ void push_pending(Decode& s, uint64_t* pend, uint64_t key, int64_t lim, bool& bad)
 {
-    hpush<kArity == 2>(pend, s.pend_n, s.pend_top, key, lim, bad);
+    hpush<kArity>(pend, s.pend_n, s.pend_top, key, lim, bad);
     if (s.n_act == 0)
         s.step_end = (int64_t)(s.pend_top >> kKeyBits);
     else if (s.w_n == 0)
@@ -352,7 +407,7 @@ __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, c
 {
     while (s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= t) {
         const uint32_t k = (uint32_t)(s.pend_top & kKeyMask);
-        hpop<kArity == 2>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
+        hpop<kArity>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
         if (--room < 0) return CTR_EOVERFLOW;
         int pos = s.w_head + s.w_n;
         if (pos >= P.cap_wait) pos -= P.cap_wait;
@@ -386,7 +441,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
             const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
             if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
             V.set_done(k, tev, bad);
-            hpop<kArity == 2>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
+            hpop<kArity>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
             s.q -= 1;
             s.kv_res -= pk + ok;
             s.kv_rsv -= pk + ok;
@@ -413,13 +468,13 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
             s.w_n -= 1;
             s.w_head = s.w_n == 0 || s.w_head + 1 == P.cap_wait ? 0 : s.w_head + 1;  // an empty ring restarts at 0
         } else {
-            hpop<kArity == 2>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
+            hpop<kArity>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
             if (--room < 0) return CTR_EOVERFLOW;
         }
         s.kv_rsv += pk + ok;
         s.kv_res += pk;
-        hpush<kArity == 2>(act, s.n_act, s.act_top, ((uint64_t)(uint32_t)(s.step_idx + ok) << kKeyBits) | k,
-                           heap_stride(P.cap_act), bad);
+        hpush<kArity>(act, s.n_act, s.act_top, ((uint64_t)(uint32_t)(s.step_idx + ok) << kKeyBits) | k,
+                      heap_stride(P.cap_act), bad);
         if (admitted > 0) V.set_first(k, (int64_t)last, bad);
         last = k;
         admitted += 1;
@@ -478,29 +533,182 @@ __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimPar
     }
 }
 
-// Per-request bounds, arrival order (CTR_EINVAL before anything is simulated).
+// A prefill lane keeps its state in decode fields it does not use (fewer live
+// registers): step_end the end of its last prefill (of the running batch, when
+// batched), act_top the ring's front entry (end << 21 | p, read while it holds
+// any), sum the prompt tokens of the prefills in the ring, w_head / w_n the ring.
+// Retire the serial prefills that ended by T.
+template <bool kSig>
+__device__ __forceinline__ void retire_prefills(Decode& s, int64_t T, const SimParams& P, const int64_t* ring, bool& bad)
+{
+    const int64_t thr = ((T + 1) << kRingPBits) - 1;  // entries whose prefill ended by T
+    while (s.w_n > 0 && s.act_top <= (uint64_t)thr) {
+        if constexpr (kSig) s.sum -= s.act_top & kRingPMask;
+        s.w_head = s.w_head + 1 == P.cap_ring ? 0 : s.w_head + 1;
+        s.w_n -= 1;
+        s.act_top = s.w_n > 0 ? (uint64_t)ck_ld(ring, s.w_head, (int64_t)P.cap_ring, bad) : (uint64_t)kNever;
+    }
+    if (s.w_n == 0) s.w_head = 0;
+}
+
+// Batched prefill: the running batch of run_n members (run_p tokens, ending at
+// step_end); the queue behind it, cut FCFS into budget-limited batches, forms
+// q_batches, the last of q_tail tokens.
+struct BatchQueue {
+    int32_t run_n, q_batches;
+    int64_t run_p, q_tail;
+};
+
+// One request as the router sees it.
+struct Request {
+    int64_t k, T;
+    uint32_t p, o_hat;
+    int cls;
+};
+
+// The cost of instance `me` (of its pool) for a request under the row's policy
+// (not round-robin), and kEmpty where the policy does not consider it.
+template <bool kSig, bool kBat>
+__device__ __forceinline__ uint64_t instance_cost(const SimParams& P, const ConstsDev& cc, int pol, bool is_pre, int me,
+                                                  const Decode& s, const BatchQueue& bq, int64_t kv_seen,
+                                                  const Request& rq)
+{
+    if (pol != CTR_POLICY_LEARNED && pol != CTR_POLICY_LEARNED_P2) {
+        if (is_pre) return (uint64_t)s.w_n;
+        return pol == CTR_POLICY_LENGTH_HEURISTIC && (int32_t)rq.o_hat >= P.heur_thresh ? (uint64_t)s.sum : (uint64_t)s.q;
+    }
+    // backlog and own work of the instance, then the cost both kinds share
+    // (feature ablation, sec. V-F, is in the constants: see ConstsDev)
+    const int64_t T = rq.T;
+    uint64_t b = 0, work;
+    if (is_pre) {
+        const int64_t rest = s.step_end > T ? s.step_end - T : 0;
+        if (kSig && cc.proxy)  // the ledger: tau_pre0 + tau_pre p per prefill not yet ended
+            b = (uint64_t)cc.tau_pre0 * (uint32_t)s.w_n + (uint64_t)cc.tau_pre * (uint64_t)s.sum;
+        else if (kBat && P.pre_batch > 0)  // the running batch's rest, then the queue's batches
+            b = (uint64_t)((bq.run_n > 0 ? rest : 0) + P.pre_base * (int64_t)bq.q_batches + P.pre_tok * (s.sum - bq.run_p));
+        else
+            b = (uint64_t)rest;
+        work = (uint64_t)cc.tau_pre * rq.p + cc.tau_pre0;
+    } else {
+        const uint32_t oh_f = rq.o_hat & cc.oh_mask;
+        int32_t kv = (int32_t)kv_seen;
+        const bool polled = kSig && cc.poll_us > 0;
+        if (!(kSig && cc.proxy && polled)) {
+            const int32_t tokens = ends_by(s, T) * s.n_act;  // of the run's steps that have ended
+            const int32_t kv_live = s.kv_res + tokens;
+            if (!polled) kv = kv_live;
+            if (!(kSig && cc.proxy)) {
+                const uint64_t R = (uint64_t)(s.sum - tokens);
+                const uint64_t step = (uint64_t)(P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act + kv_term(kv_live, P));
+                const uint32_t nd = (uint32_t)(s.n_act > 1 ? s.n_act : 1);
+                if (((R | (step << 10)) >> 32) == 0 && nd <= (uint32_t)kRecipN) {
+                    const uint64_t lo = (uint64_t)(uint32_t)R * (uint32_t)step;  // < 2^54
+                    b = nd > 1 ? __umul64hi(lo, __ldg(&kRecipTable.v[nd])) : lo;
+                } else {
+                    const uint64_t lo = R * step;
+                    b = __umul64hi(R, step) != 0 || lo >= (1ull << 62) ? (uint64_t)kBacklogClamp : lo / nd;
+                }
+            }
+        }
+        if (kSig && cc.proxy)  // the ledger: tau_dec o_hat per request routed here and not done
+            b = (uint64_t)cc.ledger_tau * (uint64_t)s.sum;
+        const uint32_t after = (uint32_t)kv + rq.p + oh_f;  // < 2^31 + 2^20 + 2^17
+        uint64_t press;
+        if (P.kv_cap_magic != 0) {
+            const uint64_t lo = (uint64_t)after * (uint32_t)P.kv_cap_magic;
+            press = ((uint64_t)after * (uint32_t)(P.kv_cap_magic >> 32) + (lo >> 32)) >> 16;
+        } else {
+            press = ((uint64_t)after << 16) / (uint64_t)P.kv_cap;
+        }
+        const uint32_t p18 = (press < kPressureClamp ? (uint32_t)press : (uint32_t)kPressureClamp) & cc.press_mask;
+        const uint64_t own = (uint64_t)oh_f * cc.tau_dec;  // < 2^37
+        work = own + ((((own * p18) >> 16) * cc.rho) >> 8);
+    }
+    if (b > (uint64_t)kBacklogClamp) b = (uint64_t)kBacklogClamp;
+    const uint32_t queue = (uint32_t)(is_pre ? s.w_n : s.q);
+    const uint64_t cost = (b * cc.w_b + work * cc.w_s) * cc.sigma[rq.cls] + cc.w_q16 * queue;
+    if (pol == CTR_POLICY_LEARNED_P2) {
+        // power of two choices: only two sampled candidates per pool are priced
+        const Philox4 u = philox4x32_10((uint32_t)rq.k, (uint32_t)T, (uint32_t)((uint64_t)T >> 32), 0x5032u, 0x243F6A88u,
+                                        0x85A308D3u);
+        const uint32_t n_pool = is_pre ? (uint32_t)P.n_pre : (uint32_t)P.n_dec;
+        const uint32_t a0 = is_pre ? u.v[2] : u.v[0], a1 = is_pre ? u.v[3] : u.v[1];
+        const uint32_t c0 = (uint32_t)(((uint64_t)a0 * n_pool) >> 32);
+        uint32_t c1 = c0;
+        if (n_pool > 1) {
+            c1 = c0 + 1 + (uint32_t)(((uint64_t)a1 * (n_pool - 1)) >> 32);
+            if (c1 >= n_pool) c1 -= n_pool;
+        }
+        if ((uint32_t)me != c0 && (uint32_t)me != c1) return kEmpty;
+    }
+    return cost;
+}
+
+// the end of a serial prefill of p tokens that reaches, at T, an instance busy until `busy`
+__device__ __forceinline__ int64_t prefill_end(const SimParams& P, int64_t busy, int64_t T, uint32_t p)
+{
+    const int64_t start = busy > T ? busy : T;
+    return start + P.pre_base + (int64_t)(int32_t)P.pre_tok * (int32_t)p;
+}
+
+// Commit a serial prefill ending at `end` to its lane (the caller has checked the time limit).
+template <bool kSig>
+__device__ __forceinline__ int push_prefill(Decode& s, int64_t end, uint32_t p, const SimParams& P, int64_t* ring,
+                                            bool& bad)
+{
+    if (s.w_n == P.cap_ring) return CTR_EOVERFLOW;
+    s.step_end = end;
+    int pos = s.w_head + s.w_n;
+    if (pos >= P.cap_ring) pos -= P.cap_ring;
+    const int64_t e = (end << kRingPBits) | p;
+    ck_st(ring, pos, (int64_t)P.cap_ring, e, bad);
+    if (s.w_n == 0) s.act_top = (uint64_t)e;
+    s.w_n += 1;
+    if constexpr (kSig) s.sum += p;
+    return CTR_OK;
+}
+
+// Commit a request to its decode lane at T: KV-ready at `ready` (-1: not known yet), `weight` its share of the
+// lane's in-flight sum.
+template <int kArity>
+__device__ __forceinline__ int queue_decode(Decode& s, int64_t T, int64_t k, int64_t ready, int64_t weight,
+                                            const SimParams& P, uint64_t* pend, uint32_t* wait, bool& bad)
+{
+    // requests routed here whose KV is not ready yet, exactly: first move
+    // those already ready (kept in the heap until the step end) if it matters
+    if (s.q - s.w_n - s.n_act >= P.cap_pend) {
+        const int rc = flush_ready<kArity>(s, T, P.cap_wait - s.w_n, P, pend, wait, bad);
+        if (rc != CTR_OK) return rc;
+    }
+    if (s.q - s.w_n - s.n_act == P.cap_pend || (ready >= 0 && s.pend_n == P.cap_pend_store)) return CTR_EOVERFLOW;
+    if (ready >= 0)
+        push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, heap_stride(P.cap_pr), bad);
+    s.q += 1;
+    s.sum += weight;
+    return CTR_OK;
+}
+
+// One request's bounds and its place in arrival order (`before`: the previous one's arrival).
+__device__ __forceinline__ bool request_valid(const SimParams& P, int64_t i, int64_t before, bool& bad)
+{
+    const int64_t t = ck_ld(P.trace.arrival_us, i, P.trace_len, bad);
+    const int64_t p = ck_ld(P.trace.prompt_len, i, P.trace_len, bad);
+    const int64_t o = ck_ld(P.trace.true_out, i, P.trace_len, bad);
+    const int64_t oh = ck_ld(P.trace.pred_out, i, P.trace_len, bad);
+    const int64_t c = ck_ld(P.trace.slo_class, i, P.trace_len, bad);
+    return !(t < 0 || t >= kArrivalLimit || p < 0 || p > (1 << 20) || o < 1 || o > (1 << 20) || p + o > P.kv_cap ||
+             oh < 0 || oh > (1 << 17) || c >= P.n_classes || t < before);
+}
+
+// Every request of a replica (CTR_EINVAL before anything is simulated); one warp.
 __device__ __forceinline__ bool row_valid(const SimParams& P, int64_t tb, int lane, bool& bad)
 {
-    int64_t prev_last = 0;
     for (int64_t base = 0; base < P.n_req; base += 32) {
         const int64_t k = base + lane;
-        const bool live = k < P.n_req;
-        int64_t t = 0;
-        bool bad = false;
-        if (live) {
-            t = ck_ld(P.trace.arrival_us, tb + k, P.trace_len, bad);
-            const int64_t p = ck_ld(P.trace.prompt_len, tb + k, P.trace_len, bad);
-            const int64_t o = ck_ld(P.trace.true_out, tb + k, P.trace_len, bad);
-            const int64_t oh = ck_ld(P.trace.pred_out, tb + k, P.trace_len, bad);
-            const int64_t c = ck_ld(P.trace.slo_class, tb + k, P.trace_len, bad);
-            bad = t < 0 || t >= kArrivalLimit || p < 0 || p > (1 << 20) || o < 1 || o > (1 << 20) ||
-                  p + o > P.kv_cap || oh < 0 || oh > (1 << 17) || c >= P.n_classes;
-        }
-        int64_t before = __shfl_up_sync(kFull, t, 1);
-        if (lane == 0) before = prev_last;
-        if (live && t < before) bad = true;
-        if (__any_sync(kFull, bad)) return false;
-        prev_last = __shfl_sync(kFull, t, 31);
+        bool ok = true;
+        if (k < P.n_req) ok = request_valid(P, tb + k, k > 0 ? ck_ld(P.trace.arrival_us, tb + k - 1, P.trace_len, bad) : 0, bad);
+        if (__any_sync(kFull, !ok)) return false;
     }
     return true;
 }
@@ -605,21 +813,18 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
         s.pend_top = kEmpty; s.act_top = kEmpty;
         s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
-        // A lane simulates a prefill or a decode instance, never both, so a prefill
-        // lane keeps its state in decode fields it does not use (fewer live registers).
-        int64_t& busy = s.step_end;    // end of the last prefill (of the running batch, when batched)
-        uint64_t& ring_front = s.act_top;  // the ring's front entry (end << 21 | p), read while ring_n > 0
-        int64_t& ring_sum_p = s.sum;       // prompt tokens of the prefills in the ring
+        // (a lane simulates a prefill or a decode instance, never both: see retire_prefills)
+        int64_t& busy = s.step_end;
+        int64_t& ring_sum_p = s.sum;
         int32_t& ring_head = s.w_head;
         int32_t& ring_n = s.w_n;
         int64_t kv_seen = 0, last_poll = -1;     // decode lanes: occupancy at the last poll instant
         int32_t rr_p = 0, rr_d = 0;
         uint64_t h = 0;
         int err = CTR_OK;
-        // batched prefill lanes: busy = end of the running batch of run_n members (run_p tokens); the
-        // queue behind it, cut FCFS into budget-limited batches, forms q_batches, the last of q_tail tokens
-        int32_t run_n = 0, q_batches = 0;
-        int64_t run_p = 0, q_tail = 0;
+        BatchQueue bq = {0, 0, 0, 0};
+        int32_t &run_n = bq.run_n, &q_batches = bq.q_batches;
+        int64_t &run_p = bq.run_p, &q_tail = bq.q_tail;
         const bool batched = kBat && P.pre_batch > 0;
 
         // Batched prefill: end every batch that ends by T, start the next at that
@@ -726,15 +931,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                             err = decode_advance<kSig, kArity>(s, T, P, pend, act, wait, V, tsnap, kv_seen,
                                                                sum_is_o_hat, oob);
                     } else if (is_pre && !batched) {
-                        const int64_t thr = ((T + 1) << kRingPBits) - 1;  // entries whose prefill ended by T
-                        while (ring_n > 0 && ring_front <= (uint64_t)thr) {
-                            if constexpr (kSig) ring_sum_p -= ring_front & kRingPMask;
-                            ring_head = ring_head + 1 == P.cap_ring ? 0 : ring_head + 1;
-                            ring_n -= 1;
-                            ring_front = ring_n > 0 ? (uint64_t)ck_ld(ring, ring_head, (int64_t)P.cap_ring, oob)
-                                                    : (uint64_t)kNever;
-                        }
-                        if (ring_n == 0) ring_head = 0;
+                        retire_prefills<kSig>(s, T, P, ring, oob);
                     }
                 }
                 if (__ballot_sync(kFull, err != CTR_OK) & gmask) live = false;
@@ -749,82 +946,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                 const int64_t ohk = __shfl_sync(kFull, my_oh, j, G);
                 // 2. price the candidates and take the argmin of each pool
                 uint64_t cost = kEmpty;
-                if (live && pol != CTR_POLICY_ROUND_ROBIN) {
-                    if (learned_row) {
-                        // backlog and own work of the lane's instance, then the cost both kinds share
-                        // (feature ablation, sec. V-F, is in the constants: see ConstsDev)
-                        uint64_t b = 0, work = 0;
-                        if (is_pre) {
-                            if (kSig && cc.proxy) {  // the ledger: tau_pre0 + tau_pre p per prefill not yet ended
-                                b = (uint64_t)cc.tau_pre0 * (uint32_t)ring_n + (uint64_t)cc.tau_pre * (uint64_t)ring_sum_p;
-                            } else if (batched) {  // the running batch's rest, then the queue's batches
-                                b = (uint64_t)((run_n > 0 && busy > T ? busy - T : 0) + P.pre_base * (int64_t)q_batches +
-                                               P.pre_tok * (ring_sum_p - run_p));
-                            } else {
-                                b = (uint64_t)(busy > T ? busy - T : 0);
-                            }
-                            work = (uint64_t)cc.tau_pre * (uint32_t)pk + cc.tau_pre0;
-                        } else if (is_dec) {
-                            const uint32_t oh_f = (uint32_t)ohk & cc.oh_mask;
-                            int32_t kv = (int32_t)kv_seen;
-                            const bool polled = kSig && cc.poll_us > 0;
-                            if (!(kSig && cc.proxy && polled)) {
-                                const int32_t tokens = ends_by(s, T) * s.n_act;  // of the run's steps that have ended
-                                const int32_t kv_live = s.kv_res + tokens;
-                                if (!polled) kv = kv_live;
-                                if (!(kSig && cc.proxy)) {
-                                    const uint64_t R = (uint64_t)(s.sum - tokens);
-                                    const uint64_t step = (uint64_t)(P.dec_base + (int64_t)(int32_t)P.dec_seq * s.n_act +
-                                                                     kv_term(kv_live, P));
-                                    const uint32_t nd = (uint32_t)(s.n_act > 1 ? s.n_act : 1);
-                                    if (((R | (step << 10)) >> 32) == 0 && nd <= (uint32_t)kRecipN) {
-                                        const uint64_t lo = (uint64_t)(uint32_t)R * (uint32_t)step;  // < 2^54
-                                        b = nd > 1 ? __umul64hi(lo, __ldg(&kRecipTable.v[nd])) : lo;
-                                    } else {
-                                        const uint64_t lo = R * step;
-                                        b = __umul64hi(R, step) != 0 || lo >= (1ull << 62) ? (uint64_t)kBacklogClamp : lo / nd;
-                                    }
-                                }
-                            }
-                            if (kSig && cc.proxy)  // the ledger: tau_dec o_hat per request routed here and not done
-                                b = (uint64_t)cc.ledger_tau * (uint64_t)s.sum;
-                            const uint32_t after = (uint32_t)kv + (uint32_t)pk + oh_f;  // < 2^31 + 2^20 + 2^17
-                            uint64_t press;
-                            if (P.kv_cap_magic != 0) {
-                                const uint64_t lo = (uint64_t)after * (uint32_t)P.kv_cap_magic;
-                                press = ((uint64_t)after * (uint32_t)(P.kv_cap_magic >> 32) + (lo >> 32)) >> 16;
-                            } else {
-                                press = ((uint64_t)after << 16) / (uint64_t)P.kv_cap;
-                            }
-                            const uint32_t p18 = (press < kPressureClamp ? (uint32_t)press : (uint32_t)kPressureClamp) &
-                                                 cc.press_mask;
-                            const uint64_t own = (uint64_t)oh_f * cc.tau_dec;  // < 2^37
-                            work = own + ((((own * p18) >> 16) * cc.rho) >> 8);
-                        }
-                        if (b > (uint64_t)kBacklogClamp) b = (uint64_t)kBacklogClamp;
-                        const uint32_t queue = (uint32_t)(is_pre ? ring_n : s.q);
-                        cost = (b * cc.w_b + work * cc.w_s) * cc.sigma[ck] + cc.w_q16 * queue;
-                    } else if (is_pre) {
-                        cost = (uint64_t)ring_n;
-                    } else {
-                        cost = pol == CTR_POLICY_LENGTH_HEURISTIC && ohk >= P.heur_thresh ? (uint64_t)s.sum : (uint64_t)s.q;
-                    }
-                    if (pol == CTR_POLICY_LEARNED_P2 && (is_pre || is_dec)) {
-                        // power of two choices: only two sampled candidates per pool are priced
-                        const Philox4 u = philox4x32_10((uint32_t)k, (uint32_t)T, (uint32_t)((uint64_t)T >> 32),
-                                                        0x5032u, 0x243F6A88u, 0x85A308D3u);
-                        const uint32_t n_pool = is_pre ? (uint32_t)P.n_pre : (uint32_t)P.n_dec;
-                        const uint32_t a0 = is_pre ? u.v[2] : u.v[0], a1 = is_pre ? u.v[3] : u.v[1];
-                        const uint32_t c0 = (uint32_t)(((uint64_t)a0 * n_pool) >> 32);
-                        uint32_t c1 = c0;
-                        if (n_pool > 1) {
-                            c1 = c0 + 1 + (uint32_t)(((uint64_t)a1 * (n_pool - 1)) >> 32);
-                            if (c1 >= n_pool) c1 -= n_pool;
-                        }
-                        const uint32_t me = is_pre ? (uint32_t)gl : (uint32_t)(gl - P.n_pre);
-                        if (me != c0 && me != c1) cost = kEmpty;
-                    }
-                }
+                if (live && pol != CTR_POLICY_ROUND_ROBIN && (is_pre || is_dec))
+                    cost = instance_cost<kSig, kBat>(P, cc, pol, is_pre, is_pre ? gl : gl - P.n_pre, s, bq, kv_seen,
+                                                     Request{k, T, (uint32_t)pk, (uint32_t)ohk, ck});
                 int ip = rr_p, id = rr_d;
                 if (G < 32 || pol != CTR_POLICY_ROUND_ROBIN) {  // a whole warp's row has one policy
                     const int amin_p = group_argmin<G>(is_pre ? cost : kEmpty, gl);
@@ -866,40 +990,13 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                         }
                     }
                 } else if (live && gl == ip) {
-                    const int64_t start = busy > T ? busy : T;
-                    const int64_t end = start + P.pre_base + (int64_t)(int32_t)P.pre_tok * (int32_t)pk;
+                    const int64_t end = prefill_end(P, busy, T, (uint32_t)pk);
                     ready = end + (int64_t)(int32_t)P.xfer_tok * (int32_t)pk;
-                    if (ready >= kTimeLimit) {
-                        err = CTR_EOVERFLOW;
-                    } else if (ring_n == P.cap_ring) {
-                        err = CTR_EOVERFLOW;
-                    } else {
-                        busy = end;
-                        int pos = ring_head + ring_n;
-                        if (pos >= P.cap_ring) pos -= P.cap_ring;
-                        const int64_t e = (end << kRingPBits) | pk;
-                        ck_st(ring, pos, (int64_t)P.cap_ring, e, oob);
-                        if (ring_n == 0) ring_front = (uint64_t)e;
-                        ring_n += 1;
-                        if constexpr (kSig) ring_sum_p += pk;
-                    }
+                    err = ready >= kTimeLimit ? CTR_EOVERFLOW : push_prefill<kSig>(s, end, (uint32_t)pk, P, ring, oob);
                 }
                 ready = __shfl_sync(kFull, ready, ip, G);
-                if (live && gl == P.n_pre + id && ready < kTimeLimit) {
-                    // requests routed here whose KV is not ready yet, exactly: first move
-                    // those already ready (kept in the heap until the step end) if it matters
-                    if (s.q - s.w_n - s.n_act >= P.cap_pend)
-                        err = flush_ready<kArity>(s, T, P.cap_wait - s.w_n, P, pend, wait, oob);
-                    if (err != CTR_OK || s.q - s.w_n - s.n_act == P.cap_pend ||
-                        (ready >= 0 && s.pend_n == P.cap_pend_store)) {
-                        err = CTR_EOVERFLOW;
-                    } else {
-                        if (ready >= 0)
-                            push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, pr_stride, oob);
-                        s.q += 1;
-                        s.sum += sum_is_o_hat ? ohk : ok;
-                    }
-                }
+                if (live && gl == P.n_pre + id && ready < kTimeLimit)
+                    err = queue_decode<kArity>(s, T, k, ready, sum_is_o_hat ? ohk : ok, P, pend, wait, oob);
                 if (gl == j) my_route = ((uint32_t)ip << 8) | (uint32_t)id;
                 if (__ballot_sync(kFull, err != CTR_OK) & gmask) live = false;
             }
@@ -933,6 +1030,161 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         if (__ballot_sync(kFull, oob) & gmask) status = CTR_EBOUNDS;
 #endif
         if (gl == 0 && has_row) {
+            P.row_status[row] = status;
+            P.row_hash[row] = status == CTR_OK ? h : 0;
+        }
+    }
+}
+
+// One block per row, one warp per instance, for launches of few rows: all lanes
+// of a warp simulate the same instance (same state, same control flow, same
+// stores), so no event waits for another instance's and the heaps are worked by
+// the whole warp.  Every warp follows the row's arrivals.  Per arrival the
+// instances' costs go through shared memory, one barrier, and each warp takes
+// both argmins itself; the ends of all prefill queues ride along in every warp
+// (lane i that of instance i), so the KV-ready time needs no second exchange and
+// a round-robin row needs no barrier at all.  Without batched prefill.
+// Bound by its longest chain an arrival: about 4,100 cycles for the learned
+// router, of them 2,500 one instance's event, 800 its price, 600 the commit
+// (cycle counters around each, 2P+6D).
+constexpr uint64_t kFailed = kEmpty - 1;  // in place of a cost: the row has failed
+template <int kMode, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const __grid_constant__ SimParams P)
+{
+    static_assert(kMode < 2, "no batched prefill");
+    constexpr bool kSig = kMode == 1;
+    constexpr int kArity = 32;
+    __shared__ uint64_t cost_s[2][kWarps];  // arrivals alternate between the two
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int n_inst = P.n_pre + P.n_dec;  // the block's warps
+    unsigned char* sb = P.ws + (int64_t)blockIdx.x * P.slot_bytes;
+    const int64_t pr_stride = heap_stride(P.cap_pr);
+    uint64_t* pend = reinterpret_cast<uint64_t*>(sb) + w * pr_stride;
+    int64_t* ring = reinterpret_cast<int64_t*>(sb) + w * pr_stride;
+    uint64_t* act = reinterpret_cast<uint64_t*>(sb + P.off_act) + w * heap_stride(P.cap_act);
+    uint32_t* wait = reinterpret_cast<uint32_t*>(sb + P.off_wait) + w * P.cap_wait;
+    const bool is_pre = w < P.n_pre;
+    const int64_t per_rep = (int64_t)P.n_sets * P.n_pols;
+    const int64_t n = P.n_req;
+
+    for (int64_t row = blockIdx.x; row < P.n_rows; row += gridDim.x) {
+        const int set = (int)((row / P.n_pols) % P.n_sets);
+        const int pol = P.pols[row % P.n_pols];
+        const ConstsDev& cc = P.sets[set];
+        const bool learned_row = pol == CTR_POLICY_LEARNED || pol == CTR_POLICY_LEARNED_P2;
+        const bool sum_is_o_hat = pol == CTR_POLICY_LENGTH_HEURISTIC || (kSig && learned_row && cc.proxy);
+        const int64_t tb = row / per_rep * n, ob = row * n;
+        const RowView<true> V(P, tb, ob);
+        bool oob = false;  // bounds-checked builds: an index of this warp fell outside its buffer
+
+        // per-request bounds and arrival order, a stretch of 32 requests per warp
+        bool bad = false;
+        for (int64_t k = (int64_t)w * 32 + lane; k < n; k += (int64_t)n_inst * 32)
+            bad = bad || !request_valid(P, tb + k, k > 0 ? ck_ld(P.trace.arrival_us, tb + k - 1, P.trace_len, oob) : 0, oob);
+        const bool valid = !__syncthreads_or(bad);
+
+        Decode s;
+        s.step_end = is_pre ? 0 : kNever; s.run = 0; s.step = 1; s.inv_step = 1.0f;
+        s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
+        s.pend_top = kEmpty; s.act_top = kEmpty;
+        s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
+        const BatchQueue bq = {0, 0, 0, 0};
+        int64_t kv_seen = 0, last_poll = -1;  // occupancy at the last poll instant
+        int64_t busy = 0;                     // lane i: the end of prefill instance i's last prefill
+        int ip = P.n_pre - 1, id = P.n_dec - 1;
+        uint64_t h = 0;
+        int err = CTR_OK;
+        bool go = valid;  // the same in every thread of the block
+        for (int64_t base = 0; go && base < n; base += 32) {
+            const int64_t kl = base + lane;
+            int64_t my_t = 0;
+            uint32_t my_pc = 0, my_o = 0, my_oh = 0, my_route = 0;
+            if (kl < n) {
+                my_t = ck_ld(P.trace.arrival_us, tb + kl, P.trace_len, oob);
+                my_pc = (uint32_t)ck_ld(P.trace.prompt_len, tb + kl, P.trace_len, oob) |
+                        ((uint32_t)ck_ld(P.trace.slo_class, tb + kl, P.trace_len, oob) << 24);
+                my_o = (uint32_t)ck_ld(P.trace.true_out, tb + kl, P.trace_len, oob);
+                my_oh = (uint32_t)ck_ld(P.trace.pred_out, tb + kl, P.trace_len, oob);
+            }
+            const int cnt = (int)(n - base < 32 ? n - base : 32);
+            for (int j = 0; go && j < cnt; ++j) {
+                const int64_t k = base + j;
+                const int64_t T = __shfl_sync(kFull, my_t, j);
+                const uint32_t pc = __shfl_sync(kFull, my_pc, j);
+                const uint32_t pk = pc & 0xFFFFFFu, ok = __shfl_sync(kFull, my_o, j), ohk = __shfl_sync(kFull, my_oh, j);
+                // 1. the instance's events up to the arrival
+                if (err == CTR_OK) {
+                    if (is_pre) {
+                        retire_prefills<kSig>(s, T, P, ring, oob);
+                    } else {
+                        int64_t tsnap = -1;  // >= 0: the occupancy at this time is recorded on the way
+                        if (kSig && cc.poll_us > 0) {
+                            const int64_t tp = (int64_t)div_recip((uint64_t)T, (uint64_t)cc.poll_us, cc.poll_recip) *
+                                               cc.poll_us;
+                            if (tp > last_poll) {
+                                tsnap = tp;
+                                last_poll = tp;
+                            }
+                        }
+                        err = decode_advance<kSig, kArity>(s, T, P, pend, act, wait, V, tsnap, kv_seen, sum_is_o_hat, oob);
+                    }
+                }
+                // 2. the costs of all instances and the argmin of each pool
+                if (pol == CTR_POLICY_ROUND_ROBIN) {
+                    ip = ip + 1 == P.n_pre ? 0 : ip + 1;
+                    id = id + 1 == P.n_dec ? 0 : id + 1;
+                } else {
+                    uint64_t cost = kFailed;
+                    if (err == CTR_OK)
+                        cost = instance_cost<kSig, false>(P, cc, pol, is_pre, is_pre ? w : w - P.n_pre, s, bq, kv_seen,
+                                                          Request{k, T, pk, ohk, (int)(pc >> 24)});
+                    uint64_t* const slot = cost_s[k & 1];
+                    if (lane == 0) slot[w] = cost;
+                    __syncthreads();
+                    const uint64_t c = lane < n_inst ? slot[lane] : kEmpty;
+                    if (__any_sync(kFull, c == kFailed)) {  // every warp reads the same costs
+                        go = false;
+                        break;
+                    }
+                    ip = warp_argmin(lane < P.n_pre ? c : kEmpty);
+                    id = warp_argmin(lane < P.n_pre ? kEmpty : c) - P.n_pre;
+                }
+                // 3. commit
+                const int64_t end = prefill_end(P, __shfl_sync(kFull, busy, ip), T, pk);
+                const int64_t ready = end + (int64_t)(int32_t)P.xfer_tok * (int32_t)pk;
+                if (ready >= kTimeLimit) {  // the same in every warp
+                    err = CTR_EOVERFLOW;
+                    go = false;
+                    break;
+                }
+                if (lane == ip) busy = end;
+                if (err == CTR_OK) {
+                    if (w == ip)
+                        err = push_prefill<kSig>(s, end, pk, P, ring, oob);
+                    else if (w == P.n_pre + id)
+                        err = queue_decode<kArity>(s, T, k, ready, sum_is_o_hat ? ohk : ok, P, pend, wait, oob);
+                }
+                if (lane == j) my_route = ((uint32_t)ip << 8) | (uint32_t)id;
+            }
+            if (go && w == 0 && kl < n) {  // the routing term of the row checksum
+                h += hterm(kl, 1, (uint64_t)my_route);
+                if (P.i_pre) ck_st(P.i_pre, ob + kl, P.out_len, (uint8_t)(my_route >> 8), oob);
+                if (P.i_dec) ck_st(P.i_dec, ob + kl, P.out_len, (uint8_t)(my_route & 0xFF), oob);
+            }
+        }
+        if (go && !is_pre && err == CTR_OK)  // drain: every remaining event
+            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat, oob);
+
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) h += __shfl_xor_sync(kFull, h, off);
+        int status = CTR_OK;
+        if (__syncthreads_or(err == CTR_ETIMEOUT)) status = CTR_ETIMEOUT;
+        if (__syncthreads_or(err == CTR_EOVERFLOW)) status = CTR_EOVERFLOW;
+        if (!valid) status = CTR_EINVAL;
+#if CTR_BOUNDS_CHECK
+        if (__syncthreads_or(oob)) status = CTR_EBOUNDS;
+#endif
+        if (threadIdx.x == 0) {
             P.row_status[row] = status;
             P.row_hash[row] = status == CTR_OK ? h : 0;
         }
@@ -1049,9 +1301,36 @@ cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+// A block per row, a warp per instance, where every block is resident at 128
+// registers (16 warps an SM) and has at most 16 warps.  2,000 requests, four
+// policies, 2P+6D: 152 rows 3.9 ms against 4.5 with a row per warp, 304 rows
+// 4.3 / 4.5, 400 rows (a second wave) 6.2 / 4.5; 3P+9D, 152 rows: 3.9 / 4.4;
+// proxy's signals, 152 rows: 3.4 / 4.3; 4P+28D (32 warps, 64 registers): 5.1 / 4.0.
+constexpr int kRowWarpsPerSM = 16;
+bool row_per_block(const SimParams& p, int sms)
+{
+    const int64_t n_inst = p.n_pre + p.n_dec;
+    return p.pre_batch == 0 && n_inst <= 16 && p.n_rows * n_inst <= (int64_t)sms * kRowWarpsPerSM && p.n_slots >= p.n_rows &&
+           p.rows_per_warp == 1;
+}
+
 template <int kMode>
 cudaError_t launch_mode(const SimParams& p, int blocks, cudaStream_t stream)
 {
+    if constexpr (kMode < 2) {
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+        const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (row_per_block(p, sms)) {
+            const unsigned threads = (unsigned)(p.n_pre + p.n_dec) * 32;
+            if (threads <= 8 * 32)
+                sim_row_kernel<kMode, 8><<<(unsigned)p.n_rows, threads, 0, stream>>>(p);
+            else
+                sim_row_kernel<kMode, 16><<<(unsigned)p.n_rows, threads, 0, stream>>>(p);
+            return cudaGetLastError();
+        }
+    }
     switch (32 / p.rows_per_warp) {
     case 4: return launch_width<4, kMode>(p, blocks, stream);
     case 8: return launch_width<8, kMode>(p, blocks, stream);

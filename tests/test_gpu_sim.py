@@ -134,6 +134,28 @@ def test_rows_per_warp_same_results(orc, sc, R, deployed):
     _check_rows(orc, sc, sets, pols, [host_trace(tr, r) for r in range(min(R, 3))], spread, N)
 
 
+@pytest.mark.parametrize("sc", [W.SimCfg(), W.SimCfg(n_prefill=2, n_decode=6), W.SimCfg(n_prefill=1, n_decode=8),
+                                W.SimCfg(n_prefill=4, n_decode=12), W.SimCfg(n_prefill=4, n_decode=13),
+                                W.SimCfg(n_prefill=2, n_decode=6, kv_cap_tokens=9_000),
+                                W.SimCfg(n_prefill=2, n_decode=6, cap_active=9, cap_waiting=8, cap_pending=8)],
+                         ids=["1p3d", "2p6d", "1p8d", "4p12d", "4p13d", "scarce", "small_caps"])
+@pytest.mark.parametrize("deployed", [0, 1])
+def test_row_per_block_same_rows(orc, sc, deployed):
+    """The same replicas in a launch of few rows (a block per row, up to 16 instances) and in one of many (rows in
+    warps): equal rows, full or failed, and the oracle's; heaps past one block of 32 children."""
+    ctr = need_gpu()
+    sets = [W.as_deployed(W.CALIBRATED) if deployed else W.CALIBRATED, W.CALIBRATED.replace(rho_q8=900, w_q_us=0)]
+    pols, R, N = list(W.ALL_POLICIES) + [W.POLICY_LEARNED_P2], 260, 900
+    tc = W.replica_sweep().trace.replace(rate_mreq=(3000, 20000), prompt_max=min(8192, sc.kv_cap_tokens // 2), out_max=4096)
+    tr = gen(ctr, tc, R, N)
+    many = simulate(ctr, sc, sets, pols, tr, R, N)
+    few = simulate(ctr, sc, sets, pols, {k: v[:2].contiguous() for k, v in tr.items()}, 2, N)
+    for key in few:
+        rows = few["status"] == 0 if key != "status" else slice(None)
+        assert np.array_equal(few[key][rows], many[key][:len(few[key])][rows]), key
+    _check_rows(orc, sc, sets, pols, [host_trace(tr, r) for r in range(2)], few, N)
+
+
 @pytest.mark.parametrize("kv_div,o_max", [(1, 1 << 13), (3, 1 << 15), (1 << 20, 1 << 20), (1 << 31, 1 << 20)])
 @pytest.mark.parametrize("dec_base,kv_cap", [(1, (1 << 23) - 1), (3_000, 1 << 23), (3_000, (1 << 31) - 1)])
 def test_long_runs_of_steps(orc, kv_div, o_max, dec_base, kv_cap):
