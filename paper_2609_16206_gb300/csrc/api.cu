@@ -385,9 +385,8 @@ int ctr_goodput(const ctr_sim_cfg* cfg, ctr_requests trace, int32_t n_replicas, 
     p.t_done = t_done_us;
     p.met = met_count;
     p.p99 = p99_ttft_us;
-    const cudaError_t e = launch_goodput(p, (cudaStream_t)stream);
-    if (e != cudaSuccess || !p99_tpot_us) return cuda_status(e);
-    return cuda_status(launch_tpot(p, p99_tpot_us, (cudaStream_t)stream));
+    p.p99_tpot = p99_tpot_us;
+    return cuda_status(launch_goodput(p, (cudaStream_t)stream));
 }
 
 }  // extern "C"

@@ -207,15 +207,17 @@ struct GoodputParams {
     const int64_t* t_done;
     int64_t* met;
     int64_t* p99;
+    int64_t* p99_tpot;          // optional, not with row_hash: nearest-rank P99 TPOT, -1 without a request of two tokens
     // optional (both or neither): add each OK row's first-token and completion
     // checksum terms to row_hash in the same pass over the outputs
     uint64_t* row_hash;
     const int32_t* row_status;
     const uint64_t* kmix;  // optional with row_hash: the table of launch_mix_table for n_req
+    // set by launch_goodput: room for kept values per P99; every row starts on 16 bytes (read two requests at a time)
+    int32_t cand_cap;
+    bool pairs;
 };
 cudaError_t launch_goodput(const GoodputParams& p, cudaStream_t stream);
-// Each row's nearest-rank P99 TPOT into p99_tpot[row] (-1 when no request has two tokens or more).
-cudaError_t launch_tpot(const GoodputParams& p, int64_t* p99_tpot, cudaStream_t stream);
 
 // ---------------------------------------------------------------- standalone scorer
 struct ScoreParams {

@@ -1,43 +1,53 @@
 // goodput.cu -- SLO goodput inputs per simulated row (ctr_goodput):
 // the count of requests meeting both SLOs of their class (sec. IV-B targets,
 // Table 2 goodput), the exact nearest-rank P99 TTFT and, on request, the
-// exact nearest-rank P99 TPOT (Table 2 columns; tpot_kernel at the end).
+// exact nearest-rank P99 TPOT (Table 2 columns).
 //
-// One block per unit of up to kRows rows of one replica, which share the
-// replica's trace and request indices.  Pass 0 reads the unit once: per
-// request the trace's arrival, output length and class, then each row's
-// t_first and t_done; per row the met count and, when the rows fit in shared
-// memory (kStage) and every TTFT lies in [0, 2^32), a histogram of the TTFTs
-// over logarithmic bins (64 per octave, monotone in the TTFT) with each
-// request's bin kept in shared memory.  For each row a block scan then finds
-// the bin holding the P99's rank; the requests of that bin (a few dozen in
-// practice) are gathered, their exact TTFTs read back, and the value of the
-// remaining rank among them counted out exactly.  A row with a TTFT outside
-// [0, 2^32), more than kCand requests in the P99's bin, or too many requests
-// to stage falls back to a radix select over the exact TTFTs read from global
-// memory (11-bit digits, most significant first).  Called from ctr_simulate
-// with kHash, pass 0 also sums each row's checksum terms of first-token and
-// completion times; the request-only half of those terms is read from the
-// call's table (launch_mix_table) when ctr_simulate has one, else mixed once
-// per request for the unit's rows.
+// One block per row.  A P99 needs the largest hundredth of its row only, so a
+// sample of the row (256 evenly spaced groups of four neighbours, a memory sector
+// each, in a histogram over logarithmic bins, 64 per octave) first gives a
+// threshold that about 3 % of the values reach, and the one pass over the row
+// then keeps those that do: per request the trace's arrival, output length and
+// class and the row's t_first and t_done.  The P99 is the value of the remaining
+// rank among the kept ones: their histogram over the same bins finds its bin,
+// whose few members are counted out.  A row whose kept values are fewer than the
+// rank needs or more than there is room for (thousands of equal values at the
+// P99), or of 2^32 and more, takes an exact radix select over all its values read
+// from global memory (11-bit digits, most significant first).  A TPOT is compared
+// without a division (floor(d / m) >= t is d >= t m) and divided only when kept.
+// Called from ctr_simulate with kHash, the pass also sums each row's checksum
+// terms of first-token and completion times; the request-only half of those terms
+// is read from the call's table (launch_mix_table) when ctr_simulate has one,
+// else mixed in the pass.
 #include "ctr_internal.cuh"
 
 namespace ctr {
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kLogBins = 2112;  // bin 0: a TTFT of 0; then 64 per octave of [1, 2^32)
-constexpr int kCand = 512;      // requests of the P99's bin selected exactly in shared memory
-constexpr int kDigit = 11;      // radix select fallback
+constexpr int kMaxThreads = 512;  // of a block: 128 in launches of many rows
+constexpr int kLogBins = 2112;  // bin 0: a value of 0; then 64 per octave of [1, 2^32)
+constexpr int kHistWords = kLogBins / 2;  // two 16-bit counts a word (no more than kSample or kMaxCand values are counted)
+constexpr int kSample = 1024;   // sampled requests of a row (all of a shorter one)
+constexpr int kMaxCand = 8192;  // most values kept
+constexpr int kFew = 128;       // members of the rank's bin counted out directly
+constexpr int kDigit = 11;      // radix select
 constexpr int kBins = 1 << kDigit;
-static_assert(kBins <= kLogBins, "the radix fallback reuses the histogram");
+static_assert(kBins <= 2 * kHistWords, "the radix select takes the place of two 16-bit histograms");
 
-// Monotone bin of a TTFT in [0, 2^32): the exponent and the top 6 mantissa bits
+// Monotone bin of a value in [0, 2^32): the exponent and the top 6 mantissa bits
 // of its fp32 value rounded toward zero (exact integer to float conversion
-// order is kept by round-toward-zero, so x <= y gives bin(x) <= bin(y)).
-__device__ __forceinline__ uint32_t log_bin(uint32_t x)
+// order is kept by round-toward-zero, so x <= y gives bin(x) <= bin(y)); values
+// outside go to the end bins.
+__device__ __forceinline__ uint32_t log_bin(int64_t x)
 {
-    return x == 0 ? 0u : (__float_as_uint(__uint2float_rz(x)) >> 17) - (126u << 6);
+    if (x <= 0) return 0u;
+    if (x >= (int64_t(1) << 32)) return kLogBins - 1;
+    return (__float_as_uint(__uint2float_rz((uint32_t)x)) >> 17) - (126u << 6);
+}
+// the least value of a bin, the least of all for bin 0
+__device__ __forceinline__ int64_t bin_floor(uint32_t b)
+{
+    return b == 0 ? INT64_MIN : (int64_t)ceilf(__uint_as_float((b + (126u << 6)) << 17));
 }
 
 template <typename T, typename Op>
@@ -49,7 +59,7 @@ __device__ T block_reduce(T v, T identity, Op op, T* scratch)
     if (lane == 0) scratch[wid] = v;
     __syncthreads();
     if (wid == 0) {
-        v = lane < kThreads / 32 ? scratch[lane] : identity;
+        v = lane < (int)blockDim.x / 32 ? scratch[lane] : identity;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, off));
         if (lane == 0) scratch[0] = v;
@@ -60,16 +70,19 @@ __device__ T block_reduce(T v, T identity, Op op, T* scratch)
     return r;
 }
 
-// The bin of hist[0 .. nb) holding 0-based rank `rank`, and the count of the
-// bins before it, to every thread: each thread sums a contiguous run of bins, a
-// block scan of the sums finds the run, its thread walks it.
-__device__ void find_rank_bin(const uint32_t* hist, int nb, int64_t rank, uint32_t* pick, uint32_t* wsum)
+// The bin holding 0-based rank `rank` among the counts of nb bins, and the count
+// of the bins before it, to every thread in pick[0] and pick[1]: each thread sums
+// a contiguous run of bins, a block scan of the sums finds the run, its thread
+// walks it.  at(b) is the count of bin b.
+template <typename At>
+__device__ void find_rank_bin(const At& at, int nb, int64_t rank, uint32_t* pick, uint32_t* wsum)
 {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int per = (nb + kThreads - 1) / kThreads;
+    const int per = (nb + (int)blockDim.x - 1) / (int)blockDim.x;
     const int b0 = tid * per, b1 = b0 + per < nb ? b0 + per : nb;
     uint32_t sum = 0;
-    for (int b = b0; b < b1; ++b) sum += hist[b];
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) sum += at(b);
     uint32_t incl = sum;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -85,11 +98,12 @@ __device__ void find_rank_bin(const uint32_t* hist, int nb, int64_t rank, uint32
         uint32_t acc = excl;
         int bin = b0;
         for (int b = b0; b < b1; ++b) {
-            if ((int64_t)(acc + hist[b]) > rank) {
+            const uint32_t c = at(b);
+            if ((int64_t)(acc + c) > rank) {
                 bin = b;
                 break;
             }
-            acc += hist[b];
+            acc += c;
         }
         pick[0] = (uint32_t)bin;
         pick[1] = acc;
@@ -97,20 +111,22 @@ __device__ void find_rank_bin(const uint32_t* hist, int nb, int64_t rank, uint32
     __syncthreads();
 }
 
-
-// Shared scratch of the per-row selection.
+// Shared scratch of the selections.
 struct SelScratch {
-    int64_t red64[kThreads / 32];
-    uint32_t wsum[kThreads / 32];
+    int64_t red64[kMaxThreads / 32];
+    uint32_t wsum[kMaxThreads / 32];
     uint32_t pick[2];
-    uint32_t n_cand;
-    int32_t cand_k[kCand];
-    int64_t cand_v[kCand];
+    uint32_t n_few;
+    uint32_t few[kFew];
 };
 
-// One row's P99 TTFT (and its met count, already reduced) into P.p99 / P.met:
-// from its histogram and staged bins when `staged`, else by the radix select
-// over the TTFTs in global memory (which reuses `hist`).  Block-collective.
+// 16-bit counts, two to a word
+__device__ __forceinline__ void count16(uint32_t* h, uint32_t b, bool& bad)
+{
+    if (ck_ok(b, kLogBins, bad)) atomicAdd(&h[b >> 1], (b & 1u) ? 0x10000u : 1u);
+}
+__device__ __forceinline__ uint32_t at16(const uint32_t* h, int b) { return (h[b >> 1] >> ((b & 1) * 16)) & 0xffffu; }
+
 #if CTR_BOUNDS_CHECK
 #define CTR_CK_FLAG_PARAM , bool& bad
 #define CTR_CK_FLAG_ARG , bad
@@ -118,73 +134,41 @@ struct SelScratch {
 #define CTR_CK_FLAG_PARAM
 #define CTR_CK_FLAG_ARG
 #endif
-__device__ void select_row(const GoodputParams& P, int64_t row, int64_t tb, int64_t n, int32_t met, bool staged,
-                           uint32_t* hist, const uint16_t* bins, SelScratch& S CTR_CK_FLAG_PARAM)
+
+// Exact radix select: the value of 0-based rank `rank` among those of
+// val(k, v) over k < n (false: k has none).  Block-collective; every thread
+// returns it.
+template <typename Val>
+__device__ int64_t radix_rank(const Val& val, int64_t n, int64_t rank, uint32_t* hist, SelScratch& S CTR_CK_FLAG_PARAM)
 {
 #if !CTR_BOUNDS_CHECK
     bool bad = false;  // dead: the accessors below compile to plain accesses
 #endif
-    const int64_t trace_len = (P.n_rows / P.rows_per_replica) * n, out_len = P.n_rows * n;
-    const int tid = threadIdx.x;
-    const int64_t ob = row * n;
-    const int64_t rank = (99 * n + 99) / 100 - 1;  // 0-based nearest rank
-    if (staged) {
-        if (tid == 0) S.n_cand = 0;
-        find_rank_bin(hist, kLogBins, rank, S.pick, S.wsum);  // its barriers also publish n_cand
-        const uint32_t B = S.pick[0];
-        const int64_t r_in = rank - (int64_t)S.pick[1];  // rank among the bin's requests
-        for (int64_t k = tid; k < n; k += kThreads) {
-            if (ck_ld(bins, k, n, bad) == B) {
-                const uint32_t i = atomicAdd(&S.n_cand, 1u);
-                if (i < (uint32_t)kCand) S.cand_k[i] = (int32_t)k;
-            }
-        }
-        __syncthreads();
-        const int c = (int)S.n_cand;
-        if (c <= kCand) {
-            for (int i = tid; i < c; i += kThreads) {
-                const int64_t k = S.cand_k[i];
-                S.cand_v[i] = ck_ld(P.t_first, ob + k, out_len, bad) - ck_ld(P.trace.arrival_us, tb + k, trace_len, bad);
-            }
-            __syncthreads();
-            // the candidate whose position in (value, slot) order is the remaining rank
-            for (int i = tid; i < c; i += kThreads) {
-                const int64_t v = S.cand_v[i];
-                int64_t pos = 0;
-                for (int j = 0; j < c; ++j) {
-                    const int64_t w = S.cand_v[j];
-                    pos += w < v || (w == v && j < i);
-                }
-                if (pos == r_in) P.p99[row] = v;
-            }
-            if (tid == 0) P.met[row] = met;
-            __syncthreads();
-            return;
-        }
-    }
-    // ---- fallback: exact radix select over (TTFT - min) read from global memory
+    const int tid = threadIdx.x, nt = blockDim.x;
     int64_t mn = INT64_MAX, mx = INT64_MIN;
-    for (int64_t k = tid; k < n; k += kThreads) {
-        const int64_t t = ck_ld(P.t_first, ob + k, out_len, bad) - ck_ld(P.trace.arrival_us, tb + k, trace_len, bad);
-        mn = t < mn ? t : mn;
-        mx = t > mx ? t : mx;
+    for (int64_t k = tid; k < n; k += nt) {
+        int64_t v;
+        if (val(k, v)) {
+            mn = v < mn ? v : mn;
+            mx = v > mx ? v : mx;
+        }
     }
     mn = block_reduce<int64_t>(mn, INT64_MAX, [](int64_t a, int64_t b) { return a < b ? a : b; }, S.red64);
     mx = block_reduce<int64_t>(mx, INT64_MIN, [](int64_t a, int64_t b) { return a > b ? a : b; }, S.red64);
     const uint64_t range = (uint64_t)mx - (uint64_t)mn;
     int shift = range == 0 ? 0 : 64 - __clzll((long long)range);  // bits still undetermined
-    uint64_t prefix = 0;                                            // chosen high bits of (ttft - mn)
-    int64_t rk = rank;                                              // rank among the candidates
+    uint64_t prefix = 0;                                            // chosen high bits of (value - mn)
     while (shift > 0) {
         const int dbits = shift < kDigit ? shift : kDigit;
         const int above = shift;  // candidates agree with prefix on bits >= above
         shift -= dbits;
-        for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+        for (int i = tid; i < kBins; i += nt) hist[i] = 0;
         __syncthreads();
         const uint32_t dmask = (1u << dbits) - 1u;
-        for (int64_t k = tid; k < n; k += kThreads) {
-            const uint64_t v = (uint64_t)(ck_ld(P.t_first, ob + k, out_len, bad) -
-                                          ck_ld(P.trace.arrival_us, tb + k, trace_len, bad)) - (uint64_t)mn;
+        for (int64_t k = tid; k < n; k += nt) {
+            int64_t tv;
+            if (!val(k, tv)) continue;
+            const uint64_t v = (uint64_t)tv - (uint64_t)mn;
             const bool match = above >= 64 || (v >> above) == (prefix >> above);
             if (match) {
                 const uint32_t b = (uint32_t)(v >> shift) & dmask;
@@ -192,271 +176,276 @@ __device__ void select_row(const GoodputParams& P, int64_t row, int64_t tb, int6
             }
         }
         __syncthreads();
-        find_rank_bin(hist, kBins, rk, S.pick, S.wsum);
+        find_rank_bin([&](int b) { return hist[b]; }, kBins, rank, S.pick, S.wsum);
         prefix |= (uint64_t)S.pick[0] << shift;
-        rk -= S.pick[1];
+        rank -= S.pick[1];
         __syncthreads();
     }
-    if (tid == 0) {
-        P.met[row] = met;
-        P.p99[row] = (int64_t)((uint64_t)mn + prefix);
+    return (int64_t)((uint64_t)mn + prefix);
+}
+
+// the nearest rank of the P99 among m values, 0-based
+__device__ __forceinline__ int64_t p99_rank(int64_t m) { return (99 * m + 99) / 100 - 1; }
+
+// A threshold that at least the top m - p99_rank(m) of about m values reach, from the histogram of `taken`
+// samples of them: the floor of the bin of the sample's j-th largest, j six standard deviations above the
+// expected count (neighbours are alike; exactly the count when every value is in the sample).
+// Block-collective.
+__device__ int64_t threshold(const uint32_t* hist, int64_t taken, int64_t m, SelScratch& S)
+{
+    if (taken <= 0) return INT64_MAX;
+    const int64_t top = m - p99_rank(m);
+    int64_t j = top;
+    if (taken < m) {
+        const float e = (float)taken * ((float)top / (float)m);
+        j = (int64_t)(e + 6.0f * sqrtf(e)) + 2;
+    }
+    find_rank_bin([&](int b) { return at16(hist, b); }, kLogBins, j < taken ? taken - j : 0, S.pick, S.wsum);
+    const int64_t t = bin_floor(S.pick[0]);
+    __syncthreads();  // pick and wsum are free again
+    return t;
+}
+
+// entries i and i + 1 as one load (bounds-checked builds also check its alignment)
+template <typename V, typename T>
+__device__ __forceinline__ V ck_ldg_pair(const T* p, int64_t i, int64_t len, bool& bad)
+{
+    static_assert(sizeof(V) == 2 * sizeof(T), "a pair");
+    if (CTR_CK_OUT(i, len - 1, bad)) return V();
+#if CTR_BOUNDS_CHECK
+    if (reinterpret_cast<uintptr_t>(p + i) % sizeof(V) != 0) {
+        bad = true;
+        return V();
+    }
+#endif
+    return __ldg(reinterpret_cast<const V*>(p + i));
+}
+
+// The value of rank `rank` among c kept ones (c <= kMaxCand).  Block-collective.
+__device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t* hist, SelScratch& S CTR_CK_FLAG_PARAM)
+{
+#if !CTR_BOUNDS_CHECK
+    bool bad = false;
+#endif
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int i = tid; i < kHistWords; i += nt) hist[i] = 0;
+    if (tid == 0) S.n_few = 0;
+    __syncthreads();
+    for (int i = tid; i < c; i += nt) count16(hist, log_bin(cand[i]), bad);
+    __syncthreads();
+    find_rank_bin([&](int b) { return at16(hist, b); }, kLogBins, rank, S.pick, S.wsum);
+    const uint32_t B = S.pick[0];
+    const int64_t r_in = rank - (int64_t)S.pick[1];  // among the bin's members
+    for (int i = tid; i < c; i += nt) {
+        if (log_bin(cand[i]) == B) {
+            const uint32_t j = atomicAdd(&S.n_few, 1u);
+            if (j < (uint32_t)kFew) S.few[j] = cand[i];
+        }
     }
     __syncthreads();
-}
-
-template <int kRows, bool kStage, bool kHash>
-__global__ void __launch_bounds__(kThreads, 2) goodput_kernel(const GoodputParams P)
-{
-    __shared__ uint32_t hist[kRows][kLogBins];
-    __shared__ SelScratch S;
-    extern __shared__ uint16_t bin_s[];  // kStage: each row's TTFT bins, [kRows][n]
-    const int tid = threadIdx.x;
-    const int64_t n = P.n_req;
-    const int64_t rpr = P.rows_per_replica;
-    const int64_t upr = (rpr + kRows - 1) / kRows;  // units per replica
-    const int64_t n_units = (P.n_rows / rpr) * upr;
-    const int64_t trace_len = (P.n_rows / rpr) * n, out_len = P.n_rows * n;  // entries of the trace and outputs
-
-    for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-        const int64_t rep = unit / upr;
-        const int64_t j0 = (unit - rep * upr) * kRows;
-        const int nr = (int)(rpr - j0 < kRows ? rpr - j0 : kRows);  // rows of this unit
-        const int64_t row0 = rep * rpr + j0;
-        const int64_t tb = rep * n;
-        if (kStage) {
-            for (int i = tid; i < kRows * kLogBins; i += kThreads) (&hist[0][0])[i] = 0;
-            __syncthreads();
-        }
-        int32_t met[kRows];
-        uint64_t h[kRows];  // kHash: each row's first-token and completion checksum terms
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            met[r] = 0;
-            h[r] = 0;
-        }
-        uint32_t wide = 0;  // bit r: row r has a TTFT outside [0, 2^32)
-        bool bad = false;   // bounds-checked builds: an index of this thread fell outside its buffer
-        for (int64_t k = tid; k < n; k += kThreads) {
-            // every load of the request issued before any is used
-            const int64_t ta = ck_ldg(P.trace.arrival_us, tb + k, trace_len, bad);
-            const int64_t o = ck_ldg(P.trace.true_out, tb + k, trace_len, bad);
-            int c = (int)ck_ldg(P.trace.slo_class, tb + k, trace_len, bad);
-            int64_t tf[kRows], td[kRows];
-#pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                if (r < nr) {
-                    tf[r] = ck_ldg(P.t_first, (row0 + r) * n + k, out_len, bad);
-                    td[r] = ck_ldg(P.t_done, (row0 + r) * n + k, out_len, bad);
-                }
-            }
-            if (c >= P.n_classes) c = P.n_classes - 1;
-            const int64_t ttft_slo = P.ttft[c], tpot_slo = P.tpot[c] * (o - 1);
-            uint64_t m2 = 0, m3 = 0;  // the request-only halves of the checksum terms
-            if (kHash) {
-                if (P.kmix) {  // mixed once per call (launch_mix_table)
-                    m2 = ck_ldg(P.kmix, k, 2 * n, bad);
-                    m3 = ck_ldg(P.kmix, n + k, 2 * n, bad);
-                } else {
-                    m2 = mix64((uint64_t(2) << 56) ^ (uint64_t)k);
-                    m3 = mix64((uint64_t(3) << 56) ^ (uint64_t)k);
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < kRows; ++r) {
-                if (r < nr) {
-                    const int64_t ttft = tf[r] - ta;
-                    met[r] += ttft <= ttft_slo && (o == 1 || td[r] - tf[r] <= tpot_slo);
-                    const bool fits = (uint64_t)ttft < (uint64_t(1) << 32);
-                    wide |= (uint32_t)!fits << r;
-                    if (kStage) {
-                        const uint32_t b = fits ? log_bin((uint32_t)ttft) : 0u;
-                        if (ck_ok(b, kLogBins, bad)) atomicAdd(&hist[r][b], 1u);
-                        ck_st(bin_s, (int64_t)r * n + k, (int64_t)kRows * n, (uint16_t)b, bad);
-                    }
-                    if (kHash) h[r] += mix64(m2 ^ (uint64_t)tf[r]) + mix64(m3 ^ (uint64_t)td[r]);
-                }
-            }
-        }
-        wide = (uint32_t)block_reduce<int32_t>((int32_t)wide, 0, [](int32_t a, int32_t b) { return a | b; },
-                                               reinterpret_cast<int32_t*>(S.red64));
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-            if (r < nr) {
-                const int32_t m_r = block_reduce<int32_t>(met[r], 0, [](int32_t a, int32_t b) { return a + b; },
-                                                          reinterpret_cast<int32_t*>(S.red64));
-                const int64_t row = row0 + r;
-                if (kHash) {
-                    const uint64_t h_r = (uint64_t)block_reduce<int64_t>((int64_t)h[r], 0, [](int64_t a, int64_t b) {
-                        return (int64_t)((uint64_t)a + (uint64_t)b);  // sum mod 2^64
-                    }, S.red64);
-                    if (tid == 0 && P.row_status[row] == CTR_OK) P.row_hash[row] += h_r;  // a failed row keeps 0
-                }
-                if (n == 0) {
-                    if (tid == 0) {
-                        P.met[row] = 0;
-                        P.p99[row] = -1;
-                    }
-                    continue;
-                }
-                select_row(P, row, tb, n, m_r, kStage && !((wide >> r) & 1u), hist[r], bin_s + (int64_t)r * n,
-                           S CTR_CK_FLAG_ARG);
-#if CTR_BOUNDS_CHECK
-                if (__syncthreads_or(bad) && tid == 0) {  // a row whose pass left a buffer: both outputs say so
-                    P.met[row] = CTR_EBOUNDS;
-                    P.p99[row] = CTR_EBOUNDS;
-                }
-#endif
-            }
-        }
+    const int m = (int)S.n_few;
+    if (m > kFew) {
+        auto val = [&](int64_t i, int64_t& v) { v = cand[i]; return true; };
+        return radix_rank(val, c, rank, hist, S CTR_CK_FLAG_ARG);
     }
+    for (int i = tid; i < m; i += nt) {  // the member whose position in (value, slot) order is the rank
+        const uint32_t v = S.few[i];
+        int pos = 0;
+        for (int j = 0; j < m; ++j) pos += S.few[j] < v || (S.few[j] == v && j < i);
+        if (pos == r_in) S.pick[0] = v;
+    }
+    __syncthreads();
+    const uint32_t v = S.pick[0];
+    __syncthreads();
+    return v;
 }
 
-// P99 TPOT per row (Table 2): one block per row, each thread taking two
-// requests per pass with all their loads issued first.  A request with o >= 2
-// output tokens has TPOT = (t_done - t_first) / (o - 1) rounded toward zero
-// (the floor, as t_done >= t_first); one-token requests have none.  Pass 1
-// counts the row's M such requests and histograms their TPOTs over the same
-// logarithmic bins as the TTFTs (32-bit quotients when the decode time is
-// below 2^32 us); a block scan finds the bin of the nearest rank
-// ceil(0.99 M) - 1; pass 2 gathers that bin's TPOTs and counts the remaining
-// rank out exactly.  A decode time outside [0, 2^32) or more than kCand
-// requests in the bin fall back to an exact radix select (11-bit digits) over
-// the 64-bit quotients.
-__device__ __forceinline__ bool tpot_of(const GoodputParams& P, int64_t tb, int64_t ob, int64_t k, int64_t& v)
-{
-    const int32_t o = __ldg(&P.trace.true_out[tb + k]);
-    if (o < 2) return false;
-    v = (__ldg(&P.t_done[ob + k]) - __ldg(&P.t_first[ob + k])) / (int64_t)(o - 1);
-    return true;
-}
-// the same for a row whose decode times all lie in [0, 2^32): one 32-bit quotient
-__device__ __forceinline__ bool tpot32_of(const GoodputParams& P, int64_t tb, int64_t ob, int64_t k, uint32_t& v)
-{
-    const int32_t o = __ldg(&P.trace.true_out[tb + k]);
-    if (o < 2) return false;
-    v = (uint32_t)(__ldg(&P.t_done[ob + k]) - __ldg(&P.t_first[ob + k])) / (uint32_t)(o - 1);
-    return true;
-}
 
-__global__ void __launch_bounds__(kThreads, 2) tpot_kernel(const GoodputParams P, int64_t* p99_tpot)
+// Bound by the pass: about 110 warp-instructions for 32 requests (64-bit times,
+// the SLO tables, one kept value in 30) and the bytes in flight.  Eight blocks
+// of 128 threads an SM overlap one row's sample and selection with the others'
+// passes.  4,096 rows x 20,000: 470 us with the P99 TPOT, 324 us without; 873 and
+// 400 us when every request's logarithmic bin was counted and staged in shared
+// memory and the TPOT took two more passes of its own.
+template <bool kHash, bool kTpot>
+__global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputParams P)
 {
-    __shared__ uint32_t hist[kLogBins];
+    __shared__ uint32_t hist[2][kHistWords];  // TTFT and TPOT
     __shared__ SelScratch S;
-    const int tid = threadIdx.x;
+    __shared__ uint32_t n_cand[2];
+    extern __shared__ uint32_t cand_s[];  // kept TTFTs, then TPOTs, cap each
+    const int tid = threadIdx.x, nt = blockDim.x;
     const int64_t n = P.n_req;
+    const int64_t trace_len = (P.n_rows / P.rows_per_replica) * n, out_len = P.n_rows * n;  // entries of trace and outputs
+    const uint32_t cap = (uint32_t)P.cand_cap;
+
     for (int64_t row = blockIdx.x; row < P.n_rows; row += gridDim.x) {
         const int64_t tb = (row / P.rows_per_replica) * n, ob = row * n;
-        for (int i = tid; i < kLogBins; i += kThreads) hist[i] = 0;
+        bool bad = false;  // bounds-checked builds: an index of this thread fell outside its buffer
+
+        // ---- the sample and the thresholds
+        for (int i = tid; i < 2 * kHistWords; i += nt) (&hist[0][0])[i] = 0;
+        if (tid < 2) n_cand[tid] = 0;
+        const int taken = n < kSample ? (int)n : kSample;
+        int32_t taken_many = 0;
         __syncthreads();
-        int32_t m = 0;
-        int32_t wide = 0;  // a decode time outside [0, 2^32)
-        for (int64_t k0 = tid; k0 < n; k0 += 2 * kThreads) {  // two requests per thread, loads first
-            int32_t o[2];
-            int64_t d[2];
+        constexpr int kBatch = 4;  // samples a thread loads before it uses any
+        for (int i0 = tid; i0 < taken; i0 += kBatch * nt) {
+            int64_t ttft[kBatch], dec[kBatch];
+            int32_t o[kBatch];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int64_t k = k0 + u * kThreads < n ? k0 + u * kThreads : k0;
-                o[u] = __ldg(&P.trace.true_out[tb + k]);
-                d[u] = __ldg(&P.t_done[ob + k]) - __ldg(&P.t_first[ob + k]);
+            for (int j = 0; j < kBatch; ++j) {
+                const int i = i0 + j * nt < taken ? i0 + j * nt : i0;
+                const int64_t k = n <= kSample ? i : ((((int64_t)(i >> 2) * n) / (kSample / 4)) & ~int64_t(3)) + (i & 3);
+                const int64_t tf = ck_ldg(P.t_first, ob + k, out_len, bad);
+                ttft[j] = tf - ck_ldg(P.trace.arrival_us, tb + k, trace_len, bad);
+                if (kTpot) {
+                    o[j] = ck_ldg(P.trace.true_out, tb + k, trace_len, bad);
+                    dec[j] = ck_ldg(P.t_done, ob + k, out_len, bad) - tf;
+                }
             }
-            if (k0 + kThreads >= n) o[1] = 0;  // past the end: no request
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (o[u] < 2) continue;
-                m += 1;
-                if ((uint64_t)d[u] < (uint64_t(1) << 32)) {
-                    atomicAdd(&hist[log_bin((uint32_t)d[u] / (uint32_t)(o[u] - 1))], 1u);
-                } else {
-                    wide = 1;
+            for (int j = 0; j < kBatch; ++j) {
+                if (i0 + j * nt >= taken) continue;
+                count16(hist[0], log_bin(ttft[j]), bad);
+                if (kTpot && o[j] >= 2) {
+                    ++taken_many;
+                    count16(hist[1], log_bin((uint64_t)dec[j] < (uint64_t(1) << 32)
+                                                 ? (int64_t)((uint32_t)dec[j] / (uint32_t)(o[j] - 1))
+                                                 : dec[j] / (o[j] - 1)), bad);
                 }
             }
         }
-        const int32_t M = block_reduce<int32_t>(m, 0, [](int32_t a, int32_t b) { return a + b; },
-                                                reinterpret_cast<int32_t*>(S.red64));
-        wide = block_reduce<int32_t>(wide, 0, [](int32_t a, int32_t b) { return a | b; },
-                                     reinterpret_cast<int32_t*>(S.red64));
-        if (M == 0) {
-            if (tid == 0) p99_tpot[row] = -1;
-            continue;
+        if (kTpot) taken_many = block_reduce<int32_t>(taken_many, 0, [](int32_t a, int32_t b) { return a + b; },
+                                                      reinterpret_cast<int32_t*>(S.red64));
+        else
+            __syncthreads();
+        const int64_t t_ttft = threshold(hist[0], taken, n, S);
+        uint32_t t_tpot = 0;  // 0: none
+        if (kTpot && taken_many > 0) {
+            const int64_t t = threshold(hist[1], taken_many, n <= kSample ? taken_many : (int64_t)taken_many * n / kSample, S);
+            t_tpot = t > 0 ? (uint32_t)t : 0;  // below 2^32
         }
-        const int64_t rank = (99 * (int64_t)M + 99) / 100 - 1;  // 0-based nearest rank among the M
-        if (!wide) {
-            if (tid == 0) S.n_cand = 0;
-            find_rank_bin(hist, kLogBins, rank, S.pick, S.wsum);  // its barriers also publish n_cand
-            const uint32_t B = S.pick[0];
-            const int64_t r_in = rank - (int64_t)S.pick[1];
-            for (int64_t k0 = tid; k0 < n; k0 += 2 * kThreads) {
-                int32_t o[2];
-                uint32_t d[2];
+
+        // ---- the pass over the row
+        int32_t met = 0;
+        uint64_t h = 0;     // kHash: the row's first-token and completion checksum terms
+        int32_t many = 0;   // kTpot: requests of two tokens or more
+        int32_t wide = 0;   // a kept TTFT or decode time of 2^32 or more
+        auto request = [&](int64_t k, int64_t ta, int32_t o, int c, int64_t tf, int64_t td) {
+            if (c >= P.n_classes) c = P.n_classes - 1;
+            const int64_t ttft = tf - ta, dec = td - tf;
+            met += ttft <= P.ttft[c] && (o == 1 || dec <= P.tpot[c] * ((int64_t)o - 1));
+            if (ttft >= t_ttft) {
+                const uint32_t i = atomicAdd(&n_cand[0], 1u);
+                if ((uint64_t)ttft >> 32) wide = 1;
+                if (i < cap) cand_s[i] = (uint32_t)ttft;
+            }
+            if (kTpot && o >= 2) {
+                ++many;
+                if (dec >= (int64_t)((uint64_t)t_tpot * (uint32_t)(o - 1))) {
+                    const uint32_t i = atomicAdd(&n_cand[1], 1u);
+                    if ((uint64_t)dec >> 32) wide = 1;
+                    if (i < cap) cand_s[cap + i] = (uint32_t)dec / (uint32_t)(o - 1);
+                }
+            }
+            if (kHash) {
+                const uint64_t m2 = P.kmix ? ck_ldg(P.kmix, k, 2 * n, bad) : mix64((uint64_t(2) << 56) ^ (uint64_t)k);
+                const uint64_t m3 = P.kmix ? ck_ldg(P.kmix, n + k, 2 * n, bad) : mix64((uint64_t(3) << 56) ^ (uint64_t)k);
+                h += mix64(m2 ^ (uint64_t)tf) + mix64(m3 ^ (uint64_t)td);
+            }
+        };
+        // kU requests a thread, every load issued before any is used: neighbours in pairs, one 16-byte load of
+        // each array, where rows are aligned (an even n), else one by one
+        constexpr int kU = 4;
+        for (int64_t base = 0; base < n; base += kU * nt) {
+            int64_t k[kU], a[kU], f[kU], d[kU];
+            int32_t o[kU];
+            int c[kU];
+            if (P.pairs) {
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int64_t k = k0 + u * kThreads < n ? k0 + u * kThreads : k0;
-                    o[u] = __ldg(&P.trace.true_out[tb + k]);
-                    d[u] = (uint32_t)(__ldg(&P.t_done[ob + k]) - __ldg(&P.t_first[ob + k]));
+                for (int u = 0; u < kU; u += 2) {
+                    k[u] = base + u * nt + 2 * tid;
+                    k[u + 1] = k[u] + 1;
+                    const int64_t e = k[u] < n ? k[u] : 0;
+                    const longlong2 a2 = ck_ldg_pair<longlong2>((const long long*)P.trace.arrival_us, tb + e, trace_len, bad);
+                    const int2 o2 = ck_ldg_pair<int2>(P.trace.true_out, tb + e, trace_len, bad);
+                    const uchar2 c2 = ck_ldg_pair<uchar2>(P.trace.slo_class, tb + e, trace_len, bad);
+                    const longlong2 f2 = ck_ldg_pair<longlong2>((const long long*)P.t_first, ob + e, out_len, bad);
+                    const longlong2 d2 = ck_ldg_pair<longlong2>((const long long*)P.t_done, ob + e, out_len, bad);
+                    a[u] = a2.x; a[u + 1] = a2.y;
+                    o[u] = o2.x; o[u + 1] = o2.y;
+                    c[u] = c2.x; c[u + 1] = c2.y;
+                    f[u] = f2.x; f[u + 1] = f2.y;
+                    d[u] = d2.x; d[u + 1] = d2.y;
                 }
-                if (k0 + kThreads >= n) o[1] = 0;
+            } else {
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    if (o[u] < 2) continue;
-                    const uint32_t v = d[u] / (uint32_t)(o[u] - 1);
-                    if (log_bin(v) == B) {
-                        const uint32_t i = atomicAdd(&S.n_cand, 1u);
-                        if (i < (uint32_t)kCand) S.cand_v[i] = (int64_t)v;
-                    }
+                for (int u = 0; u < kU; ++u) {
+                    k[u] = base + u * nt + tid;
+                    const int64_t e = k[u] < n ? k[u] : 0;
+                    a[u] = ck_ldg(P.trace.arrival_us, tb + e, trace_len, bad);
+                    o[u] = ck_ldg(P.trace.true_out, tb + e, trace_len, bad);
+                    c[u] = ck_ldg(P.trace.slo_class, tb + e, trace_len, bad);
+                    f[u] = ck_ldg(P.t_first, ob + e, out_len, bad);
+                    d[u] = ck_ldg(P.t_done, ob + e, out_len, bad);
                 }
             }
-            __syncthreads();
-            const int c = (int)S.n_cand;
-            if (c <= kCand) {
-                for (int i = tid; i < c; i += kThreads) {
-                    const int64_t v = S.cand_v[i];
-                    int64_t pos = 0;
-                    for (int j = 0; j < c; ++j) {
-                        const int64_t w = S.cand_v[j];
-                        pos += w < v || (w == v && j < i);
-                    }
-                    if (pos == r_in) p99_tpot[row] = v;
-                }
-                __syncthreads();
-                continue;
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (k[u] < n) request(k[u], a[u], o[u], c[u], f[u], d[u]);
+        }
+        auto add = [](int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); };  // mod 2^64
+        // met and (below it) the multi-token requests, both < 2^24, and the threads with a wide value
+        const int64_t sums = block_reduce<int64_t>(((int64_t)met << 40) + ((int64_t)many << 16) + wide, 0, add,
+                                                   S.red64);  // its barriers publish the kept values
+        many = (int32_t)(sums >> 16) & 0xffffff;
+        const bool packs = (sums & 0xffff) == 0;
+        if (kHash) {
+            h = (uint64_t)block_reduce<int64_t>((int64_t)h, 0, add, S.red64);
+            if (tid == 0 && P.row_status[row] == CTR_OK) P.row_hash[row] += h;  // a failed row keeps 0
+        }
+
+        // ---- the rank among the kept values, or among all
+        int64_t p99 = -1, p99_tpot = -1;
+        if (n > 0) {
+            const int64_t below = n - (int64_t)n_cand[0], rank = p99_rank(n);
+            if (n_cand[0] <= cap && rank >= below && packs) {
+                p99 = kept_rank(cand_s, (int)n_cand[0], rank - below, hist[0], S CTR_CK_FLAG_ARG);
+            } else {
+                auto ttft_of = [&](int64_t k, int64_t& v) {
+                    v = ck_ld(P.t_first, ob + k, out_len, bad) - ck_ld(P.trace.arrival_us, tb + k, trace_len, bad);
+                    return true;
+                };
+                p99 = radix_rank(ttft_of, n, rank, hist[0], S CTR_CK_FLAG_ARG);
             }
         }
-        // exact radix select over (TPOT - min) of the row's multi-token requests
-        int64_t mn = INT64_MAX, mx = INT64_MIN;
-        for (int64_t k = tid; k < n; k += kThreads) {
-            int64_t v;
-            if (tpot_of(P, tb, ob, k, v)) {
-                mn = v < mn ? v : mn;
-                mx = v > mx ? v : mx;
+        if (kTpot && many > 0) {
+            const int64_t below = many - (int64_t)n_cand[1], rank = p99_rank(many);
+            if (t_tpot > 0 && n_cand[1] <= cap && rank >= below && packs) {
+                p99_tpot = kept_rank(cand_s + cap, (int)n_cand[1], rank - below, hist[0], S CTR_CK_FLAG_ARG);
+            } else {
+                auto tpot_of = [&](int64_t k, int64_t& v) {
+                    const int32_t ok = ck_ld(P.trace.true_out, tb + k, trace_len, bad);
+                    if (ok < 2) return false;
+                    v = (ck_ld(P.t_done, ob + k, out_len, bad) - ck_ld(P.t_first, ob + k, out_len, bad)) / (int64_t)(ok - 1);
+                    return true;
+                };
+                p99_tpot = radix_rank(tpot_of, n, rank, hist[0], S CTR_CK_FLAG_ARG);
             }
         }
-        mn = block_reduce<int64_t>(mn, INT64_MAX, [](int64_t a, int64_t b) { return a < b ? a : b; }, S.red64);
-        mx = block_reduce<int64_t>(mx, INT64_MIN, [](int64_t a, int64_t b) { return a > b ? a : b; }, S.red64);
-        const uint64_t range = (uint64_t)mx - (uint64_t)mn;
-        int shift = range == 0 ? 0 : 64 - __clzll((long long)range);
-        uint64_t prefix = 0;
-        int64_t rk = rank;
-        while (shift > 0) {
-            const int dbits = shift < kDigit ? shift : kDigit;
-            const int above = shift;
-            shift -= dbits;
-            for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
-            __syncthreads();
-            const uint32_t dmask = (1u << dbits) - 1u;
-            for (int64_t k = tid; k < n; k += kThreads) {
-                int64_t tv;
-                if (!tpot_of(P, tb, ob, k, tv)) continue;
-                const uint64_t v = (uint64_t)tv - (uint64_t)mn;
-                if (above >= 64 || (v >> above) == (prefix >> above)) atomicAdd(&hist[(uint32_t)(v >> shift) & dmask], 1u);
-            }
-            __syncthreads();
-            find_rank_bin(hist, kBins, rk, S.pick, S.wsum);
-            prefix |= (uint64_t)S.pick[0] << shift;
-            rk -= S.pick[1];
-            __syncthreads();
+#if CTR_BOUNDS_CHECK
+        const bool out = __syncthreads_or(bad);  // a row whose pass left a buffer: both outputs say so
+#endif
+        if (tid == 0) {
+            P.met[row] = sums >> 40;
+            P.p99[row] = p99;
+            if (kTpot) P.p99_tpot[row] = p99_tpot;
+#if CTR_BOUNDS_CHECK
+            if (out) P.met[row] = P.p99[row] = CTR_EBOUNDS;
+#endif
         }
-        if (tid == 0) p99_tpot[row] = (int64_t)((uint64_t)mn + prefix);
-        __syncthreads();
+        __syncthreads();  // the shared arrays are free for the next row
     }
 }
 
@@ -469,41 +458,26 @@ __global__ void __launch_bounds__(256) mix_table_kernel(uint64_t* t, int64_t n)
     }
 }
 
-template <int kRows, bool kStage>
-cudaError_t launch_rows(const GoodputParams& p, int64_t dyn_bytes, bool hash, int sms, cudaStream_t stream)
+template <bool kHash, bool kTpot>
+cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
 {
-    const void* k = hash ? (const void*)goodput_kernel<kRows, kStage, true>
-                         : (const void*)goodput_kernel<kRows, kStage, false>;
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_bytes);
+    const auto k = goodput_kernel<kHash, kTpot>;
+    const size_t dyn_bytes = (size_t)p.cand_cap * 4 * (kTpot ? 2 : 1);
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCand * 8);
     if (err != cudaSuccess) return err;
+    // 128 threads a row, which overlap best, more while that leaves an SM's 1,024 threads partly idle (4 rows of
+    // 2,000: 15 us with 512, 21 with 128; 32 rows of 50,000: 62 and 169)
+    const int threads = p.n_rows <= (int64_t)sms * 2 ? 512 : p.n_rows <= (int64_t)sms * 4 ? 256 : 128;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, (size_t)dyn_bytes);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn_bytes);
     if (err != cudaSuccess) return err;
-    const int64_t rpr = p.rows_per_replica;
-    int64_t blocks = (p.n_rows / rpr) * ((rpr + kRows - 1) / kRows);
     const int64_t cap = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    if (blocks > cap) blocks = cap;
-    if (hash)
-        goodput_kernel<kRows, kStage, true><<<(unsigned)blocks, kThreads, (size_t)dyn_bytes, stream>>>(p);
-    else
-        goodput_kernel<kRows, kStage, false><<<(unsigned)blocks, kThreads, (size_t)dyn_bytes, stream>>>(p);
+    const int64_t blocks = p.n_rows < cap ? p.n_rows : cap;
+    k<<<(unsigned)blocks, threads, dyn_bytes, stream>>>(p);
     return cudaGetLastError();
 }
 
 }  // namespace
-
-cudaError_t launch_tpot(const GoodputParams& p, int64_t* p99_tpot, cudaStream_t stream)
-{
-    if (p.n_rows == 0) return cudaSuccess;
-    int dev = 0, sms = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (err != cudaSuccess) return err;
-    const int64_t blocks = p.n_rows < (int64_t)sms * 2 ? p.n_rows : (int64_t)sms * 2;
-    tpot_kernel<<<(unsigned)blocks, kThreads, 0, stream>>>(p, p99_tpot);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_mix_table(uint64_t* t, int64_t n, cudaStream_t stream)
 {
@@ -514,27 +488,23 @@ cudaError_t launch_mix_table(uint64_t* t, int64_t n, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-cudaError_t launch_goodput(const GoodputParams& p, cudaStream_t stream)
+cudaError_t launch_goodput(const GoodputParams& given, cudaStream_t stream)
 {
-    if (p.n_rows == 0) return cudaSuccess;
+    if (given.n_rows == 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    // Two blocks per SM when a unit's staged bins, histograms and scratch fit in half the shared memory;
-    // two rows per unit when the replica has them (they share the trace's reads and, without a table, the
-    // request-only checksum mixes).
-    constexpr int64_t kSmemBudget = 108 * 1024;
-    const int64_t fixed = (int64_t)sizeof(SelScratch) + 256;
-    const bool hash = p.row_hash != nullptr;
-    const int64_t n2 = p.n_req * 2;
-    auto fits = [&](int rows) { return n2 > 0 && rows * (n2 + 4 * kLogBins) + fixed <= kSmemBudget; };
-    if (p.rows_per_replica >= 2 && fits(2)) return launch_rows<2, true>(p, 2 * n2, hash, sms, stream);
-    if (fits(1)) return launch_rows<1, true>(p, n2, hash, sms, stream);
-    constexpr int64_t kStageMaxBytes = 200 * 1024;  // one row staged, one block per SM
-    if (n2 > 0 && n2 + 4 * kLogBins + fixed <= kStageMaxBytes) return launch_rows<1, true>(p, n2, hash, sms, stream);
-    return launch_rows<1, false>(p, 0, hash, sms, stream);  // rows too long to stage
+    GoodputParams p = given;
+    p.pairs = p.n_req % 2 == 0 &&
+              ((uintptr_t)p.trace.arrival_us | (uintptr_t)p.t_first | (uintptr_t)p.t_done | (uintptr_t)p.kmix) % 16 == 0 &&
+              (uintptr_t)p.trace.true_out % 8 == 0 && (uintptr_t)p.trace.slo_class % 2 == 0;
+    // room for a sixteenth of the row (3 % is expected, more where a bin holds many)
+    const int64_t room = p.n_req / 16 + 64;
+    p.cand_cap = (int32_t)(room < 512 ? 512 : room > kMaxCand ? kMaxCand : room);
+    if (p.row_hash) return launch_rows<true, false>(p, sms, stream);
+    return p.p99_tpot ? launch_rows<false, true>(p, sms, stream) : launch_rows<false, false>(p, sms, stream);
 }
 
 }  // namespace ctr

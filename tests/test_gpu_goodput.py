@@ -210,3 +210,33 @@ def test_p99_tpot_adversarial(orc, case):
         assert tpot[r] == orc.p99_tpot({"true_out": o[r]}, tf[r], td[r]), (case, r)
     if case in ("one_token", "empty"):
         assert tpot.tolist() == [-1, -1, -1]
+
+
+@pytest.mark.parametrize("N", [1, 3, 127, 1023, 1024, 1025, 2047, 4096, 4101, 9001, 140_002])
+@pytest.mark.parametrize("shape", ["spread", "rising", "falling", "burst", "equal", "two_values", "heavy_tail"])
+def test_p99_threshold_from_the_sample(orc, N, shape):
+    """Rows around the sample's size, aligned and not, whose largest hundredth the sample sees (spread), sees at one end
+    only (rising, falling), misses (one burst between two of its groups) or cannot split (equal values)."""
+    ctr = need_gpu()
+    rng = np.random.default_rng(N)
+    R = 3
+    base = {"spread": rng.integers(1, 10**7, (R, N)), "rising": np.arange(1, N + 1) * 997 + rng.integers(0, 50, (R, N)),
+            "falling": np.arange(N, 0, -1) * 997 + rng.integers(0, 50, (R, N)),
+            "burst": rng.integers(1, 1000, (R, N)), "equal": np.full((R, N), 12_345),
+            "two_values": rng.choice([7, 10**6], (R, N), p=[0.985, 0.015]),
+            "heavy_tail": np.floor(np.exp(rng.standard_normal((R, N)) * 3 + 8)).astype(np.int64) + 1}[shape].astype(np.int64)
+    if shape == "burst":
+        base[:, N // 3:N // 3 + N // 50 + 1] += 10**8
+    o = rng.integers(1, 400, (R, N))
+    arr = np.sort(rng.integers(0, 10**9, (R, N)), axis=1)
+    tf = arr + base
+    td = tf + rng.permutation(base.T).T * np.maximum(o - 1, 0) % (1 << 31) + rng.integers(0, 3, (R, N))
+    trh = {"arrival_us": arr, "prompt_len": np.ones((R, N)), "true_out": o, "pred_out": np.ones((R, N)),
+           "slo_class": rng.integers(0, 2, (R, N))}
+    tr, tfd, tdd = to_dev(trh), torch.from_numpy(tf).cuda(), torch.from_numpy(td).cuda()
+    met, p99 = _goodput(ctr, W.SimCfg(), tr, R, 1, N, tfd, tdd)
+    tpot = _p99_tpot(ctr, W.SimCfg(), tr, R, 1, N, tfd, tdd)
+    for r in range(R):
+        row = {k: v[r] for k, v in trh.items()}
+        assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), row, tf[r], td[r]), r
+        assert tpot[r] == orc.p99_tpot({"true_out": o[r]}, tf[r], td[r]), r
