@@ -45,6 +45,10 @@ constexpr uint64_t kEmpty = ~0ull;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarpsPerBlock = 4;
 constexpr int64_t kNever = INT64_MAX;
+// an empty pending heap's top as a time: later than any event (the last one of a row that has not failed starts a step
+// before 2^40, and a step lasts less than 2^38)
+constexpr int64_t kIdle = (int64_t)(kEmpty >> kKeyBits);
+constexpr int64_t kDrain = kIdle - 1;  // every event is at or before this
 constexpr int64_t kBacklogClamp = int64_t(1) << 40;
 constexpr uint64_t kPressureClamp = uint64_t(1) << 18;
 constexpr int kRecipN = 1024;  // batch sizes with a tabulated reciprocal
@@ -83,7 +87,12 @@ __device__ __forceinline__ uint64_t div_recip(uint64_t num, uint64_t d, uint64_t
 // An estimate of x / d for 0 <= x < 2^31 and 1 <= d < 2^31 whose quotient is
 // below 2^20, inv being recip_estimate(d): x and d rounded to fp32, a reciprocal
 // good to a few 2^-24 and a product, so it is off by less than one unit either way.
-__device__ __forceinline__ float recip_estimate(int32_t d) { return __fdividef(1.0f, __int2float_rn(d)); }
+__device__ __forceinline__ float recip_estimate(int32_t d)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__int2float_rn(d)));  // within 1 ulp
+    return r;
+}
 __device__ __forceinline__ int32_t div_estimate(int32_t x, float inv)
 {
     return __float2int_rz(__int2float_rn(x) * inv);
@@ -340,7 +349,7 @@ struct RowView {
 // they are until the event: the running step ends at step_end, `run` more of
 // `step` us follow, and the event is at step_end + run * step.  An idle lane
 // (n_act = 0) has run = 0 and step_end the time of its next KV-ready request
-// (kNever without one).  run * step stays below 2^31, so a time inside the run
+// (kIdle without one).  run * step stays below 2^31, so a time inside the run
 // is a 32-bit offset from step_end.  step_idx, kv_res and a true-backlog sum
 // are the values before the step that ends at step_end.
 // `sum` is the one in-flight sum the row's policy reads: the true remaining
@@ -354,8 +363,16 @@ struct Decode {
     int32_t step_idx;        // steps ended; the step budget keeps it and every completion step below 2^31
     int32_t kv_res, kv_rsv;  // resident <= reserved <= C < 2^31 tokens
     uint64_t pend_top, act_top;
-    int32_t n_act, q, pend_n, w_head, w_n;  // n_act is also the active heap's size
+    int32_t n_act, pend_n, w_head, w_n;  // n_act is also the active heap's size
+    int32_t q;  // batched prefill: requests routed here and not completed (else the sum of the three counts, see in_flight)
 };
+
+// requests routed to a decode lane and not completed
+template <bool kBat>
+__device__ __forceinline__ int32_t in_flight(const Decode& s)
+{
+    return kBat ? s.q : s.n_act + s.pend_n + s.w_n;
+}
 
 __device__ __forceinline__ int64_t next_event(const Decode& s) { return s.step_end + (int64_t)s.run * s.step; }
 
@@ -405,7 +422,8 @@ template <int kArity>
 __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, const SimParams& P, uint64_t* pend,
                                            uint32_t* wait, bool& bad)
 {
-    while (s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= t) {
+    const uint64_t by = (uint64_t)(t + 1) << kKeyBits;  // keys of requests KV-ready by t are below (kEmpty is not)
+    while (s.pend_top < by) {
         const uint32_t k = (uint32_t)(s.pend_top & kKeyMask);
         hpop<kArity>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
         if (--room < 0) return CTR_EOVERFLOW;
@@ -429,7 +447,7 @@ template <int kArity, bool kPtr>
 __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimParams& P, uint64_t* pend, uint64_t* act,
                                             uint32_t* wait, const RowView<kPtr>& V, bool sum_is_o_hat, bool& bad)
 {
-    if (tev >= kTimeLimit) return CTR_EOVERFLOW;
+    if ((int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32)) return CTR_EOVERFLOW;  // the limit's low word is 0
     if (s.n_act > 0) {  // (1) run + 1 steps end: as many tokens for every active request
         const int32_t ends = s.run + 1;
         const int32_t tokens = ends * s.n_act;  // within the reservation
@@ -442,7 +460,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
             if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
             V.set_done(k, tev, bad);
             hpop<kArity>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
-            s.q -= 1;
+            if constexpr (kArity == 2) s.q -= 1;
             s.kv_res -= pk + ok;
             s.kv_rsv -= pk + ok;
         }
@@ -450,12 +468,13 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     // (2) admission in FCFS order: the waiting FIFO, then the requests KV-ready by now in (time, index)
     // order, which join the FIFO once its head does not fit.  Before any admission the FIFO holds all of
     // them, so its room counts those admitted from the pending heap too.
+    const uint64_t by = (uint64_t)(tev + 1) << kKeyBits;  // as in flush_ready
     int32_t room = P.cap_wait - s.w_n;
     int32_t admitted = 0;
     uint32_t last = 0;  // the request admitted last; the others are chained through their t_first entries
     for (;;) {
         const bool fifo = s.w_n > 0;
-        if (!fifo && !(s.pend_n > 0 && (int64_t)(s.pend_top >> kKeyBits) <= tev)) break;
+        if (!fifo && s.pend_top >= by) break;
         const uint32_t k = fifo ? ck_ld(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
         const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
         if ((uint32_t)s.kv_rsv + (uint32_t)(pk + ok) > (uint32_t)P.kv_cap) {  // < 2^31 + 2^21
@@ -481,15 +500,16 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     }
     // (3) the next step and the next event
     if (s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
-    const int64_t tp = s.pend_n > 0 ? (int64_t)(s.pend_top >> kKeyBits) : kNever;
+    const int64_t tp = (int64_t)(s.pend_top >> kKeyBits);  // kIdle when empty
     if (s.n_act == 0) {
         s.step_end = tp;
         s.run = 0;
         return CTR_OK;
     }
     const int32_t n = s.n_act;
-    const int64_t fixed = P.dec_base + (int64_t)(int32_t)P.dec_seq * n;
-    s.step_end = tev + fixed + kv_term(s.kv_res, P);
+    // dec_base <= 2^24 and a KV term below 2^31 add up in 32 bits
+    s.step_end = tev + (int64_t)((uint64_t)(uint32_t)P.dec_seq * (uint32_t)n) +
+                 (int64_t)(uint64_t)((uint32_t)P.dec_base + (uint32_t)kv_term(s.kv_res, P));
     for (; admitted > 0; --admitted) {  // first token at the end of this step
         const int64_t prev = admitted > 1 ? V.first(last, bad) : 0;
         V.set_first(last, s.step_end, bad);
@@ -504,10 +524,10 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         m = __float2int_rz(__fdividef(__uint2float_rn(room1), __int2float_rn(n)));
         m -= (uint64_t)(uint32_t)m * (uint32_t)n > room1;
     }
-    s.step = (int32_t)fixed + q1;  // run_max = 0 where a step could reach 2^31 us
+    s.step = (int32_t)P.dec_base + (int32_t)P.dec_seq * n + q1;  // run_max = 0 where a step could reach 2^31 us
     s.inv_step = recip_estimate(s.step);
     s.run = m < P.run_max ? m : P.run_max;
-    if (s.w_n == 0 && s.pend_n > 0) cut_run(s, tp);
+    if (s.w_n == 0) cut_run(s, tp);
     return CTR_OK;
 }
 
@@ -575,7 +595,8 @@ __device__ __forceinline__ uint64_t instance_cost(const SimParams& P, const Cons
 {
     if (pol != CTR_POLICY_LEARNED && pol != CTR_POLICY_LEARNED_P2) {
         if (is_pre) return (uint64_t)s.w_n;
-        return pol == CTR_POLICY_LENGTH_HEURISTIC && (int32_t)rq.o_hat >= P.heur_thresh ? (uint64_t)s.sum : (uint64_t)s.q;
+        return pol == CTR_POLICY_LENGTH_HEURISTIC && (int32_t)rq.o_hat >= P.heur_thresh ? (uint64_t)s.sum
+                                                                                        : (uint64_t)in_flight<kBat>(s);
     }
     // backlog and own work of the instance, then the cost both kinds share
     // (feature ablation, sec. V-F, is in the constants: see ConstsDev)
@@ -626,7 +647,7 @@ __device__ __forceinline__ uint64_t instance_cost(const SimParams& P, const Cons
         work = own + ((((own * p18) >> 16) * cc.rho) >> 8);
     }
     if (b > (uint64_t)kBacklogClamp) b = (uint64_t)kBacklogClamp;
-    const uint32_t queue = (uint32_t)(is_pre ? s.w_n : s.q);
+    const uint32_t queue = (uint32_t)(is_pre ? s.w_n : in_flight<kBat>(s));
     const uint64_t cost = (b * cc.w_b + work * cc.w_s) * cc.sigma[rq.cls] + cc.w_q16 * queue;
     if (pol == CTR_POLICY_LEARNED_P2) {
         // power of two choices: only two sampled candidates per pool are priced
@@ -677,14 +698,16 @@ __device__ __forceinline__ int queue_decode(Decode& s, int64_t T, int64_t k, int
 {
     // requests routed here whose KV is not ready yet, exactly: first move
     // those already ready (kept in the heap until the step end) if it matters
-    if (s.q - s.w_n - s.n_act >= P.cap_pend) {
+    constexpr bool kBat = kArity == 2;
+    if (in_flight<kBat>(s) - s.w_n - s.n_act >= P.cap_pend) {
         const int rc = flush_ready<kArity>(s, T, P.cap_wait - s.w_n, P, pend, wait, bad);
         if (rc != CTR_OK) return rc;
+        if (in_flight<kBat>(s) - s.w_n - s.n_act == P.cap_pend) return CTR_EOVERFLOW;
     }
-    if (s.q - s.w_n - s.n_act == P.cap_pend || (ready >= 0 && s.pend_n == P.cap_pend_store)) return CTR_EOVERFLOW;
-    if (ready >= 0)
+    if (kBat && ready >= 0 && s.pend_n == P.cap_pend_store) return CTR_EOVERFLOW;
+    if (!kBat || ready >= 0)
         push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, heap_stride(P.cap_pr), bad);
-    s.q += 1;
+    if constexpr (kBat) s.q += 1;
     s.sum += weight;
     return CTR_OK;
 }
@@ -704,13 +727,11 @@ __device__ __forceinline__ bool request_valid(const SimParams& P, int64_t i, int
 // Every request of a replica (CTR_EINVAL before anything is simulated); one warp.
 __device__ __forceinline__ bool row_valid(const SimParams& P, int64_t tb, int lane, bool& bad)
 {
-    for (int64_t base = 0; base < P.n_req; base += 32) {
-        const int64_t k = base + lane;
-        bool ok = true;
-        if (k < P.n_req) ok = request_valid(P, tb + k, k > 0 ? ck_ld(P.trace.arrival_us, tb + k - 1, P.trace_len, bad) : 0, bad);
-        if (__any_sync(kFull, !ok)) return false;
-    }
-    return true;
+    bool ok = true;
+#pragma unroll 4
+    for (int64_t k = lane; k < P.n_req; k += 32)
+        ok = request_valid(P, tb + k, k > 0 ? ck_ld(P.trace.arrival_us, tb + k - 1, P.trace_len, bad) : 0, bad) && ok;
+    return __all_sync(kFull, ok);
 }
 
 // argmin of 64-bit values within aligned groups of G lanes (ties -> lowest lane),
@@ -798,18 +819,23 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         // per-request bounds, one row at a time with the whole warp
         bool oob = false;  // bounds-checked builds: an index of this lane fell outside its buffer
         bool valid = false;
+        int64_t checked = -1;
+        bool ok = false, oob_g = false;
         for (int g = 0; g < kRowsPerWarp; ++g) {
             const int64_t r = base_row + g;
             if (r >= P.n_rows) break;
-            bool oob_g = false;
-            const bool ok = row_valid(P, (r / per_rep) * n, lane, oob_g);
+            if (r / per_rep != checked) {  // the warp's rows are mostly one replica's
+                checked = r / per_rep;
+                oob_g = false;
+                ok = row_valid(P, checked * n, lane, oob_g);
+            }
             if (g == grp) oob = oob_g;
             if (g == grp) valid = ok;
         }
         bool live = has_row && valid;
 
         Decode s;
-        s.step_end = is_dec ? kNever : 0; s.run = 0; s.step = 1; s.inv_step = 1.0f;
+        s.step_end = is_dec ? kIdle : 0; s.run = 0; s.step = 1; s.inv_step = 1.0f;
         s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
         s.pend_top = kEmpty; s.act_top = kEmpty;
         s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
@@ -995,7 +1021,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                     err = ready >= kTimeLimit ? CTR_EOVERFLOW : push_prefill<kSig>(s, end, (uint32_t)pk, P, ring, oob);
                 }
                 ready = __shfl_sync(kFull, ready, ip, G);
-                if (live && gl == P.n_pre + id && ready < kTimeLimit)
+                if (live && gl == P.n_pre + id && ready < kTimeLimit && err == CTR_OK)
                     err = queue_decode<kArity>(s, T, k, ready, sum_is_o_hat ? ohk : ok, P, pend, wait, oob);
                 if (gl == j) my_route = ((uint32_t)ip << 8) | (uint32_t)id;
                 if (__ballot_sync(kFull, err != CTR_OK) & gmask) live = false;
@@ -1011,12 +1037,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         // drain: every remaining batch, then every remaining event
         if constexpr (kBat) {
             if (batched) {
-                prefill_batches(kNever - 1);
+                prefill_batches(kDrain);
                 if (__ballot_sync(kFull, err != CTR_OK) & gmask) live = false;
             }
         }
         if (live && is_dec) {
-            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat,
+            err = decode_advance<false, kArity>(s, kDrain, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat,
                                                 oob);
         }
 
@@ -1084,7 +1110,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
         const bool valid = !__syncthreads_or(bad);
 
         Decode s;
-        s.step_end = is_pre ? 0 : kNever; s.run = 0; s.step = 1; s.inv_step = 1.0f;
+        s.step_end = is_pre ? 0 : kIdle; s.run = 0; s.step = 1; s.inv_step = 1.0f;
         s.step_idx = 0; s.kv_res = 0; s.kv_rsv = 0; s.sum = 0;
         s.pend_top = kEmpty; s.act_top = kEmpty;
         s.n_act = 0; s.q = 0; s.pend_n = 0; s.w_head = 0; s.w_n = 0;
@@ -1173,7 +1199,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
             }
         }
         if (go && !is_pre && err == CTR_OK)  // drain: every remaining event
-            err = decode_advance<false, kArity>(s, kNever - 1, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat, oob);
+            err = decode_advance<false, kArity>(s, kDrain, P, pend, act, wait, V, -1, kv_seen, sum_is_o_hat, oob);
 
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) h += __shfl_xor_sync(kFull, h, off);
