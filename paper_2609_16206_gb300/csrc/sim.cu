@@ -393,10 +393,9 @@ __device__ __forceinline__ int32_t ends_by(const Decode& s, int64_t t)
 // at which nothing changes).
 __device__ __forceinline__ void cut_run(Decode& s, int64_t tp)
 {
-    if (tp <= s.step_end) {
-        s.run = 0;
-    } else if (tp < next_event(s)) {
-        const int32_t rel = (int32_t)(tp - s.step_end);
+    const int64_t d = tp - s.step_end;
+    if (d < (int64_t)s.run * s.step) {
+        const int32_t rel = d > 0 ? (int32_t)d : 0;
         int32_t q = div_estimate(rel, s.inv_step);
         q += rel > q * s.step;
         s.run = q;
@@ -447,23 +446,22 @@ template <int kArity, bool kPtr>
 __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimParams& P, uint64_t* pend, uint64_t* act,
                                             uint32_t* wait, const RowView<kPtr>& V, bool sum_is_o_hat, bool& bad)
 {
-    if ((int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32)) return CTR_EOVERFLOW;  // the limit's low word is 0
-    if (s.n_act > 0) {  // (1) run + 1 steps end: as many tokens for every active request
-        const int32_t ends = s.run + 1;
+    {  // (1) run + 1 steps end (none of an idle instance): as many tokens for every active request
+        const int32_t ends = s.n_act > 0 ? s.run + 1 : 0;
         const int32_t tokens = ends * s.n_act;  // within the reservation
         s.step_idx += ends;
         s.kv_res += tokens;
         if (!sum_is_o_hat) s.sum -= tokens;
-        while ((int32_t)(s.act_top >> kKeyBits) == s.step_idx) {  // never with an empty heap: its top is all ones
-            const uint32_t k = (uint32_t)(s.act_top & kKeyMask);
-            const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
-            if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
-            V.set_done(k, tev, bad);
-            hpop<kArity>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
-            if constexpr (kArity == 2) s.q -= 1;
-            s.kv_res -= pk + ok;
-            s.kv_rsv -= pk + ok;
-        }
+    }
+    while ((int32_t)(s.act_top >> kKeyBits) == s.step_idx) {  // never with an empty heap: its top is all ones
+        const uint32_t k = (uint32_t)(s.act_top & kKeyMask);
+        const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
+        if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
+        V.set_done(k, tev, bad);
+        hpop<kArity>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
+        if constexpr (kArity == 2) s.q -= 1;
+        s.kv_res -= pk + ok;
+        s.kv_rsv -= pk + ok;
     }
     // (2) admission in FCFS order: the waiting FIFO, then the requests KV-ready by now in (time, index)
     // order, which join the FIFO once its head does not fit.  Before any admission the FIFO holds all of
@@ -477,18 +475,19 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         if (!fifo && s.pend_top >= by) break;
         const uint32_t k = fifo ? ck_ld(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
         const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
-        if ((uint32_t)s.kv_rsv + (uint32_t)(pk + ok) > (uint32_t)P.kv_cap) {  // < 2^31 + 2^21
+        const bool fits = (uint32_t)s.kv_rsv + (uint32_t)(pk + ok) <= (uint32_t)P.kv_cap;  // < 2^31 + 2^21
+        if (!fits || s.n_act == P.cap_act) {
+            if (fits) return CTR_EOVERFLOW;
             const int rc = flush_ready<kArity>(s, tev, room, P, pend, wait, bad);
             if (rc != CTR_OK) return rc;
             break;
         }
-        if (s.n_act == P.cap_act) return CTR_EOVERFLOW;
         if (fifo) {
             s.w_n -= 1;
             s.w_head = s.w_n == 0 || s.w_head + 1 == P.cap_wait ? 0 : s.w_head + 1;  // an empty ring restarts at 0
         } else {
             hpop<kArity>(pend, s.pend_n, s.pend_top, heap_stride(P.cap_pr), bad);
-            if (--room < 0) return CTR_EOVERFLOW;
+            --room;
         }
         s.kv_rsv += pk + ok;
         s.kv_res += pk;
@@ -499,7 +498,10 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         admitted += 1;
     }
     // (3) the next step and the next event
-    if (s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps) return CTR_ETIMEOUT;  // steps started on this instance
+    // the FIFO's room, the steps started on this instance, the time (its limit's low word is 0)
+    if (room < 0 || s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps ||
+        (int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32))
+        return s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps ? CTR_ETIMEOUT : CTR_EOVERFLOW;
     const int64_t tp = (int64_t)(s.pend_top >> kKeyBits);  // kIdle when empty
     if (s.n_act == 0) {
         s.step_end = tp;
@@ -520,10 +522,10 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     const int32_t q1 = kv_term(s.kv_res + n, P);
     const uint32_t room1 = (uint32_t)(q1 + 1) * (uint32_t)P.kv_div - 1u - (uint32_t)s.kv_res;
     int32_t m = (int32_t)(s.act_top >> kKeyBits) - s.step_idx - 1;  // plain ends before the next completion, <= 2^20
-    if ((uint64_t)(uint32_t)m * (uint32_t)n > room1) {  // the term changes first: at most room1 / n (one less is fine)
-        m = __float2int_rz(__fdividef(__uint2float_rn(room1), __int2float_rn(n)));
-        m -= (uint64_t)(uint32_t)m * (uint32_t)n > room1;
-    }
+    // the steps before the term changes, room1 / n (or one less): the estimate is within one where it is below m
+    int32_t before = __float2int_rz(__uint2float_rn(room1) * recip_estimate(n));
+    before -= (uint32_t)before * (uint32_t)n > room1;  // room1 < kv_div + n, so a product that matters fits
+    m = before < m ? before : m;
     s.step = (int32_t)P.dec_base + (int32_t)P.dec_seq * n + q1;  // run_max = 0 where a step could reach 2^31 us
     s.inv_step = recip_estimate(s.step);
     s.run = m < P.run_max ? m : P.run_max;
