@@ -391,10 +391,10 @@ __device__ __forceinline__ int32_t ends_by(const Decode& s, int64_t t)
 // A request becomes KV-ready at tp: the event moves up to the first step end at
 // or after tp (or, where the estimate is one low, to the end before it, an event
 // at which nothing changes).
-__device__ __forceinline__ void cut_run(Decode& s, int64_t tp)
+__device__ __forceinline__ void cut_run(Decode& s, int64_t tp, bool when)
 {
     const int64_t d = tp - s.step_end;
-    if (d < (int64_t)s.run * s.step) {
+    if (when & (d < (int64_t)s.run * s.step)) {
         const int32_t rel = d > 0 ? (int32_t)d : 0;
         int32_t q = div_estimate(rel, s.inv_step);
         q += rel > q * s.step;
@@ -409,10 +409,9 @@ template <int kArity>
 __device__ __forceinline__ void push_pending(Decode& s, uint64_t* pend, uint64_t key, int64_t lim, bool& bad)
 {
     hpush<kArity>(pend, s.pend_n, s.pend_top, key, lim, bad);
-    if (s.n_act == 0)
-        s.step_end = (int64_t)(s.pend_top >> kKeyBits);
-    else if (s.w_n == 0)
-        cut_run(s, (int64_t)(key >> kKeyBits));
+    const int64_t tp = (int64_t)(key >> kKeyBits);
+    s.step_end = (s.n_act == 0) & (tp < s.step_end) ? tp : s.step_end;  // an idle instance's next event
+    cut_run(s, tp, s.w_n == 0);
 }
 
 // Move every pending request whose KV is ready by t into the waiting FIFO, in
@@ -503,15 +502,12 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         (int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32))
         return s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps ? CTR_ETIMEOUT : CTR_EOVERFLOW;
     const int64_t tp = (int64_t)(s.pend_top >> kKeyBits);  // kIdle when empty
-    if (s.n_act == 0) {
-        s.step_end = tp;
-        s.run = 0;
-        return CTR_OK;
-    }
     const int32_t n = s.n_act;
+    const bool idle = n == 0;  // then what follows computes nothing that is kept
     // dec_base <= 2^24 and a KV term below 2^31 add up in 32 bits
-    s.step_end = tev + (int64_t)((uint64_t)(uint32_t)P.dec_seq * (uint32_t)n) +
-                 (int64_t)(uint64_t)((uint32_t)P.dec_base + (uint32_t)kv_term(s.kv_res, P));
+    const int64_t end = tev + (int64_t)((uint64_t)(uint32_t)P.dec_seq * (uint32_t)n) +
+                        (int64_t)(uint64_t)((uint32_t)P.dec_base + (uint32_t)kv_term(s.kv_res, P));
+    s.step_end = idle ? tp : end;
     for (; admitted > 0; --admitted) {  // first token at the end of this step
         const int64_t prev = admitted > 1 ? V.first(last, bad) : 0;
         V.set_first(last, s.step_end, bad);
@@ -528,8 +524,8 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     m = before < m ? before : m;
     s.step = (int32_t)P.dec_base + (int32_t)P.dec_seq * n + q1;  // run_max = 0 where a step could reach 2^31 us
     s.inv_step = recip_estimate(s.step);
-    s.run = m < P.run_max ? m : P.run_max;
-    if (s.w_n == 0) cut_run(s, tp);
+    s.run = idle ? 0 : m < P.run_max ? m : P.run_max;
+    cut_run(s, tp, s.w_n == 0);
     return CTR_OK;
 }
 
