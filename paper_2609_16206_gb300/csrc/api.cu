@@ -117,7 +117,6 @@ int ctr_gen_trace(const ctr_trace_cfg* cfg, int32_t n_replicas, int64_t replica_
     p.seed = cfg->seed;
     p.n_seeds = cfg->n_seeds;
     p.arrival_kind = cfg->arrival_kind;
-    p.n_classes = cfg->n_classes;
     p.rate[0] = cfg->rate_mreq[0];
     p.rate[1] = cfg->rate_mreq[1];
     p.rate_recip[0] = ~0ull / (uint64_t)cfg->rate_mreq[0];
@@ -132,14 +131,15 @@ int ctr_gen_trace(const ctr_trace_cfg* cfg, int32_t n_replicas, int64_t replica_
     p.long_mu = (float)cfg->long_mu;
     p.long_sigma = (float)cfg->long_sigma;
     p.noise_sigma = (float)cfg->noise_sigma;
-    p.prompt_min = cfg->prompt_min;
-    p.prompt_max = cfg->prompt_max;
-    p.out_min = cfg->out_min;
-    p.out_max = cfg->out_max;
-    p.pred_min = cfg->pred_min;
-    p.pred_max = cfg->pred_max;
+    p.prompt = {cfg->prompt_min, cfg->prompt_max, (float)cfg->prompt_max};
+    p.outlen = {cfg->out_min, cfg->out_max, (float)cfg->out_max};
+    p.pred = {cfg->pred_min, cfg->pred_max, (float)cfg->pred_max};
     p.mix_short_thr = cfg->mix_short_thr;
-    for (int i = 0; i < 3; ++i) p.class_thr[i] = cfg->class_thr[i];
+    for (int i = 0; i < 3; ++i) {
+        const bool used = i < cfg->n_classes - 1;
+        p.class_base += used && cfg->class_thr[i] == 0;
+        p.class_below[i] = used && cfg->class_thr[i] > 0 ? (uint32_t)(cfg->class_thr[i] - 1) : ~0u;
+    }
     p.n_replicas = n_replicas;
     p.replica_offset = replica_offset;
     p.n_req = n_req;

@@ -94,8 +94,9 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
 {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+        const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
+        const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
         const uint32_t n0 = hi1 ^ c1 ^ k0, n2 = hi0 ^ c3 ^ k1;
         c0 = n0;
         c1 = lo1;
@@ -112,15 +113,20 @@ struct TraceParams {
     uint64_t seed;
     int64_t n_seeds;
     int32_t arrival_kind;
-    int32_t n_classes;
     int64_t rate[2];
     uint64_t rate_recip[2];     // floor((2^64 - 1) / rate)
     int64_t dwell_mean_us;
     float dwell_mean_f;         // dwell_mean_us rounded once to fp32
     float prompt_mu, prompt_sigma, short_mu, short_sigma, long_mu, long_sigma, noise_sigma;
-    int64_t prompt_min, prompt_max, out_min, out_max, pred_min, pred_max;
+    struct Clip {
+        int32_t lo, hi;
+        float hi_f;
+    } prompt, outlen, pred;     // length ranges
     uint64_t mix_short_thr;
-    uint64_t class_thr[3];
+    // classes by 32-bit words: class_base leading thresholds are 0, class_below[i] is a further one less 1
+    // (all ones past the last, which no word exceeds)
+    int32_t class_base;
+    uint32_t class_below[3];
     int64_t n_replicas, replica_offset, n_req;
     ctr_requests out;
     uint64_t minus_zeros;       // two fp32 -0 (see mul2 in trace.cu)

@@ -91,25 +91,6 @@ __device__ float det_logf(float x)
     return add(mul(ed, 0x1.62e4p-1f), add(mul(ed, 0x1.7f7d1cp-20f), ln_m));
 }
 
-// exp: k = nearest integer to x / ln2 (halves away from zero),
-// r = (x - k ln2_hi) - k ln2_lo, e^r by its degree-7 Taylor polynomial, times
-// 2^k through the exponent field.  x is clamped to [-87, 88].
-__device__ float det_expf(float x)
-{
-    const float inv_fact[8] = {0x1p+0f, 0x1p+0f, 0x1p-1f, 0x1.555556p-3f, 0x1.555556p-5f, 0x1.111112p-7f,
-                               0x1.6c16c2p-10f, 0x1.a01a02p-13f};
-    if (x > 88.0f) x = 88.0f;
-    if (x < -87.0f) x = -87.0f;
-    const float kf = mul(x, 0x1.715476p+0f);
-    const int k = __float2int_rz(kf >= 0.0f ? add(kf, 0.5f) : sub(kf, 0.5f));
-    const float kd = __int2float_rn(k);
-    const float r = sub(sub(x, mul(kd, 0x1.62e4p-1f)), mul(kd, 0x1.7f7d1cp-20f));
-    float acc = inv_fact[7];
-#pragma unroll
-    for (int i = 6; i >= 0; --i) acc = add(mul(acc, r), inv_fact[i]);
-    return mul(acc, __uint_as_float((uint32_t)(k + 127) << 23));
-}
-
 // Two fp32 operations in one instruction, each rounded to nearest on its own.
 struct F2 {
     uint64_t v;
@@ -137,6 +118,48 @@ __device__ __forceinline__ F2 mul2(F2 a, F2 b, uint64_t minus_zeros)
     return r;
 }
 
+// exp: k = nearest integer to x / ln2 (halves away from zero),
+// r = (x - k ln2_hi) - k ln2_lo, e^r by its degree-7 Taylor polynomial, times
+// 2^k through the exponent field.  x is clamped to [-87, 88].
+__device__ float det_expf(float x)
+{
+    const float inv_fact[8] = {0x1p+0f, 0x1p+0f, 0x1p-1f, 0x1.555556p-3f, 0x1.555556p-5f, 0x1.111112p-7f,
+                               0x1.6c16c2p-10f, 0x1.a01a02p-13f};
+    if (x > 88.0f) x = 88.0f;
+    if (x < -87.0f) x = -87.0f;
+    const float kf = mul(x, 0x1.715476p+0f);
+    const int k = __float2int_rz(kf >= 0.0f ? add(kf, 0.5f) : sub(kf, 0.5f));
+    const float kd = __int2float_rn(k);
+    const float r = sub(sub(x, mul(kd, 0x1.62e4p-1f)), mul(kd, 0x1.7f7d1cp-20f));
+    float acc = inv_fact[7];
+#pragma unroll
+    for (int i = 6; i >= 0; --i) acc = add(mul(acc, r), inv_fact[i]);
+    return mul(acc, __uint_as_float((uint32_t)(k + 127) << 23));
+}
+
+// exp of two values, operation by operation the same (k ln2 is negated to subtract it by an addition)
+__device__ __forceinline__ void det_expf2(float x0, float x1, uint64_t mz, float& e0, float& e1)
+{
+    const float inv_fact[8] = {0x1p+0f, 0x1p+0f, 0x1p-1f, 0x1.555556p-3f, 0x1.555556p-5f, 0x1.111112p-7f,
+                               0x1.6c16c2p-10f, 0x1.a01a02p-13f};
+    if (x0 > 88.0f) x0 = 88.0f;
+    if (x0 < -87.0f) x0 = -87.0f;
+    if (x1 > 88.0f) x1 = 88.0f;
+    if (x1 < -87.0f) x1 = -87.0f;
+    const F2 x = pack(x0, x1);
+    float f0, f1;
+    unpack(mul2(x, pack(0x1.715476p+0f, 0x1.715476p+0f), mz), f0, f1);
+    const int k0 = __float2int_rz(add(f0, copysignf(0.5f, f0))), k1 = __float2int_rz(add(f1, copysignf(0.5f, f1)));
+    const F2 kd = pack(__int2float_rn(k0), __int2float_rn(k1));
+    const F2 r = add2(add2(x, mul2(kd, pack(-0x1.62e4p-1f, -0x1.62e4p-1f), mz)),
+                      mul2(kd, pack(-0x1.7f7d1cp-20f, -0x1.7f7d1cp-20f), mz));
+    F2 acc = pack(inv_fact[7], inv_fact[7]);
+#pragma unroll
+    for (int i = 6; i >= 0; --i) acc = add2(mul2(acc, r, mz), pack(inv_fact[i], inv_fact[i]));
+    unpack(mul2(acc, pack(__uint_as_float((uint32_t)(k0 + 127) << 23), __uint_as_float((uint32_t)(k1 + 127) << 23)), mz), e0,
+           e1);
+}
+
 // Wichura (1988), algorithm AS241 PPND16 in fp32: rational approximations of
 // degree 7 in r = 0.180625 - q^2 (|q| <= 0.425, q = U - 1/2) or in
 // r = sqrt(-ln min(U, 1 - U)) shifted by 1.6 (r <= 5) or by 5.  The numerator
@@ -162,15 +185,32 @@ __device__ __forceinline__ float centred(uint32_t u)
 
 constexpr float kCentre = 0x1.b33334p-2f;  // |q| up to here: the central approximation
 
-__device__ __forceinline__ float ndtri_centre(float q, uint64_t mz)
+// the central approximation of three words, side by side so that each coefficient pair is fetched once
+__device__ __forceinline__ void ndtri_centre3(const float (&q)[3], uint64_t mz, float (&z)[3])
 {
     const float a[8] = {0x1.b18d92p+1f, 0x1.0a4888p+7f, 0x1.ece5d2p+10f, 0x1.ad1d8cp+13f,
                         0x1.66c3e8p+15f, 0x1.06c1c6p+16f, 0x1.052d26p+15f, 0x1.39a296p+11f};
     const float b[8] = {0x1p+0f, 0x1.5281b4p+5f, 0x1.5797fp+9f, 0x1.512322p+12f,
                         0x1.4b772ep+14f, 0x1.3317cap+15f, 0x1.c0e458p+14f, 0x1.46a7ecp+12f};
-    float n, d;
-    ratio7(a, b, sub(0x1.71eb86p-3f, mul(q, q)), mz, n, d);
-    return dvd(mul(q, n), d);
+    F2 rr[3], acc[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float r = sub(0x1.71eb86p-3f, mul(q[i], q[i]));
+        rr[i] = pack(r, r);
+        acc[i] = pack(a[7], b[7]);
+    }
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        const F2 c = pack(a[j], b[j]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) acc[i] = add2(mul2(acc[i], rr[i], mz), c);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float n, d;
+        unpack(acc[i], n, d);
+        z[i] = dvd(mul(q[i], n), d);
+    }
 }
 
 __device__ float ndtri_tail(uint32_t u, uint64_t mz)
@@ -206,17 +246,18 @@ __device__ __forceinline__ void ndtri3(const uint32_t (&u)[3], float (&z)[3], ui
     uint32_t m[3], pos[3];
     uint32_t total = 0;
     const uint32_t below = (1u << lane) - 1u;
+    float c[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const float c = centred(u[i]);
-        const bool tail = fabsf(c) > kCentre;
-        z[i] = ndtri_centre(c, mz);
+        c[i] = centred(u[i]);
+        const bool tail = fabsf(c[i]) > kCentre;
         const uint32_t b = __ballot_sync(0xffffffffu, tail);
         pos[i] = total + __popc(b & below);
         total += __popc(b);
-        m[i] = (b >> lane) & 1u;
+        m[i] = tail;
         if (m[i]) q[pos[i]] = u[i];
     }
+    ndtri_centre3(c, mz, z);
     __syncwarp();
     for (uint32_t i = lane; i < total; i += 32) q[i] = __float_as_uint(ndtri_tail(q[i], mz));
     __syncwarp();
@@ -226,13 +267,12 @@ __device__ __forceinline__ void ndtri3(const uint32_t (&u)[3], float (&z)[3], ui
     __syncwarp();  // the queue is free for the next chunk
 }
 
-// clip(floor(v + 1/2), lo, hi) for v >= 0 (NaN / inf / huge -> hi); hi <= 2^20
-__device__ __forceinline__ int64_t round_clip(float v, int64_t lo, int64_t hi)
+// clip(floor(v + 1/2), lo, hi) for v >= 0 (NaN / inf / huge -> hi); hi <= 2^20, exact in fp32
+__device__ __forceinline__ int32_t round_clip(float v, const TraceParams::Clip& c)
 {
     const float y = add(v, 0.5f);
-    if (!(y < __int2float_rn((int)hi))) return hi;
-    const int64_t t = __float2int_rz(y);
-    return t < lo ? lo : t;
+    const int32_t t = __float2int_rz(y);
+    return !(y < c.hi_f) ? c.hi : t < c.lo ? c.lo : t;
 }
 
 // floor(num / d) for num >= 0 with recip = floor((2^64 - 1) / d): the estimate is low by at most 2
@@ -273,14 +313,15 @@ __device__ __forceinline__ int64_t request(const TraceParams& P, const Stream& S
     const bool is_short = (uint64_t)x.v[1] < P.mix_short_thr;
     const float mu = is_short ? P.short_mu : P.long_mu;
     const float sg = is_short ? P.short_sigma : P.long_sigma;
-    const int64_t p = round_clip(det_expf(add(P.prompt_mu, mul(P.prompt_sigma, z[0]))), P.prompt_min, P.prompt_max);
-    const int64_t o = round_clip(det_expf(add(mu, mul(sg, z[1]))), P.out_min, P.out_max);
-    const int64_t oh = round_clip(mul(__int2float_rn((int)o), det_expf(mul(P.noise_sigma, z[2]))), P.pred_min, P.pred_max);
-    int c = 0;
-    while (c < P.n_classes - 1 && (uint64_t)y.v[0] >= P.class_thr[c]) ++c;
-    P.out.prompt_len[row + k] = (int32_t)p;
-    P.out.true_out[row + k] = (int32_t)o;
-    P.out.pred_out[row + k] = (int32_t)oh;
+    float ep, eo;
+    det_expf2(add(P.prompt_mu, mul(P.prompt_sigma, z[0])), add(mu, mul(sg, z[1])), P.minus_zeros, ep, eo);
+    const int32_t p = round_clip(ep, P.prompt), o = round_clip(eo, P.outlen);
+    const int32_t oh = round_clip(mul(__int2float_rn(o), det_expf(mul(P.noise_sigma, z[2]))), P.pred);
+    // the cumulative thresholds at or below the word: those of 0 always are, t is at or below it when t - 1 is less
+    const int c = P.class_base + (y.v[0] > P.class_below[0]) + (y.v[0] > P.class_below[1]) + (y.v[0] > P.class_below[2]);
+    P.out.prompt_len[row + k] = p;
+    P.out.true_out[row + k] = o;
+    P.out.pred_out[row + k] = oh;
     P.out.slo_class[row + k] = (uint8_t)c;
     return trunc_pos(mul(-det_logf(u01(y.v[1])), 0x1.dcd65p+29f));
 }
@@ -356,8 +397,8 @@ struct Arrivals {
 };
 
 // One warp per replica.  Bound by instruction issue (Philox, the fp32 variates): 4,096 x 20,000 MMPP requests took
-// 2.95 ms with a tail path per variate, scalar polynomials and one dwell at a time, and take 2.43 ms; 21 B a
-// request are 0.7 TB/s of stores.  72 registers keep the 27 warps an SM of that size in one wave.
+// 2.95 ms (980 warp-instructions a chunk of 32) with a tail path per variate, scalar polynomials and one dwell at a
+// time, and take 2.26 ms (804, 0.68 of the issue slots); 21 B a request are 0.76 TB/s of stores.  72 registers keep the 27 warps an SM of that size in one wave.
 constexpr int kWalkWarps = 4;
 __global__ void __launch_bounds__(kWalkWarps * 32, 7) trace_kernel(const TraceParams P)
 {
