@@ -329,10 +329,10 @@ int ctr_simulate(const ctr_sim_cfg* cfg, const ctr_cost_consts* consts, int32_t 
     const bool goodput = met_count != nullptr;
     e = launch_sim(p, blocks, wpb, s);
     if (e != cudaSuccess) return cuda_status(e);
-    // Once the simulation has ended its per-warp structures are dead, so the slots hold, when they have
+    // Once the simulation has ended its per-warp structures are dead, so the workspace holds, when it has
     // room, the table of the checksum terms' request-only halves for the pass that follows.
     uint64_t* kmix = nullptr;
-    if (n_rows > 0 && n_req > 0 && slots * p.slot_bytes >= 16 * n_req) {
+    if (n_rows > 0 && n_req > 0 && (int64_t)(workspace_bytes - 256) >= 16 * n_req) {
         kmix = reinterpret_cast<uint64_t*>(p.ws);
         e = launch_mix_table(kmix, n_req, s);
         if (e != cudaSuccess) return cuda_status(e);

@@ -9,10 +9,11 @@
 // i < n_pre being prefill instance i and lane n_pre + d decode instance d, and
 // a warp carries 32 / G rows side by side (the policies of one replica, which
 // share arrival times).  Warps are persistent and pull row groups from an
-// atomic counter in the workspace.  For every arrival k:
-//   1. each decode lane advances its own instance's event loop to t_k
-//      (runs of plain steps in closed form, step ends, KV-ready requests,
-//      FCFS admissions, step starts); each prefill lane retires prefills that
+// atomic counter in the workspace.  (Launches of very few rows take a block per
+// row instead: sim_row_kernel.)  For every arrival k:
+//   1. each decode lane takes its own instance's events up to t_k (the step
+//      ends at which something changes, see Decode: completions, FCFS
+//      admissions, step starts); each prefill lane retires prefills that
 //      ended by t_k (or, with batched prefill, ends and starts its batches
 //      first and hands the members' KV-ready times to the decode lanes);
 //   2. every lane prices its instance for the row's policy, and two argmins
@@ -170,8 +171,8 @@ __device__ __forceinline__ void heap_pop(uint64_t* h, int32_t& n, uint64_t& top,
 // Binary 1-based variants (children 2i and 2i + 1 in one 16-byte word), kept
 // for batched prefill: its short-output document workload keeps decode batches
 // small, where the extra compares of a 4-ary level cost more than the saved
-// levels (4,096 x 10,000: 97.6 ms binary, 104.1 ms 4-ary; the replica sweep and
-// the large pool are 2 % and 6 % faster 4-ary).  Same region stride.
+// levels (4,096 x 2,000: 13.4 ms binary, 13.7 ms 4-ary; the replica sweep and
+// the large pool were 2 % and 6 % faster 4-ary).  Same region stride.
 __device__ __forceinline__ void heap_push_bin(uint64_t* h, int32_t& n, uint64_t& top, uint64_t key, int64_t lim,
                                               bool& bad)
 {
@@ -1068,9 +1069,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
 // both argmins itself; the ends of all prefill queues ride along in every warp
 // (lane i that of instance i), so the KV-ready time needs no second exchange and
 // a round-robin row needs no barrier at all.  Without batched prefill.
-// Bound by its longest chain an arrival: about 4,100 cycles for the learned
-// router, of them 2,500 one instance's event, 800 its price, 600 the commit
-// (cycle counters around each, 2P+6D).
+// Bound by its longest chain an arrival: about 3,600 cycles for the learned
+// router; of 4,100 on an earlier source 2,500 were one instance's event, 800 its
+// price and 600 the commit (cycle counters around each, 2P+6D).
 constexpr uint64_t kFailed = kEmpty - 1;  // in place of a cost: the row has failed
 template <int kMode, int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const __grid_constant__ SimParams P)
@@ -1270,11 +1271,12 @@ int sim_group_width(int n_instances)
 
 // Rows of a launch are spread over more warps, fewer to a warp, while that
 // leaves at most kSpreadWarps warps an SM: a warp of one row has fewer diverged
-// event sequences to serialise (2,000 requests on 2P+6D, four policies: 6.2 ms
-// a row alone, 7.7 ms two, 8.8 ms four to a warp), and as long as few warps share an SM
-// a launch lasts as long as one warp.  With more of them the issue slots run
-// out and packing wins: rows = 2,048 take 8.5 / 8.5 / 8.9 ms with 1 / 2 / 4 to a
-// warp, 3,072 take 10.1 / 9.3 / 10.2, 4,096 take 12.3 / 10.5 / 10.3.
+// event sequences to serialise, and as long as few warps share an SM a launch
+// lasts as long as one warp.  With more of them the issue slots run out and
+// packing wins.  1,500 requests on 2P+6D, four policies, with 1 / 2 / 4 rows to a
+// warp: 1,536 rows take 3.6 / 3.8 / 4.1 ms, 2,048 take 3.9 / 3.8 / 4.1, 3,072
+// take 5.0 / 4.3 / 4.7, 4,096 take 6.1 / 4.8 / 4.7; learned rows of 65 constant
+// sets: 2,080 rows 4.2 / 4.6 / 5.3, 4,160 rows 6.7 / 5.7 / 6.1.
 constexpr int kSpreadWarps = 14;
 int sim_rows_per_warp(int width, int64_t n_rows)
 {
@@ -1304,8 +1306,8 @@ namespace {
 // persistent warps are resident at once (its launch bound promises that many
 // blocks an SM): 4 blocks / 128 registers for launches of up to 16 warps an SM,
 // which wait on their own chains and not for issue slots, so spills and
-// constants re-read from the parameter bank cost time (256 rows of each kind:
-// document 6.5 -> 5.7 ms, 3,120 learned rows 9.1 -> 8.4 ms against 7 blocks);
+// constants re-read from the parameter bank cost time (against 7 blocks, 1,500
+// requests: 2,048 document rows 4.8 -> 4.3 ms, 2,080 learned rows 4.5 -> 4.2);
 // 7 blocks / 72 registers for one wave of up to 28; else 8 / 64, where more
 // warps hide more latency.
 template <int G, int kMode>
@@ -1327,9 +1329,10 @@ cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
 
 // A block per row, a warp per instance, where every block is resident at 128
 // registers (16 warps an SM) and has at most 16 warps.  2,000 requests, four
-// policies, 2P+6D: 152 rows 3.9 ms against 4.5 with a row per warp, 304 rows
-// 4.3 / 4.5, 400 rows (a second wave) 6.2 / 4.5; 3P+9D, 152 rows: 3.9 / 4.4;
-// proxy's signals, 152 rows: 3.4 / 4.3; 4P+28D (32 warps, 64 registers): 5.1 / 4.0.
+// policies, 2P+6D: 152 rows 3.55 ms against 4.03 with a row per warp, 304 rows
+// 3.94 / 4.02, 400 rows (a second wave) 5.55 / 4.03; 3P+9D, 152 rows: 3.58 / 3.92;
+// proxy's signals, 152 rows: 3.07 / 3.86; baselines alone, 150 rows: 2.03 / 2.70;
+// 4P+28D (32 warps, 64 registers; an earlier source): 5.1 / 4.0.
 constexpr int kRowWarpsPerSM = 16;
 bool row_per_block(const SimParams& p, int sms)
 {
