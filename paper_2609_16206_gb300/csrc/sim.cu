@@ -381,12 +381,11 @@ __device__ __forceinline__ int64_t next_event(const Decode& s) { return s.step_e
 // (the quotient is below run <= 2^20).
 __device__ __forceinline__ int32_t ends_by(const Decode& s, int64_t t)
 {
-    if (s.n_act == 0 || t < s.step_end) return 0;
-    const int32_t dt = (int32_t)(t - s.step_end);
+    const int32_t dt = (int32_t)(t - s.step_end);  // what follows from a time before step_end is not kept
     int32_t q = div_estimate(dt, s.inv_step);
     const int32_t r = dt - q * s.step;
     q += (r >= s.step) - (r < 0);
-    return q + 1;
+    return (s.n_act == 0) | (t < s.step_end) ? 0 : q + 1;
 }
 
 // A request becomes KV-ready at tp: the event moves up to the first step end at
@@ -456,7 +455,9 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     while ((int32_t)(s.act_top >> kKeyBits) == s.step_idx) {  // never with an empty heap: its top is all ones
         const uint32_t k = (uint32_t)(s.act_top & kKeyMask);
         const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
-        if (sum_is_o_hat) s.sum -= V.o_hat(k, bad);
+        int32_t gone = 0;
+        if (sum_is_o_hat) gone = V.o_hat(k, bad);
+        s.sum -= gone;
         V.set_done(k, tev, bad);
         hpop<kArity>(act, s.n_act, s.act_top, heap_stride(P.cap_act), bad);
         if constexpr (kArity == 2) s.q -= 1;
@@ -509,11 +510,12 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     const int64_t end = tev + (int64_t)((uint64_t)(uint32_t)P.dec_seq * (uint32_t)n) +
                         (int64_t)(uint64_t)((uint32_t)P.dec_base + (uint32_t)kv_term(s.kv_res, P));
     s.step_end = idle ? tp : end;
-    for (; admitted > 0; --admitted) {  // first token at the end of this step
-        const int64_t prev = admitted > 1 ? V.first(last, bad) : 0;
+    for (; admitted > 1; --admitted) {  // first token at the end of this step
+        const uint32_t prev = (uint32_t)V.first(last, bad);
         V.set_first(last, s.step_end, bad);
-        last = (uint32_t)prev;
+        last = prev;
     }
+    if (admitted == 1) V.set_first(last, s.step_end, bad);
     // after j of the run's ends the KV term is that of kv_res + j n, and it stays q1 while j n <= room1
     // (q1 + 1 <= 2^31 and kv_div <= 2^31; the sum is below 2^32)
     const int32_t q1 = kv_term(s.kv_res + n, P);
