@@ -219,8 +219,9 @@ struct GoodputParams {
     uint64_t* row_hash;
     const int32_t* row_status;
     const uint64_t* kmix;  // optional with row_hash: the table of launch_mix_table for n_req
-    // set by launch_goodput: room for kept values per P99; every row starts on 16 bytes (read two requests at a time)
-    int32_t cand_cap;
+    // set by launch_goodput: log2 of a row's sampled requests; room for kept values per P99; every row starts on 16 bytes
+    // (read two requests at a time)
+    int32_t sample_log2, cand_cap;
     bool pairs;
 };
 cudaError_t launch_goodput(const GoodputParams& p, cudaStream_t stream);

@@ -4,9 +4,9 @@
 // exact nearest-rank P99 TPOT (Table 2 columns).
 //
 // One block per row.  A P99 needs the largest hundredth of its row only, so a
-// sample of the row (256 evenly spaced groups of four neighbours, a memory sector
-// each, in a histogram over logarithmic bins, 64 per octave) first gives a
-// threshold that about 3 % of the values reach, and the one pass over the row
+// sample of the row (256 or, of long rows, more evenly spaced groups of four
+// neighbours, a memory sector each, in a histogram over logarithmic bins, 64 per
+// octave) first gives a threshold that about 3 % of the values reach, and the one pass over the row
 // then keeps those that do: per request the trace's arrival, output length and
 // class and the row's t_first and t_done.  The P99 is the value of the remaining
 // rank among the kept ones: their histogram over the same bins finds its bin,
@@ -26,8 +26,8 @@ namespace {
 
 constexpr int kMaxThreads = 512;  // of a block: 128 in launches of many rows
 constexpr int kLogBins = 2112;  // bin 0: a value of 0; then 64 per octave of [1, 2^32)
-constexpr int kHistWords = kLogBins / 2;  // two 16-bit counts a word (no more than kSample or kMaxCand values are counted)
-constexpr int kSample = 1024;   // sampled requests of a row (all of a shorter one)
+constexpr int kHistWords = kLogBins / 2;  // two 16-bit counts a word (no more than the sample or kMaxCand are counted)
+constexpr int kMinSampleLog2 = 10, kMaxSampleLog2 = 13;  // sampled requests of a row (all of a shorter one)
 constexpr int kMaxCand = 8192;  // most values kept
 constexpr int kFew = 128;       // members of the rank's bin counted out directly
 constexpr int kDigit = 11;      // radix select
@@ -286,7 +286,8 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         // ---- the sample and the thresholds
         for (int i = tid; i < 2 * kHistWords; i += nt) (&hist[0][0])[i] = 0;
         if (tid < 2) n_cand[tid] = 0;
-        const int taken = n < kSample ? (int)n : kSample;
+        const int sample = 1 << P.sample_log2;
+        const int taken = n < sample ? (int)n : sample;
         int32_t taken_many = 0;
         __syncthreads();
         constexpr int kBatch = 4;  // samples a thread loads before it uses any
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 const int i = i0 + j * nt < taken ? i0 + j * nt : i0;
-                const int64_t k = n <= kSample ? i : ((((int64_t)(i >> 2) * n) / (kSample / 4)) & ~int64_t(3)) + (i & 3);
+                const int64_t k = n <= sample ? i : ((((int64_t)(i >> 2) * n) >> (P.sample_log2 - 2)) & ~int64_t(3)) + (i & 3);
                 const int64_t tf = ck_ldg(P.t_first, ob + k, out_len, bad);
                 ttft[j] = tf - ck_ldg(P.trace.arrival_us, tb + k, trace_len, bad);
                 if (kTpot) {
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         const int64_t t_ttft = threshold(hist[0], taken, n, S);
         uint32_t t_tpot = 0;  // 0: none
         if (kTpot && taken_many > 0) {
-            const int64_t t = threshold(hist[1], taken_many, n <= kSample ? taken_many : (int64_t)taken_many * n / kSample, S);
+            const int64_t t = threshold(hist[1], taken_many, n <= sample ? taken_many : ((int64_t)taken_many * n) >> P.sample_log2, S);
             t_tpot = t > 0 ? (uint32_t)t : 0;  // below 2^32
         }
 
@@ -458,6 +459,8 @@ __global__ void __launch_bounds__(256) mix_table_kernel(uint64_t* t, int64_t n)
     }
 }
 
+constexpr int64_t kLongRow = 30000, kHugeRow = 65536;  // see launch_rows
+
 template <bool kHash, bool kTpot>
 cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
 {
@@ -465,9 +468,24 @@ cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
     const size_t dyn_bytes = (size_t)p.cand_cap * 4 * (kTpot ? 2 : 1);
     cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCand * 8);
     if (err != cudaSuccess) return err;
-    // 128 threads a row, which overlap best, more while that leaves an SM's 1,024 threads partly idle (4 rows of
-    // 2,000: 15 us with 512, 21 with 128; 32 rows of 50,000: 62 and 169)
-    const int threads = p.n_rows <= (int64_t)sms * 2 ? 512 : p.n_rows <= (int64_t)sms * 4 ? 256 : 128;
+    // 128 threads a row, which overlap best (4,096 rows of 20,000 with the P99 TPOT: 481 us, 521 with 256), except
+    // - while that leaves an SM's 1,024 threads partly idle (4 rows of 2,000: 15 us with 512, 21 with 128; 32 rows of
+    //   50,000: 62 and 169);
+    // - for long rows, as the eight rows of an SM drift apart and read their replica's trace again, and their kept
+    //   values leave room for fewer blocks (4,096 rows, 128 / 256 / 512 threads: 28,000 requests 637 / 674 / 748 us,
+    //   32,000 763 / 756 / 821, 60,000 1,782 / 1,342 / 1,338; 1,824 rows of 90,000 1,243 / 911 / 837);
+    // - where eight rows an SM at a time leave the last turn so empty that four at a time take clearly fewer row
+    //   times (2,500 rows of 20,000: 343 us with 128, 318 with 256; 1,300: 231 and 196; 3,040 even; rows of 5,000
+    //   lose up to 10 %).
+    const auto turns = [&](int64_t rows_at_once) {  // row times of an SM
+        const int64_t slots = sms * rows_at_once;
+        return (p.n_rows + slots - 1) / slots * rows_at_once;
+    };
+    int threads = 128;
+    if (p.n_rows <= (int64_t)sms * 2 || p.n_req >= kHugeRow)
+        threads = 512;
+    else if (p.n_rows <= (int64_t)sms * 4 || p.n_req >= kLongRow || (p.n_req >= 10000 && 20 * turns(8) > 23 * turns(4)))
+        threads = 256;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn_bytes);
     if (err != cudaSuccess) return err;
@@ -500,6 +518,10 @@ cudaError_t launch_goodput(const GoodputParams& given, cudaStream_t stream)
     p.pairs = p.n_req % 2 == 0 &&
               ((uintptr_t)p.trace.arrival_us | (uintptr_t)p.t_first | (uintptr_t)p.t_done | (uintptr_t)p.kmix) % 16 == 0 &&
               (uintptr_t)p.trace.true_out % 8 == 0 && (uintptr_t)p.trace.slo_class % 2 == 0;
+    // one request in 32 to 64 of a long row, so that the kept values, 3 % of a row at 1,024 samples, still have room:
+    // 1,200 rows of 200,000: 1,093 us, 3,980 with 1,024 samples (past kMaxCand a row takes the radix select)
+    p.sample_log2 = kMinSampleLog2;
+    while (p.sample_log2 < kMaxSampleLog2 && (int64_t(64) << p.sample_log2) < p.n_req) ++p.sample_log2;
     // room for a sixteenth of the row (3 % is expected, more where a bin holds many)
     const int64_t room = p.n_req / 16 + 64;
     p.cand_cap = (int32_t)(room < 512 ? 512 : room > kMaxCand ? kMaxCand : room);

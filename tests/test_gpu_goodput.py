@@ -240,3 +240,26 @@ def test_p99_threshold_from_the_sample(orc, N, shape):
         row = {k: v[r] for k, v in trh.items()}
         assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), row, tf[r], td[r]), r
         assert tpot[r] == orc.p99_tpot({"true_out": o[r]}, tf[r], td[r]), r
+
+
+@pytest.mark.parametrize("rows,N", [(1217, 9_999), (1217, 10_000), (1216, 10_002), (609, 29_999), (609, 30_000),
+                                    (305, 30_001), (5, 65_535), (5, 65_536), (5, 65_538), (3, 131_075), (2, 524_290)])
+def test_block_size_and_sample_by_row_length(orc, rows, N):
+    """Both sides of the row lengths and row counts at which a row's block widens and its sample grows."""
+    ctr = need_gpu()
+    g = torch.Generator(device="cuda").manual_seed(N + rows)
+    o = torch.randint(1, 400, (rows, N), generator=g, device="cuda")
+    arr = torch.sort(torch.randint(0, 10**9, (rows, N), generator=g, device="cuda"), dim=1).values
+    tf = arr + torch.exp(13 + torch.randn((rows, N), generator=g, device="cuda")).long()
+    td = tf + torch.randint(10**4, 10**5, (rows, N), generator=g, device="cuda") * (o - 1) + 1
+    cls = torch.randint(0, 2, (rows, N), generator=g, device="cuda")
+    one = torch.ones_like(o)
+    tr = {"arrival_us": arr, "prompt_len": one.int(), "true_out": o.int(), "pred_out": one.int(),
+          "slo_class": cls.to(torch.uint8)}
+    met, p99 = _goodput(ctr, W.SimCfg(), tr, rows, 1, N, tf, td)
+    tpot = _p99_tpot(ctr, W.SimCfg(), tr, rows, 1, N, tf, td)
+    for r in sorted({*range(0, rows, 151), rows - 1}):
+        row = {k: v[r].cpu().numpy() for k, v in tr.items()}
+        f, d = tf[r].cpu().numpy(), td[r].cpu().numpy()
+        assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), row, f, d), r
+        assert tpot[r] == orc.p99_tpot({"true_out": row["true_out"]}, f, d), r
