@@ -530,7 +530,8 @@ def run_ours(args, rank, world, local_rank):
     if cnt is not None:
         # executed warp-instructions scale with routed requests (every row group's instruction stream is
         # fixed by its inputs), so the slice's count per routed request times this launch's routed requests
-        # is this launch's count; DRAM bytes are scaled the same way (the slice holds fewer warps per SM)
+        # is this launch's count (both carry four rows a warp); DRAM bytes are scaled the same way (the slice
+        # holds 17 warps an SM, the launch 27)
         routed_launch = rows * N
         sim_roof["achieved"] = cnt["warp_inst_per_routed"] * routed_launch / (per_kernel_ms["sim"] / 1e3) / 1e9
         sim_roof["frac"] = sim_roof["achieved"] / issue_peak
@@ -605,21 +606,22 @@ def run_ours(args, rank, world, local_rank):
 
 # Counters of one sim_kernel launch on a slice of the benchmarked workload
 # (ncu sm__inst_executed.sum, smsp__thread_inst_executed.sum and DRAM bytes of
-# 1,024 replicas x 20,000 requests x 4 policies, a few GB on the device),
-# per routed request, keyed by a hash of the simulator's code: a stale entry
+# 2,560 replicas x 8,000 requests x 4 policies, a few GB on the device; enough
+# rows that a warp carries four of them, as in the full launch), per routed
+# request, keyed by a hash of the simulator's code: a stale entry
 # (the kernel changed since the counters were taken) reports null.
 SIM_SLICE_COUNTERS: dict = {
-    "5b2cb8e0e1f5e9de": {"warp_inst_per_routed": 34162633267 / 81_920_000,
-                         "thread_inst_per_warp_inst": 281165931678 / 34162633267,
-                         "dram_bytes_per_routed": (2383411200 + 1563864576) / 81_920_000,
-                         "slice": "ncu on one launch of 1,024 replicas x 20,000 requests x 4 policies "
-                                  "(81.92 M routed requests): 3.416e10 warp-instructions, 2.812e11 thread-"
-                                  "instructions, 2.383 GB DRAM read + 1.564 GB written"},
+    "64afa14802b7ece5": {"warp_inst_per_routed": 22899474615 / 81_920_000,
+                         "thread_inst_per_warp_inst": 184476552804 / 22899474615,
+                         "dram_bytes_per_routed": (1615253504 + 2389551616) / 81_920_000,
+                         "slice": "ncu on one launch of 2,560 replicas x 8,000 requests x 4 policies "
+                                  "(81.92 M routed requests): 2.290e10 warp-instructions, 1.845e11 thread-"
+                                  "instructions, 1.615 GB DRAM read + 2.390 GB written"},
 }
 
 # DRAM bytes of one scorer launch (2^20 requests x 64 instances) inside the step.
 SCORE_DRAM_PER_LAUNCH: dict = {
-    "f16cba77579b1bc7": {"read": 9484800.0, "write": 0.0},
+    "44c805c02eec218b": {"read": 9467648.0, "write": 0.0},
 }
 
 

@@ -260,7 +260,6 @@ __device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t
     return v;
 }
 
-
 // Bound by the pass: about 110 warp-instructions for 32 requests (64-bit times,
 // the SLO tables, one kept value in 30) and the bytes in flight.  Eight blocks
 // of 128 threads an SM overlap one row's sample and selection with the others'
