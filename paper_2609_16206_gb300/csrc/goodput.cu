@@ -13,8 +13,10 @@
 // whose few members are counted out.  A row whose kept values are fewer than the
 // rank needs or more than there is room for (thousands of equal values at the
 // P99), or of 2^32 and more, takes an exact radix select over all its values read
-// from global memory (11-bit digits, most significant first).  A TPOT is compared
-// without a division (floor(d / m) >= t is d >= t m) and divided only when kept.
+// from global memory (10-bit digits, most significant first).  A TPOT is compared
+// without a division (floor(d / m) >= t is d >= t m) and divided only when kept,
+// after the pass where there is room for the divisors: in the pass the few lanes
+// that keep one would make their whole warp divide.
 // Called from ctr_simulate with kHash, the pass also sums each row's checksum
 // terms of first-token and completion times; the request-only half of those terms
 // is read from the call's table (launch_mix_table) when ctr_simulate has one,
@@ -30,9 +32,9 @@ constexpr int kHistWords = kLogBins / 2;  // two 16-bit counts a word (no more t
 constexpr int kMinSampleLog2 = 10, kMaxSampleLog2 = 13;  // sampled requests of a row (all of a shorter one)
 constexpr int kMaxCand = 8192;  // most values kept
 constexpr int kFew = 128;       // members of the rank's bin counted out directly
-constexpr int kDigit = 11;      // radix select
+constexpr int kDigit = 10;      // radix select
 constexpr int kBins = 1 << kDigit;
-static_assert(kBins <= 2 * kHistWords, "the radix select takes the place of two 16-bit histograms");
+static_assert(kBins <= kHistWords, "the radix select takes the place of a 16-bit histogram");
 
 // Monotone bin of a value in [0, 2^32): the exponent and the top 6 mantissa bits
 // of its fp32 value rounded toward zero (exact integer to float conversion
@@ -263,16 +265,19 @@ __device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t
 // Bound by the pass: about 110 warp-instructions for 32 requests (64-bit times,
 // the SLO tables, one kept value in 30) and the bytes in flight.  Eight blocks
 // of 128 threads an SM overlap one row's sample and selection with the others'
-// passes.  4,096 rows x 20,000: 470 us with the P99 TPOT, 324 us without; 873 and
+// passes.  4,096 rows x 20,000: 459 us with the P99 TPOT, 322 us without; 873 and
 // 400 us when every request's logarithmic bin was counted and staged in shared
 // memory and the TPOT took two more passes of its own.
-template <bool kHash, bool kTpot>
+template <bool kHash, bool kTpot, bool kLater>
 __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputParams P)
 {
-    __shared__ uint32_t hist[2][kHistWords];  // TTFT and TPOT
+    __shared__ uint32_t hist_s[kHistWords];  // of the TTFTs, then of the kept values
     __shared__ SelScratch S;
     __shared__ uint32_t n_cand[2];
-    extern __shared__ uint32_t cand_s[];  // kept TTFTs, then TPOTs, cap each
+    // kept TTFTs, then TPOTs (with kLater decode times, then output lengths less 1), cap each; before the pass the
+    // TPOTs' histogram.  Little shared memory leaves the pass more L1 for its loads in flight.
+    extern __shared__ uint32_t cand_s[];
+    uint32_t* const hist[2] = {hist_s, cand_s};
     const int tid = threadIdx.x, nt = blockDim.x;
     const int64_t n = P.n_req;
     const int64_t trace_len = (P.n_rows / P.rows_per_replica) * n, out_len = P.n_rows * n;  // entries of trace and outputs
@@ -283,7 +288,10 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         bool bad = false;  // bounds-checked builds: an index of this thread fell outside its buffer
 
         // ---- the sample and the thresholds
-        for (int i = tid; i < 2 * kHistWords; i += nt) (&hist[0][0])[i] = 0;
+        for (int i = tid; i < kHistWords; i += nt) {
+            hist[0][i] = 0;
+            if (kTpot) hist[1][i] = 0;
+        }
         if (tid < 2) n_cand[tid] = 0;
         const int sample = 1 << P.sample_log2;
         const int taken = n < sample ? (int)n : sample;
@@ -346,7 +354,12 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
                 if (dec >= (int64_t)((uint64_t)t_tpot * (uint32_t)(o - 1))) {
                     const uint32_t i = atomicAdd(&n_cand[1], 1u);
                     if ((uint64_t)dec >> 32) wide = 1;
-                    if (i < cap) cand_s[cap + i] = (uint32_t)dec / (uint32_t)(o - 1);
+                    if (i < cap && kLater) {
+                        cand_s[cap + i] = (uint32_t)dec;
+                        cand_s[2 * cap + i] = (uint32_t)(o - 1);
+                    } else if (i < cap) {
+                        cand_s[cap + i] = (uint32_t)dec / (uint32_t)(o - 1);
+                    }
                 }
             }
             if (kHash) {
@@ -423,6 +436,9 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         if (kTpot && many > 0) {
             const int64_t below = many - (int64_t)n_cand[1], rank = p99_rank(many);
             if (t_tpot > 0 && n_cand[1] <= cap && rank >= below && packs) {
+                if (kLater)
+                    for (int i = tid; i < (int)n_cand[1]; i += nt) cand_s[cap + i] /= cand_s[2 * cap + i];
+                // (its barriers order the divided values)
                 p99_tpot = kept_rank(cand_s + cap, (int)n_cand[1], rank - below, hist[0], S CTR_CK_FLAG_ARG);
             } else {
                 auto tpot_of = [&](int64_t k, int64_t& v) {
@@ -463,11 +479,8 @@ constexpr int64_t kLongRow = 30000, kHugeRow = 65536;  // see launch_rows
 template <bool kHash, bool kTpot>
 cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
 {
-    const auto k = goodput_kernel<kHash, kTpot>;
-    const size_t dyn_bytes = (size_t)p.cand_cap * 4 * (kTpot ? 2 : 1);
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCand * 8);
-    if (err != cudaSuccess) return err;
-    // 128 threads a row, which overlap best (4,096 rows of 20,000 with the P99 TPOT: 481 us, 521 with 256), except
+    // 128 threads a row, which overlap best (4,096 rows of 20,000 with the P99 TPOT, as all figures here, TPOTs divided
+    // in the pass: 481 us, 521 with 256), except
     // - while that leaves an SM's 1,024 threads partly idle (4 rows of 2,000: 15 us with 512, 21 with 128; 32 rows of
     //   50,000: 62 and 169);
     // - for long rows, as the eight rows of an SM drift apart and read their replica's trace again, and their kept
@@ -485,6 +498,17 @@ cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
         threads = 512;
     else if (p.n_rows <= (int64_t)sms * 4 || p.n_req >= kLongRow || (p.n_req >= 10000 && 20 * turns(8) > 23 * turns(4)))
         threads = 256;
+    // TPOTs are divided after the pass while their divisors leave L1 60 KB of the SM's 256 (with 128 threads up to
+    // rows of 23,400, with 256 of 56,000, with 512 of 120,000; with the P99 TPOT, us without / with: 4,096 rows of
+    // 20,000 483 / 459, 3,040 of 20,000 384 / 365, 4,096 of 40,000 894 / 848; past it 4,096 of 28,000 633 / 683,
+    // 4,096 of 60,000 1,338 / 1,428)
+    const size_t block_bytes = sizeof(SelScratch) + kHistWords * 4 + 1024;
+    const bool later = kTpot && (kMaxThreads * 2 / threads) * (block_bytes + (size_t)p.cand_cap * 12) <= 196 * 1024;
+    const auto k = later ? goodput_kernel<kHash, kTpot, kTpot> : goodput_kernel<kHash, kTpot, false>;
+    size_t dyn_bytes = (size_t)p.cand_cap * 4 * (later ? 3 : kTpot ? 2 : 1);
+    if (kTpot && dyn_bytes < kHistWords * 4) dyn_bytes = kHistWords * 4;
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCand * 12);
+    if (err != cudaSuccess) return err;
     int per_sm = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn_bytes);
     if (err != cudaSuccess) return err;

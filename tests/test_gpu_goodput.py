@@ -243,9 +243,11 @@ def test_p99_threshold_from_the_sample(orc, N, shape):
 
 
 @pytest.mark.parametrize("rows,N", [(1217, 9_999), (1217, 10_000), (1216, 10_002), (609, 29_999), (609, 30_000),
-                                    (305, 30_001), (5, 65_535), (5, 65_536), (5, 65_538), (3, 131_075), (2, 524_290)])
+                                    (305, 30_001), (5, 65_535), (5, 65_536), (5, 65_538), (3, 124_831), (3, 124_832),
+                                    (3, 131_075), (2, 524_290)])
 def test_block_size_and_sample_by_row_length(orc, rows, N):
-    """Both sides of the row lengths and row counts at which a row's block widens and its sample grows."""
+    """Both sides of the row lengths and row counts at which a row's block widens, its sample grows and its TPOTs are
+    divided in the pass instead of after it."""
     ctr = need_gpu()
     g = torch.Generator(device="cuda").manual_seed(N + rows)
     o = torch.randint(1, 400, (rows, N), generator=g, device="cuda")
