@@ -508,10 +508,15 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream)
     // against 2 us for the 8 of a block): 1 x 10,000 requests 459 -> 11.5 us, 64 x 10,000 469 -> 34,
     // 1,024 x 5,000 271 -> 167, 3,000 x 5,000 457 -> 441.  Short traces leave a block's warps idle and stay
     // with one warp a replica unless there are very few of them: 1,000 x 64 takes 6.3 us there, 13 us split.
+    // The fewer its chunks, the fewer replicas pay for a block's barriers and uneven last chunks (MMPP, split / whole:
+    // 512 requests 1,520 replicas 36 / 37 us, 1,824 41 / 37, 3,040 64 / 51; 1,000 requests 2,128 78 / 80, 2,432 88 / 80;
+    // 2,500 requests 2,736 217 / 228, 3,040 240 / 228; 4,000 requests 3,040 371 / 421).
     const int64_t n_chunks = (p.n_req + 31) / 32;
-    if (p.n_replicas <= (int64_t)sms * 20 && n_chunks >= (p.n_replicas <= sms ? 4 : 16)) {
-        // blocks per replica: up to 8 blocks an SM in all, at least 2 chunks a block; clusters of 16 only for a few replicas, as they are slow to place (16 x 10,000: 19.6 us with 8
-        // blocks, 16.8 with 16; 64 x 10,000: 34 us with 4 or 8, 40 with 16)
+    const int64_t most = (int64_t)sms * (n_chunks < 32 ? 10 : n_chunks < 64 ? 15 : n_chunks < 100 ? 18 : 20);
+    if (p.n_replicas <= most && n_chunks >= (p.n_replicas <= sms ? 4 : 16)) {
+        // blocks per replica: up to 8 blocks an SM in all, at least 2 chunks a block; clusters of 16 only for a few
+        // replicas, as they are slow to place (16 x 10,000: 19.6 us with 8 blocks, 16.8 with 16; 64 x 10,000: 34 us
+        // with 4 or 8, 40 with 16)
         int cluster = 1;
         while (cluster < kMaxCluster &&
                ((p.n_replicas * cluster * 2 <= (cluster < 8 ? sms * 8 : sms * 2) && n_chunks >= cluster * 4) ||

@@ -35,7 +35,8 @@ def test_trace_bit_identical(orc, name, tc, R, N, off):
 
 
 @pytest.mark.parametrize("R,N", [(1, 32), (1, 63), (2, 64), (1, 65), (3, 1025), (1, 10_000), (17, 10_001), (130, 257),
-                                 (1, 700_001), (700, 40), (152, 128), (153, 128), (3040, 513), (3041, 513)])
+                                 (1, 700_001), (700, 40), (152, 128), (153, 128), (1520, 513), (1521, 513), (2280, 1025),
+                                 (2281, 1025), (2736, 2049), (2737, 2049), (3040, 3201), (3041, 3201)])
 @pytest.mark.parametrize("tc", [W.replica_sweep().trace, W.TraceCfg(seed=11, n_classes=1, class_thr=()),
                                 W.TraceCfg(seed=3, n_seeds=2, arrival_kind=1, rate_mreq=(9_000_000, 40),
                                            dwell_mean_us=1_000)], ids=["mmpp", "poisson", "short_dwell"])
