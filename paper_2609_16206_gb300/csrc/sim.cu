@@ -222,18 +222,30 @@ __device__ __forceinline__ void heap_pop_bin(uint64_t* h, int32_t& n, uint64_t& 
 // two redux.sync, so a level costs one child's worth of instructions instead of
 // 32 and a heap of up to 33 keys has one.  Node j sits at position j + 3, its
 // children at 32 j + 4 .. 32 j + 35: the 4-ary region's size serves.
+// Nothing but a __syncwarp keeps the lanes of a warp in step, so what they share
+// in memory follows one rule: a word has one lane that stores it, and a __syncwarp
+// stands between that store and the other lanes' later loads, and between the
+// other lanes' loads and a later store.  Every heap operation ends with one.
+template <typename T, typename I>
+__device__ __forceinline__ void lane_st(int lane, T* p, I i, int64_t lim, T v, bool& bad)
+{
+    if ((int)(threadIdx.x & 31) == lane) ck_st(p, i, lim, v, bad);
+}
+
 __device__ __forceinline__ void heap_push_warp(uint64_t* h, int32_t& n, uint64_t& top, uint64_t key, int64_t lim,
                                                bool& bad)
 {
     int i = kHeapRoot + n++;
     while (i > kHeapRoot) {
         const int parent = ((i - 4) >> 5) + kHeapRoot;
-        const uint64_t pv = ck_ld(h, parent, lim, bad);
+        const uint64_t pv = parent == kHeapRoot ? top : ck_ld(h, parent, lim, bad);
         if (pv < key) break;
-        ck_st(h, i, lim, pv, bad);
+        __syncwarp();  // the parent has been read; it is stored to next
+        lane_st(0, h, i, lim, pv, bad);
         i = parent;
     }
-    ck_st(h, i, lim, key, bad);
+    lane_st(0, h, i, lim, key, bad);
+    __syncwarp();
     if (i == kHeapRoot) top = key;
 }
 
@@ -248,6 +260,7 @@ __device__ __forceinline__ void heap_pop_warp(uint64_t* h, int32_t& n, uint64_t&
     const int lastp = kHeapRoot + m - 1;
     const uint64_t last = ck_ld(h, lastp, lim, bad);
     int i = kHeapRoot;
+    int reader = 0;         // the only lane that has read position i
     uint64_t first = last;  // what comes to the root
     for (;;) {
         const int c = 32 * (i - kHeapRoot) + 4;  // first child
@@ -259,10 +272,12 @@ __device__ __forceinline__ void heap_pop_warp(uint64_t* h, int32_t& n, uint64_t&
         const uint64_t cv = ((uint64_t)mhi << 32) | mlo;
         if (last < cv) break;
         if (i == kHeapRoot) first = cv;
-        ck_st(h, i, lim, cv, bad);
-        i = c + __ffs(__ballot_sync(kFull, v == cv)) - 1;
+        lane_st(reader, h, i, lim, cv, bad);
+        reader = __ffs(__ballot_sync(kFull, v == cv)) - 1;
+        i = c + reader;
     }
-    ck_st(h, i, lim, last, bad);
+    lane_st(reader, h, i, lim, last, bad);
+    __syncwarp();
     top = first;
 }
 
@@ -289,6 +304,30 @@ __device__ __forceinline__ void hpop(uint64_t* h, int32_t& n, uint64_t& top, int
         heap_pop(h, n, top, lim, bad);
 }
 
+// Accesses to an instance's other structures and to its requests' entries: plain ones of the lane that simulates it,
+// or those of a warp that does together.  own_ld: its lanes have all read.
+template <int kArity, typename T, typename I>
+__device__ __forceinline__ T own_ld(const T* p, I i, int64_t lim, bool& bad)
+{
+    const T v = ck_ld(p, i, lim, bad);
+    if constexpr (kArity == 32) __syncwarp();
+    return v;
+}
+template <int kArity, typename T, typename I>
+__device__ __forceinline__ void own_st(T* p, I i, int64_t lim, T v, bool& bad)
+{
+    if constexpr (kArity == 32)
+        lane_st(0, p, i, lim, v, bad);
+    else
+        ck_st(p, i, lim, v, bad);
+}
+// what own_st has stored may be read from here on
+template <int kArity>
+__device__ __forceinline__ void own_stored()
+{
+    if constexpr (kArity == 32) __syncwarp();
+}
+
 // argmin over the lanes of 64-bit values (ties -> lowest lane)
 __device__ __forceinline__ int warp_argmin(uint64_t v)
 {
@@ -303,7 +342,7 @@ __device__ __forceinline__ int warp_argmin(uint64_t v)
 // registers allow (kPtr: 128 of them), else two offsets added on each access
 // (pointers in every instantiation: single replica 4.72 -> 4.65 ms, but the
 // replica sweep at 72 registers 137.0 -> 137.8).
-template <bool kPtr>
+template <bool kPtr, int kArity>
 struct RowView {
     const SimParams& P;
     const int32_t *p_ = nullptr, *o_ = nullptr;
@@ -332,15 +371,15 @@ struct RowView {
     }
     __device__ __forceinline__ int64_t first(uint32_t k, bool& bad) const
     {
-        return kPtr ? ck_ld(tf_, k, P.n_req, bad) : ck_ld(P.t_first, ob + k, P.out_len, bad);
+        return kPtr ? own_ld<kArity>(tf_, k, P.n_req, bad) : own_ld<kArity>(P.t_first, ob + k, P.out_len, bad);
     }
     __device__ __forceinline__ void set_first(uint32_t k, int64_t v, bool& bad) const
     {
-        kPtr ? ck_st(tf_, k, P.n_req, v, bad) : ck_st(P.t_first, ob + k, P.out_len, v, bad);
+        kPtr ? own_st<kArity>(tf_, k, P.n_req, v, bad) : own_st<kArity>(P.t_first, ob + k, P.out_len, v, bad);
     }
     __device__ __forceinline__ void set_done(uint32_t k, int64_t v, bool& bad) const
     {
-        kPtr ? ck_st(td_, k, P.n_req, v, bad) : ck_st(P.t_done, ob + k, P.out_len, v, bad);
+        kPtr ? own_st<kArity>(td_, k, P.n_req, v, bad) : own_st<kArity>(P.t_done, ob + k, P.out_len, v, bad);
     }
 };
 
@@ -427,7 +466,8 @@ __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, c
         if (--room < 0) return CTR_EOVERFLOW;
         int pos = s.w_head + s.w_n;
         if (pos >= P.cap_wait) pos -= P.cap_wait;
-        ck_st(wait, pos, P.cap_wait, k, bad);
+        own_st<kArity>(wait, pos, P.cap_wait, k, bad);
+        own_stored<kArity>();
         s.w_n += 1;
     }
     return CTR_OK;
@@ -443,7 +483,7 @@ __device__ __forceinline__ int flush_ready(Decode& s, int64_t t, int32_t room, c
 // overflowed.
 template <int kArity, bool kPtr>
 __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimParams& P, uint64_t* pend, uint64_t* act,
-                                            uint32_t* wait, const RowView<kPtr>& V, bool sum_is_o_hat, bool& bad)
+                                            uint32_t* wait, const RowView<kPtr, kArity>& V, bool sum_is_o_hat, bool& bad)
 {
     {  // (1) run + 1 steps end (none of an idle instance): as many tokens for every active request
         const int32_t ends = s.n_act > 0 ? s.run + 1 : 0;
@@ -474,7 +514,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     for (;;) {
         const bool fifo = s.w_n > 0;
         if (!fifo && s.pend_top >= by) break;
-        const uint32_t k = fifo ? ck_ld(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
+        const uint32_t k = fifo ? own_ld<kArity>(wait, s.w_head, P.cap_wait, bad) : (uint32_t)(s.pend_top & kKeyMask);
         const int32_t pk = V.p(k, bad), ok = V.o(k, bad);
         const bool fits = (uint32_t)s.kv_rsv + (uint32_t)(pk + ok) <= (uint32_t)P.kv_cap;  // < 2^31 + 2^21
         if (!fits || s.n_act == P.cap_act) {
@@ -510,6 +550,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     const int64_t end = tev + (int64_t)((uint64_t)(uint32_t)P.dec_seq * (uint32_t)n) +
                         (int64_t)(uint64_t)((uint32_t)P.dec_base + (uint32_t)kv_term(s.kv_res, P));
     s.step_end = idle ? tp : end;
+    if (kArity == 32 && admitted > 1) own_stored<kArity>();
     for (; admitted > 1; --admitted) {  // first token at the end of this step
         const uint32_t prev = (uint32_t)V.first(last, bad);
         V.set_first(last, s.step_end, bad);
@@ -537,7 +578,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
 // at times <= tsnap (an occupancy poll; tsnap <= T).
 template <bool kSnap, int kArity, bool kPtr>
 __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimParams& P, uint64_t* pend, uint64_t* act,
-                                              uint32_t* wait, const RowView<kPtr>& V, int64_t tsnap, int64_t& kv_snap,
+                                              uint32_t* wait, const RowView<kPtr, kArity>& V, int64_t tsnap, int64_t& kv_snap,
                                               bool sum_is_o_hat, bool& bad)
 {
     for (;;) {
@@ -559,7 +600,7 @@ __device__ __forceinline__ int decode_advance(Decode& s, int64_t T, const SimPar
 // batched), act_top the ring's front entry (end << 21 | p, read while it holds
 // any), sum the prompt tokens of the prefills in the ring, w_head / w_n the ring.
 // Retire the serial prefills that ended by T.
-template <bool kSig>
+template <bool kSig, int kArity>
 __device__ __forceinline__ void retire_prefills(Decode& s, int64_t T, const SimParams& P, const int64_t* ring, bool& bad)
 {
     const int64_t thr = ((T + 1) << kRingPBits) - 1;  // entries whose prefill ended by T
@@ -567,7 +608,7 @@ __device__ __forceinline__ void retire_prefills(Decode& s, int64_t T, const SimP
         if constexpr (kSig) s.sum -= s.act_top & kRingPMask;
         s.w_head = s.w_head + 1 == P.cap_ring ? 0 : s.w_head + 1;
         s.w_n -= 1;
-        s.act_top = s.w_n > 0 ? (uint64_t)ck_ld(ring, s.w_head, (int64_t)P.cap_ring, bad) : (uint64_t)kNever;
+        s.act_top = s.w_n > 0 ? (uint64_t)own_ld<kArity>(ring, s.w_head, P.cap_ring, bad) : (uint64_t)kNever;
     }
     if (s.w_n == 0) s.w_head = 0;
 }
@@ -675,7 +716,7 @@ __device__ __forceinline__ int64_t prefill_end(const SimParams& P, int64_t busy,
 }
 
 // Commit a serial prefill ending at `end` to its lane (the caller has checked the time limit).
-template <bool kSig>
+template <bool kSig, int kArity>
 __device__ __forceinline__ int push_prefill(Decode& s, int64_t end, uint32_t p, const SimParams& P, int64_t* ring,
                                             bool& bad)
 {
@@ -684,7 +725,8 @@ __device__ __forceinline__ int push_prefill(Decode& s, int64_t end, uint32_t p, 
     int pos = s.w_head + s.w_n;
     if (pos >= P.cap_ring) pos -= P.cap_ring;
     const int64_t e = (end << kRingPBits) | p;
-    ck_st(ring, pos, (int64_t)P.cap_ring, e, bad);
+    own_st<kArity>(ring, pos, P.cap_ring, e, bad);
+    own_stored<kArity>();
     if (s.w_n == 0) s.act_top = (uint64_t)e;
     s.w_n += 1;
     if constexpr (kSig) s.sum += p;
@@ -815,7 +857,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
         const bool sum_is_o_hat = pol == CTR_POLICY_LENGTH_HEURISTIC || (kSig && learned_row && cc.proxy);
         const int64_t tb = rep * n;
         const int64_t ob = row * n;
-        const RowView<kBlocksPerSM <= 4> V(P, tb, ob);
+        const RowView<kBlocksPerSM <= 4, kArity> V(P, tb, ob);
 
         // per-request bounds, one row at a time with the whole warp
         bool oob = false;  // bounds-checked builds: an index of this lane fell outside its buffer
@@ -958,7 +1000,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                             err = decode_advance<kSig, kArity>(s, T, P, pend, act, wait, V, tsnap, kv_seen,
                                                                sum_is_o_hat, oob);
                     } else if (is_pre && !batched) {
-                        retire_prefills<kSig>(s, T, P, ring, oob);
+                        retire_prefills<kSig, kArity>(s, T, P, ring, oob);
                     }
                 }
                 if (__ballot_sync(kFull, err != CTR_OK) & gmask) live = false;
@@ -1019,7 +1061,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                 } else if (live && gl == ip) {
                     const int64_t end = prefill_end(P, busy, T, (uint32_t)pk);
                     ready = end + (int64_t)(int32_t)P.xfer_tok * (int32_t)pk;
-                    err = ready >= kTimeLimit ? CTR_EOVERFLOW : push_prefill<kSig>(s, end, (uint32_t)pk, P, ring, oob);
+                    err = ready >= kTimeLimit ? CTR_EOVERFLOW : push_prefill<kSig, kArity>(s, end, (uint32_t)pk, P, ring, oob);
                 }
                 ready = __shfl_sync(kFull, ready, ip, G);
                 if (live && gl == P.n_pre + id && ready < kTimeLimit && err == CTR_OK)
@@ -1064,8 +1106,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
 }
 
 // One block per row, one warp per instance, for launches of few rows: all lanes
-// of a warp simulate the same instance (same state, same control flow, same
-// stores), so no event waits for another instance's and the heaps are worked by
+// of a warp simulate the same instance (same state, same control flow; what they
+// share in memory follows heap_push_warp's rule), so no event waits for another instance's and the heaps are worked by
 // the whole warp.  Every warp follows the row's arrivals.  Per arrival the
 // instances' costs go through shared memory, one barrier, and each warp takes
 // both argmins itself; the ends of all prefill queues ride along in every warp
@@ -1101,7 +1143,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
         const bool learned_row = pol == CTR_POLICY_LEARNED || pol == CTR_POLICY_LEARNED_P2;
         const bool sum_is_o_hat = pol == CTR_POLICY_LENGTH_HEURISTIC || (kSig && learned_row && cc.proxy);
         const int64_t tb = row / per_rep * n, ob = row * n;
-        const RowView<true> V(P, tb, ob);
+        const RowView<true, kArity> V(P, tb, ob);
         bool oob = false;  // bounds-checked builds: an index of this warp fell outside its buffer
 
         // per-request bounds and arrival order, a stretch of 32 requests per warp
@@ -1142,7 +1184,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
                 // 1. the instance's events up to the arrival
                 if (err == CTR_OK) {
                     if (is_pre) {
-                        retire_prefills<kSig>(s, T, P, ring, oob);
+                        retire_prefills<kSig, kArity>(s, T, P, ring, oob);
                     } else {
                         int64_t tsnap = -1;  // >= 0: the occupancy at this time is recorded on the way
                         if (kSig && cc.poll_us > 0) {
@@ -1187,7 +1229,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
                 if (lane == ip) busy = end;
                 if (err == CTR_OK) {
                     if (w == ip)
-                        err = push_prefill<kSig>(s, end, pk, P, ring, oob);
+                        err = push_prefill<kSig, kArity>(s, end, pk, P, ring, oob);
                     else if (w == P.n_pre + id)
                         err = queue_decode<kArity>(s, T, k, ready, sum_is_o_hat ? ohk : ok, P, pend, wait, oob);
                 }
@@ -1331,9 +1373,10 @@ cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
 
 // A block per row, a warp per instance, where every block is resident at 128
 // registers (16 warps an SM) and has at most 16 warps.  2,000 requests, four
-// policies, 2P+6D: 152 rows 3.55 ms against 4.03 with a row per warp, 304 rows
-// 3.94 / 4.02, 400 rows (a second wave) 5.55 / 4.03; 3P+9D, 152 rows: 3.58 / 3.92;
-// proxy's signals, 152 rows: 3.07 / 3.86; baselines alone, 150 rows: 2.03 / 2.70;
+// policies, 2P+6D: 152 rows 3.58 ms against 3.91 with a row per warp, 304 rows
+// 3.95 / 3.91 (proxy's signals 3.38 / 3.73, baselines alone 2.23 / 2.65), 400 rows
+// (a second wave; an earlier source) 5.55 / 4.03; 3P+9D, 152 rows: 3.63 / 3.81,
+// 200 (a second wave): 5.11 / 3.82; 4P+12D, 152 rows: 3.66 / 3.75;
 // 4P+28D (32 warps, 64 registers; an earlier source): 5.1 / 4.0.
 constexpr int kRowWarpsPerSM = 16;
 bool row_per_block(const SimParams& p, int sms)

@@ -1,0 +1,45 @@
+"""The simulator's kernels on the CPU (simlanes), the lanes of a warp as far
+apart as its barriers allow: every row the oracle's, and no access to shared
+structures that only a lockstep warp would keep in order."""
+import numpy as np
+import pytest
+
+import simlanes
+from paper_2609_16206_gb300 import workloads as W
+
+ALL_FIVE = list(W.ALL_POLICIES) + [W.POLICY_LEARNED_P2]
+
+
+@pytest.fixture(scope="module")
+def lanes(tmp_path_factory):
+    return simlanes.build(str(tmp_path_factory.mktemp("simlanes")))
+
+
+def check(orc, lanes, sc, sets, pols, traces, order, **kw):
+    res, races, stuck = simlanes.simulate(lanes, sc, sets, pols, traces, order=order, **kw)
+    assert (races, stuck) == (0, 0)
+    row = 0
+    for tr in traces:
+        for cc in sets:
+            for pol in pols:
+                o = orc.simulate(sc, cc, pol, tr)
+                assert res["status"][row] == o["status"], (row, pol)
+                if o["status"] == 0:
+                    assert int(res["hash"][row]) == o["hash"], (row, pol)
+                    for key in ("t_first_us", "t_done_us", "i_pre", "i_dec"):
+                        assert np.array_equal(res[key][row], o[key]), (row, pol, key)
+                row += 1
+    return res
+
+
+@pytest.mark.parametrize("order", [0, 1, 7])
+@pytest.mark.parametrize("sc,deployed", [
+    (W.SimCfg(), 0), (W.SimCfg(n_prefill=2, n_decode=7), 1),
+    (W.SimCfg(n_prefill=2, n_decode=2, kv_cap_tokens=16_000), 0),  # requests wait in the FIFO
+    (W.SimCfg(n_decode=1, pre_base_us=1, pre_us_per_tok=0), 0),  # heaps of more than 33 keys
+    (W.SimCfg(n_prefill=2, n_decode=2, kv_cap_tokens=16_000, cap_active=9, cap_waiting=8, cap_pending=8), 1)],
+    ids=["1p3d", "2p7d", "scarce", "deep", "small_caps"])
+def test_block_per_row(orc, lanes, sc, deployed, order):
+    tc = W.replica_sweep().trace.replace(rate_mreq=(8_000, 60_000), prompt_max=min(8192, sc.kv_cap_tokens // 2))
+    sets = [W.as_deployed(W.CALIBRATED) if deployed else W.CALIBRATED]
+    check(orc, lanes, sc, sets, ALL_FIVE, [orc.gen_trace(tc, 150)], order)
