@@ -1063,6 +1063,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                     ready = end + (int64_t)(int32_t)P.xfer_tok * (int32_t)pk;
                     err = ready >= kTimeLimit ? CTR_EOVERFLOW : push_prefill<kSig, kArity>(s, end, (uint32_t)pk, P, ring, oob);
                 }
+                if constexpr (kBat) __syncwarp();  // the decode lanes will read the ring entries stored here
                 ready = __shfl_sync(kFull, ready, ip, G);
                 if (live && gl == P.n_pre + id && ready < kTimeLimit && err == CTR_OK)
                     err = queue_decode<kArity>(s, T, k, ready, sum_is_o_hat ? ohk : ok, P, pend, wait, oob);

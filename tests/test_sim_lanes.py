@@ -43,3 +43,17 @@ def test_block_per_row(orc, lanes, sc, deployed, order):
     tc = W.replica_sweep().trace.replace(rate_mreq=(8_000, 60_000), prompt_max=min(8192, sc.kv_cap_tokens // 2))
     sets = [W.as_deployed(W.CALIBRATED) if deployed else W.CALIBRATED]
     check(orc, lanes, sc, sets, ALL_FIVE, [orc.gen_trace(tc, 150)], order)
+
+
+@pytest.mark.parametrize("order", [0, 1, 7])
+@pytest.mark.parametrize("sc,ws_rows", [
+    (W.SimCfg(prefill_batch_tokens=2048), None), (W.SimCfg(n_prefill=3, n_decode=5, prefill_batch_tokens=900), 1),
+    (W.SimCfg(n_prefill=2, n_decode=2, kv_cap_tokens=16_000, cap_active=9, cap_waiting=8, prefill_batch_tokens=4096), 1),
+    (W.SimCfg(n_prefill=2, n_decode=6), 1), (W.SimCfg(n_prefill=4, n_decode=13), None)],
+    ids=["batched", "batched_packed", "batched_small_caps", "packed", "4p13d"])
+def test_rows_in_warps(orc, lanes, sc, ws_rows, order):
+    """A row or (ws_rows=1: a workspace of one slot) several to a warp; with batched prefill the decode lanes read the
+    prefill lanes' rings."""
+    tc = W.replica_sweep().trace.replace(rate_mreq=(8_000, 60_000), prompt_max=min(8192, sc.kv_cap_tokens // 2))
+    sets = [W.CALIBRATED, W.as_deployed(W.CALIBRATED)]
+    check(orc, lanes, sc, sets, ALL_FIVE, [orc.gen_trace(tc, 90)], order, ws_rows=ws_rows)
