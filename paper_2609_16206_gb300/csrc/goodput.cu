@@ -409,10 +409,11 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
                 if (k[u] < n) request(k[u], a[u], o[u], c[u], f[u], d[u]);
         }
         auto add = [](int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); };  // mod 2^64
-        // met and (below it) the multi-token requests, both < 2^24, and the threads with a wide value
-        const int64_t sums = block_reduce<int64_t>(((int64_t)met << 40) + ((int64_t)many << 16) + wide, 0, add,
-                                                   S.red64);  // its barriers publish the kept values
-        many = (int32_t)(sums >> 16) & 0xffffff;
+        // met and (below it) the multi-token requests, both at most 2^23, and the threads with a wide value: 2^23 met
+        // requests are the top bit, so the word is read unsigned
+        const uint64_t sums = (uint64_t)block_reduce<int64_t>(((int64_t)met << 40) + ((int64_t)many << 16) + wide, 0, add,
+                                                              S.red64);  // its barriers publish the kept values
+        many = (int32_t)((sums >> 16) & 0xffffffu);
         const bool packs = (sums & 0xffff) == 0;
         if (kHash) {
             h = (uint64_t)block_reduce<int64_t>((int64_t)h, 0, add, S.red64);
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         const bool out = __syncthreads_or(bad);  // a row whose pass left a buffer: both outputs say so
 #endif
         if (tid == 0) {
-            P.met[row] = sums >> 40;
+            P.met[row] = (int64_t)(sums >> 40);
             P.p99[row] = p99;
             if (kTpot) P.p99_tpot[row] = p99_tpot;
 #if CTR_BOUNDS_CHECK

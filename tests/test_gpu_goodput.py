@@ -265,3 +265,35 @@ def test_block_size_and_sample_by_row_length(orc, rows, N):
         f, d = tf[r].cpu().numpy(), td[r].cpu().numpy()
         assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), row, f, d), r
         assert tpot[r] == orc.p99_tpot({"true_out": row["true_out"]}, f, d), r
+
+
+@pytest.mark.parametrize("N", [(1 << 23) - 1, 1 << 23])
+@pytest.mark.parametrize("slow", [0, 1])
+def test_longest_row_meeting_every_slo(N, slow):
+    """The longest rows the library takes, all or all but one of their requests within their SLOs: the met count uses
+    every bit it has; through ctr_goodput and (all o = 1) inside ctr_simulate."""
+    ctr = need_gpu()
+    k = torch.arange(N, device="cuda").view(1, N)
+    ttft = (k * 7919) % 999_983 + 1
+    o = (k % 5 + 1).int()
+    tr = {"arrival_us": k * 50, "prompt_len": torch.ones_like(o), "true_out": o, "pred_out": torch.ones_like(o),
+          "slo_class": (k % 2).to(torch.uint8)}
+    if slow:
+        ttft[0, N // 2] = 1 << 41
+    tf = tr["arrival_us"] + ttft
+    td = tf + (o - 1).long() * (k % 1000)
+    sc = W.SimCfg(ttft_slo_us=(1 << 40, 1 << 40), tpot_slo_us=(1 << 20, 1 << 20), pre_base_us=1, pre_us_per_tok=0,
+                  xfer_us_per_tok=0, dec_base_us=1, dec_us_per_seq=0, n_prefill=1, n_decode=1)
+    met, p99 = _goodput(ctr, sc, tr, 1, 1, N, tf, td)
+    tpot = _p99_tpot(ctr, sc, tr, 1, 1, N, tf, td)
+    assert met[0] == N - slow
+    assert p99[0] == int(ttft.view(-1).kthvalue((99 * N + 99) // 100).values)
+    many = ((td - tf) // (o - 1).clamp(min=1))[o >= 2]
+    assert tpot[0] == int(many.kthvalue((99 * many.numel() + 99) // 100).values)
+    if slow == 0 and N == 1 << 23:
+        tr["true_out"] = torch.ones_like(o)
+        out = [torch.full((1,), -5, dtype=torch.int64, device="cuda") for _ in range(3)]
+        st = torch.full((1,), -5, dtype=torch.int32, device="cuda")
+        ctr.ctr_simulate(sc, [W.CALIBRATED], [W.POLICY_RR], tr, 1, N, tf, td, out[0], st,
+                         ctr.simulate_workspace(sc, 1, N, "cuda"), met_count=out[1], p99_ttft_us=out[2])
+        assert (int(st), int(out[1])) == (0, N)
