@@ -1113,7 +1113,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
 // instances' costs go through shared memory, one barrier, and each warp takes
 // both argmins itself; the ends of all prefill queues ride along in every warp
 // (lane i that of instance i), so the KV-ready time needs no second exchange and
-// a round-robin row needs no barrier at all.  Without batched prefill.
+// a round-robin row needs no barrier until its end.  Without batched prefill.
 // Bound by its longest chain an arrival: about 3,600 cycles for the learned
 // router; of 4,100 on an earlier source 2,500 were one instance's event, 800 its
 // price and 600 the commit (cycle counters around each, 2P+6D).
@@ -1164,6 +1164,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
         int ip = P.n_pre - 1, id = P.n_dec - 1;
         uint64_t h = 0;
         int err = CTR_OK;
+        uint32_t failed_by = CTR_MAX_REQUESTS;  // round robin: the request by whose routing this instance had failed
         bool go = valid;  // the same in every thread of the block
         for (int64_t base = 0; go && base < n; base += 32) {
             const int64_t kl = base + lane;
@@ -1201,6 +1202,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
                 }
                 // 2. the costs of all instances and the argmin of each pool
                 if (pol == CTR_POLICY_ROUND_ROBIN) {
+                    if (err != CTR_OK && failed_by == CTR_MAX_REQUESTS) failed_by = (uint32_t)k;
                     ip = ip + 1 == P.n_pre ? 0 : ip + 1;
                     id = id + 1 == P.n_dec ? 0 : id + 1;
                 } else {
@@ -1223,7 +1225,7 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
                 const int64_t end = prefill_end(P, __shfl_sync(kFull, busy, ip), T, pk);
                 const int64_t ready = end + (int64_t)(int32_t)P.xfer_tok * (int32_t)pk;
                 if (ready >= kTimeLimit) {  // the same in every warp
-                    err = CTR_EOVERFLOW;
+                    if (err == CTR_OK) err = CTR_EOVERFLOW;
                     go = false;
                     break;
                 }
@@ -1247,9 +1249,14 @@ __global__ void __launch_bounds__(kWarps * 32, 16 / kWarps) sim_row_kernel(const
 
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) h += __shfl_xor_sync(kFull, h, off);
-        int status = CTR_OK;
-        if (__syncthreads_or(err == CTR_ETIMEOUT)) status = CTR_ETIMEOUT;
-        if (__syncthreads_or(err == CTR_EOVERFLOW)) status = CTR_EOVERFLOW;
+        // The row's status is that of its first failure.  Costs that are exchanged end a row there, an overflow of the
+        // commit before or of the same advance counting before a timeout; the warps of a round-robin row, which exchange
+        // nothing, ran on, so the earliest of theirs is looked for.
+        __syncthreads();  // the last costs have been read
+        if (lane == 0) cost_s[0][w] = err == CTR_OK ? ~0u : 2 * failed_by + (err == CTR_ETIMEOUT);
+        __syncthreads();  // (the next row's check has a barrier before its first cost)
+        const uint32_t first = __reduce_min_sync(kFull, lane < n_inst ? (uint32_t)cost_s[0][lane] : ~0u);
+        int status = first == ~0u ? CTR_OK : (first & 1u) != 0 ? CTR_ETIMEOUT : CTR_EOVERFLOW;
         if (!valid) status = CTR_EINVAL;
 #if CTR_BOUNDS_CHECK
         if (__syncthreads_or(oob)) status = CTR_EBOUNDS;

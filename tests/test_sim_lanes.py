@@ -57,3 +57,23 @@ def test_rows_in_warps(orc, lanes, sc, ws_rows, order):
     tc = W.replica_sweep().trace.replace(rate_mreq=(8_000, 60_000), prompt_max=min(8192, sc.kv_cap_tokens // 2))
     sets = [W.CALIBRATED, W.as_deployed(W.CALIBRATED)]
     check(orc, lanes, sc, sets, ALL_FIVE, [orc.gen_trace(tc, 90)], order, ws_rows=ws_rows)
+
+
+def _two_failures(max_steps, burst_at=40):
+    """Round robin on two decode instances: the even requests run instance 0 out of its steps, then a burst at one
+    instant has more requests pending than either instance may hold."""
+    k = np.arange(burst_at + 20)
+    tr = {"arrival_us": np.minimum(k, burst_at) * 10_000, "prompt_len": np.full(k.size, 10), "true_out": np.where(k % 2, 1, 8),
+          "pred_out": np.full(k.size, 4), "slo_class": k % 2}
+    return W.SimCfg(n_prefill=1, n_decode=2, pre_base_us=100, pre_us_per_tok=0, xfer_us_per_tok=1, dec_base_us=1_000,
+                    cap_pending=4, max_steps_per_instance=max_steps), tr
+
+
+@pytest.mark.parametrize("max_steps,status", [(100, -4), (152, -4), (153, -4), (161, -3), (1 << 20, -3)])
+@pytest.mark.parametrize("ws_rows", [None, 1])
+def test_first_failure_is_the_rows(orc, lanes, max_steps, status, ws_rows):
+    """A row's status is that of its first failure, in a block per row (where round-robin warps do not meet) as in a
+    warp."""
+    sc, tr = _two_failures(max_steps)
+    res = check(orc, lanes, sc, [W.CALIBRATED], [W.POLICY_RR] * 3 + [W.POLICY_JSQ] * 2, [tr] * 4, 0, ws_rows=ws_rows)
+    assert (res["status"].reshape(4, 5)[:, :3] == status).all()
