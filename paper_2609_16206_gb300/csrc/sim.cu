@@ -385,8 +385,8 @@ struct RowView {
 
 // A decode lane's state.  Its next event is the end of a step at which
 // something can change (a completion, an admission, the floor(KV / kv_div) term
-// of the step time), and the steps before it are a run of equal ones, left as
-// they are until the event: the running step ends at step_end, `run` more of
+// of the step time) or fail (the FIFO, the step budget), and the steps before it
+// are a run of equal ones, left as they are until the event: the running step ends at step_end, `run` more of
 // `step` us follow, and the event is at step_end + run * step.  An idle lane
 // (n_act = 0) has run = 0 and step_end the time of its next KV-ready request
 // (kIdle without one).  run * step stays below 2^31, so a time inside the run
@@ -442,15 +442,19 @@ __device__ __forceinline__ void cut_run(Decode& s, int64_t tp, bool when)
 }
 
 // A new key of the pending heap (ready at key >> 23).  While requests wait for
-// admission (w_n > 0) the next event does not depend on it: either the head
-// waits for a completion, or an event no later than this one is set already.
+// admission (w_n > 0) the next event does not depend on it -- either the head
+// waits for a completion, or an event no later than this one is set already --
+// unless it could overflow the FIFO, which counts from the step end at which it does.
 template <int kArity>
-__device__ __forceinline__ void push_pending(Decode& s, uint64_t* pend, uint64_t key, int64_t lim, bool& bad)
+__device__ __forceinline__ void push_pending(Decode& s, uint64_t* pend, uint64_t key, const SimParams& P, int64_t lim,
+                                             bool& bad)
 {
     hpush<kArity>(pend, s.pend_n, s.pend_top, key, lim, bad);
     const int64_t tp = (int64_t)(key >> kKeyBits);
     s.step_end = (s.n_act == 0) & (tp < s.step_end) ? tp : s.step_end;  // an idle instance's next event
-    cut_run(s, tp, s.w_n == 0);
+    bool cut = s.w_n == 0;
+    if (!cut) cut = s.w_n + s.pend_n > P.cap_wait;
+    cut_run(s, tp, cut);
 }
 
 // Move every pending request whose KV is ready by t into the waiting FIFO, in
@@ -510,6 +514,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     const uint64_t by = (uint64_t)(tev + 1) << kKeyBits;  // as in flush_ready
     int32_t room = P.cap_wait - s.w_n;
     int32_t admitted = 0;
+    bool hold = false;  // the FIFO's head waits, and no further request can overflow the FIFO (see push_pending)
     uint32_t last = 0;  // the request admitted last; the others are chained through their t_first entries
     for (;;) {
         const bool fifo = s.w_n > 0;
@@ -521,6 +526,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
             if (fits) return CTR_EOVERFLOW;
             const int rc = flush_ready<kArity>(s, tev, room, P, pend, wait, bad);
             if (rc != CTR_OK) return rc;
+            hold = s.w_n + s.pend_n <= P.cap_wait;
             break;
         }
         if (fifo) {
@@ -539,10 +545,11 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
         admitted += 1;
     }
     // (3) the next step and the next event
-    // the FIFO's room, the steps started on this instance, the time (its limit's low word is 0)
+    // the FIFO's room, the steps started on this instance, the time (its limit's low word is 0): a step that ended too
+    // late was started within the budget
     if (room < 0 || s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps ||
         (int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32))
-        return s.step_idx + (s.n_act > 0) > (int32_t)P.max_steps ? CTR_ETIMEOUT : CTR_EOVERFLOW;
+        return room < 0 || (int32_t)(tev >> 32) >= (int32_t)(kTimeLimit >> 32) ? CTR_EOVERFLOW : CTR_ETIMEOUT;
     const int64_t tp = (int64_t)(s.pend_top >> kKeyBits);  // kIdle when empty
     const int32_t n = s.n_act;
     const bool idle = n == 0;  // then what follows computes nothing that is kept
@@ -561,7 +568,9 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     // (q1 + 1 <= 2^31 and kv_div <= 2^31; the sum is below 2^32)
     const int32_t q1 = kv_term(s.kv_res + n, P);
     const uint32_t room1 = (uint32_t)(q1 + 1) * (uint32_t)P.kv_div - 1u - (uint32_t)s.kv_res;
-    int32_t m = (int32_t)(s.act_top >> kKeyBits) - s.step_idx - 1;  // plain ends before the next completion, <= 2^20
+    // plain ends before the next completion or the end of the step budget, <= 2^20
+    const int32_t fin = (int32_t)(s.act_top >> kKeyBits);
+    int32_t m = (fin < (int32_t)P.max_steps ? fin : (int32_t)P.max_steps) - s.step_idx - 1;
     // the steps before the term changes, room1 / n (or one less): the estimate is within one where it is below m
     int32_t before = __float2int_rz(__uint2float_rn(room1) * recip_estimate(n));
     before -= (uint32_t)before * (uint32_t)n > room1;  // room1 < kv_div + n, so a product that matters fits
@@ -569,7 +578,7 @@ __device__ __forceinline__ int decode_event(Decode& s, int64_t tev, const SimPar
     s.step = (int32_t)P.dec_base + (int32_t)P.dec_seq * n + q1;  // run_max = 0 where a step could reach 2^31 us
     s.inv_step = recip_estimate(s.step);
     s.run = idle ? 0 : m < P.run_max ? m : P.run_max;
-    cut_run(s, tp, s.w_n == 0);
+    cut_run(s, tp, !hold);
     return CTR_OK;
 }
 
@@ -749,7 +758,7 @@ __device__ __forceinline__ int queue_decode(Decode& s, int64_t T, int64_t k, int
     }
     if (kBat && ready >= 0 && s.pend_n == P.cap_pend_store) return CTR_EOVERFLOW;
     if (!kBat || ready >= 0)
-        push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, heap_stride(P.cap_pr), bad);
+        push_pending<kArity>(s, pend, ((uint64_t)ready << kKeyBits) | (uint64_t)k, P, heap_stride(P.cap_pr), bad);
     if constexpr (kBat) s.q += 1;
     s.sum += weight;
     return CTR_OK;
@@ -951,7 +960,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocksPerSM) sim_kernel(
                                 } else {
                                     push_pending<kArity>(s, pend,
                                                          ((uint64_t)ready << kKeyBits) | (uint64_t)(v >> kRingKShift),
-                                                         pr_stride, oob);
+                                                         P, pr_stride, oob);
                                 }
                             }
                             pos = pos + 1 == P.cap_ring ? 0 : pos + 1;

@@ -137,8 +137,11 @@ def test_rows_per_warp_same_results(orc, sc, R, deployed):
 @pytest.mark.parametrize("sc", [W.SimCfg(), W.SimCfg(n_prefill=2, n_decode=6), W.SimCfg(n_prefill=1, n_decode=8),
                                 W.SimCfg(n_prefill=4, n_decode=12), W.SimCfg(n_prefill=4, n_decode=13),
                                 W.SimCfg(n_prefill=2, n_decode=6, kv_cap_tokens=9_000),
-                                W.SimCfg(n_prefill=2, n_decode=6, cap_active=9, cap_waiting=8, cap_pending=8)],
-                         ids=["1p3d", "2p6d", "1p8d", "4p12d", "4p13d", "scarce", "small_caps"])
+                                W.SimCfg(n_prefill=2, n_decode=6, cap_active=9, cap_waiting=8, cap_pending=8),
+                                W.SimCfg(n_prefill=2, n_decode=6, max_steps_per_instance=900, cap_pending=12),
+                                W.SimCfg(n_prefill=2, n_decode=6, max_steps_per_instance=900, kv_cap_tokens=9_000, cap_waiting=3)],
+                         ids=["1p3d", "2p6d", "1p8d", "4p12d", "4p13d", "scarce", "small_caps", "budget_or_pending",
+                              "budget_or_fifo"])
 @pytest.mark.parametrize("deployed", [0, 1])
 def test_row_per_block_same_rows(orc, sc, deployed):
     """The same replicas in a launch of few rows (a block per row, up to 16 instances) and in one of many (rows in

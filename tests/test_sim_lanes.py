@@ -77,3 +77,39 @@ def test_first_failure_is_the_rows(orc, lanes, max_steps, status, ws_rows):
     sc, tr = _two_failures(max_steps)
     res = check(orc, lanes, sc, [W.CALIBRATED], [W.POLICY_RR] * 3 + [W.POLICY_JSQ] * 2, [tr] * 4, 0, ws_rows=ws_rows)
     assert (res["status"].reshape(4, 5)[:, :3] == status).all()
+
+
+def _trace(rows):
+    """(arrival, prompt, output) per request."""
+    a = np.array(rows).T
+    return {"arrival_us": a[0], "prompt_len": a[1], "true_out": a[2], "pred_out": a[2] % 512, "slo_class": a[0] * 0}
+
+
+# two decode instances in turns, 1 ms steps; every request KV-ready at once
+_BASE = W.SimCfg(n_prefill=1, n_decode=2, pre_base_us=1, pre_us_per_tok=0, xfer_us_per_tok=0, dec_base_us=1_000,
+                 dec_us_per_seq=0, dec_kv_tokens_per_us=1 << 31, kv_cap_tokens=5_000)
+
+
+@pytest.mark.parametrize("name,sc,rows,status", [
+    # instance 0 runs out of steps in the middle of a long run, then a burst overflows the pending heap of instance 1
+    ("budget_in_a_run", _BASE.replace(max_steps_per_instance=50, cap_pending=3, pre_base_us=500),
+     [(0, 1, 2000), (0, 1, 1)] + [(200_000, 1, 1)] * 12, -4),
+    # instance 0's FIFO overflows behind a request that fills its KV, long before instance 1 runs out of steps
+    ("fifo_behind_its_head", _BASE.replace(max_steps_per_instance=900, cap_waiting=2),
+     [(0, 1, 4500), (0, 1, 2000)] + [(10_000 + 1000 * k, 1, 800 if k % 2 == 0 else 1) for k in range(12)] +
+     [(3_000_000, 1, 1)], -3),
+    # the same FIFO, filled to its last place: instance 0 runs out of steps
+    ("fifo_full", _BASE.replace(max_steps_per_instance=900, cap_waiting=6),
+     [(0, 1, 4500), (0, 1, 2000)] + [(10_000 + 1000 * k, 1, 800 if k % 2 == 0 else 1) for k in range(12)] +
+     [(3_000_000, 1, 1)], -4),
+    # a FIFO overflow at the very step end at which the budget is used up
+    ("both_at_one_step_end", _BASE.replace(max_steps_per_instance=40, cap_waiting=3),
+     [(0, 1, 40), (0, 1, 1)] + [(39_500, 1, 30), (39_500, 1, 1)] * 4, -3)], ids=lambda v: v if isinstance(v, str) else "")
+@pytest.mark.parametrize("ws_rows", [None, 1])
+def test_failure_inside_a_run_of_steps(orc, lanes, name, sc, rows, status, ws_rows):
+    """What fails between two events of an instance fails before what another instance does later."""
+    tr = _trace(rows)
+    res = check(orc, lanes, sc, [W.CALIBRATED], [W.POLICY_RR] * 5, [tr] * 2, 0, ws_rows=ws_rows)
+    assert (res["status"] == status).all(), res["status"]
+    sc = sc.replace(prefill_batch_tokens=1)
+    check(orc, lanes, sc, [W.CALIBRATED], [W.POLICY_RR, W.POLICY_LEARNED], [tr], 0, ws_rows=ws_rows)
