@@ -10,10 +10,10 @@
 // then keeps those that do: per request the trace's arrival, output length and
 // class and the row's t_first and t_done.  The P99 is the value of the remaining
 // rank among the kept ones: their histogram over the same bins finds its bin,
-// whose few members are counted out.  A row whose kept values are fewer than the
-// rank needs or more than there is room for (thousands of equal values at the
-// P99), or of 2^32 and more, takes an exact radix select over all its values read
-// from global memory (10-bit digits, most significant first).  A TPOT is compared
+// whose members are counted out or, if many, selected by their digits.  A row
+// whose kept values are fewer than the rank needs or more than there is room for
+// (thousands of equal values at the P99), or of 2^32 and more, takes an exact
+// radix select over all its values read from global memory (row_rank).  A TPOT is compared
 // without a division (floor(d / m) >= t is d >= t m) and divided only when kept,
 // after the pass where there is room for the divisors: in the pass the few lanes
 // that keep one would make their whole warp divide.
@@ -34,6 +34,7 @@ constexpr int kMaxCand = 8192;  // most values kept
 constexpr int kFew = 128;       // members of the rank's bin counted out directly
 constexpr int kDigit = 10;      // radix select
 constexpr int kBins = 1 << kDigit;
+constexpr int kSubBins = 256;   // parts of a crowded bin (see finer_threshold)
 static_assert(kBins <= kHistWords, "the radix select takes the place of a 16-bit histogram");
 
 // Monotone bin of a value in [0, 2^32): the exponent and the top 6 mantissa bits
@@ -137,75 +138,206 @@ __device__ __forceinline__ uint32_t at16(const uint32_t* h, int b) { return (h[b
 #define CTR_CK_FLAG_ARG
 #endif
 
-// Exact radix select: the value of 0-based rank `rank` among those of
-// val(k, v) over k < n (false: k has none).  Block-collective; every thread
-// returns it.
-template <typename Val>
-__device__ int64_t radix_rank(const Val& val, int64_t n, int64_t rank, uint32_t* hist, SelScratch& S CTR_CK_FLAG_PARAM)
+// use(v) for each value of src over k < n, a few loaded before any is made up
+template <typename Src, typename Use>
+__device__ __forceinline__ void for_each_value(const Src& src, int64_t n, const Use& use)
+{
+    constexpr int kBatch = 4;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int64_t k0 = tid; k0 < n; k0 += kBatch * nt) {
+        typename Src::Raw raw[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) raw[u] = src.load(k0 + u * nt < n ? k0 + u * nt : k0);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            int64_t v;
+            if (k0 + u * nt < n && src.value(raw[u], v)) use(v);
+        }
+    }
+}
+
+// Exact radix select: the value of 0-based rank `rank` among those of src that lie in [lo, lo + 2^bits), all of which
+// fit in it when bits is 64 (10-bit digits, most significant first).  Block-collective; every thread returns it.
+template <typename Src>
+__device__ int64_t radix_rank(const Src& src, int64_t n, int64_t rank, int64_t lo, int bits, uint32_t* hist,
+                              SelScratch& S CTR_CK_FLAG_PARAM)
 {
 #if !CTR_BOUNDS_CHECK
     bool bad = false;  // dead: the accessors below compile to plain accesses
 #endif
     const int tid = threadIdx.x, nt = blockDim.x;
-    int64_t mn = INT64_MAX, mx = INT64_MIN;
-    for (int64_t k = tid; k < n; k += nt) {
-        int64_t v;
-        if (val(k, v)) {
-            mn = v < mn ? v : mn;
-            mx = v > mx ? v : mx;
-        }
-    }
-    mn = block_reduce<int64_t>(mn, INT64_MAX, [](int64_t a, int64_t b) { return a < b ? a : b; }, S.red64);
-    mx = block_reduce<int64_t>(mx, INT64_MIN, [](int64_t a, int64_t b) { return a > b ? a : b; }, S.red64);
-    const uint64_t range = (uint64_t)mx - (uint64_t)mn;
-    int shift = range == 0 ? 0 : 64 - __clzll((long long)range);  // bits still undetermined
-    uint64_t prefix = 0;                                            // chosen high bits of (value - mn)
-    while (shift > 0) {
+    uint64_t prefix = 0;  // chosen high bits of (value - lo)
+    for (int shift = bits; shift > 0;) {
         const int dbits = shift < kDigit ? shift : kDigit;
         const int above = shift;  // candidates agree with prefix on bits >= above
         shift -= dbits;
         for (int i = tid; i < kBins; i += nt) hist[i] = 0;
         __syncthreads();
         const uint32_t dmask = (1u << dbits) - 1u;
-        for (int64_t k = tid; k < n; k += nt) {
-            int64_t tv;
-            if (!val(k, tv)) continue;
-            const uint64_t v = (uint64_t)tv - (uint64_t)mn;
+        for_each_value(src, n, [&](int64_t tv) {
+            const uint64_t v = (uint64_t)tv - (uint64_t)lo;
             const bool match = above >= 64 || (v >> above) == (prefix >> above);
             if (match) {
                 const uint32_t b = (uint32_t)(v >> shift) & dmask;
                 if (ck_ok(b, kBins, bad)) atomicAdd(&hist[b], 1u);
             }
-        }
+        });
         __syncthreads();
         find_rank_bin([&](int b) { return hist[b]; }, kBins, rank, S.pick, S.wsum);
         prefix |= (uint64_t)S.pick[0] << shift;
         rank -= S.pick[1];
         __syncthreads();
     }
-    return (int64_t)((uint64_t)mn + prefix);
+    return (int64_t)((uint64_t)lo + prefix);
+}
+__device__ __forceinline__ int bits_of(uint64_t range) { return range == 0 ? 0 : 64 - __clzll((long long)range); }
+
+// (t_done - t_first) / (o - 1) of o >= 2 tokens, toward zero: 32-bit where it may be
+__device__ __forceinline__ int64_t tpot_value(int64_t dec, int32_t o)
+{
+    return (uint64_t)dec < (uint64_t(1) << 32) ? (int64_t)((uint32_t)dec / (uint32_t)(o - 1)) : dec / (int64_t)(o - 1);
+}
+
+// A row's values in memory: x - y, or with kTpot (x - y) / (o - 1) where o >= 2.
+template <bool kTpot>
+struct RowValues {
+    const int64_t *x, *y;
+    const int32_t* o;
+    int64_t n;
+    bool& bad;
+    struct Raw {
+        int64_t d;
+        int32_t o;
+    };
+    __device__ __forceinline__ Raw load(int64_t k) const
+    {
+        return {ck_ldg(x, k, n, bad) - ck_ldg(y, k, n, bad), kTpot ? ck_ldg(o, k, n, bad) : 2};
+    }
+    __device__ __forceinline__ bool value(const Raw& r, int64_t& v) const
+    {
+        v = r.d;
+        if (kTpot && r.o >= 2) v = tpot_value(r.d, r.o);
+        return !kTpot || r.o >= 2;
+    }
+};
+// Kept values.
+struct KeptValues {
+    const uint32_t* cand;
+    using Raw = uint32_t;
+    __device__ __forceinline__ Raw load(int64_t k) const { return cand[k]; }
+    __device__ __forceinline__ bool value(Raw r, int64_t& v) const
+    {
+        v = r;
+        return true;
+    }
+};
+
+// The value of rank `rank` among all of a row.  A first count over logarithmic bins, 32 per octave, leaves a range whose
+// digits the radix select takes (10,000 TPOTs near 15 ms: two passes over memory in all, TTFTs near 1 s: three); a rank
+// among values below 1 or from 2^32 on starts from the least and the greatest value.  Block-collective.
+template <bool kTpot>
+__device__ __noinline__ int64_t row_rank(const int64_t* x, const int64_t* y, const int32_t* o, int64_t n, int64_t rank,
+                                         uint32_t* hist, SelScratch& S CTR_CK_FLAG_PARAM)
+{
+#if !CTR_BOUNDS_CHECK
+    bool bad = false;
+#endif
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const RowValues<kTpot> src = {x, y, o, n, bad};
+    for (int i = tid; i < kHistWords; i += nt) hist[i] = 0;
+    __syncthreads();
+    for_each_value(src, n, [&](int64_t v) {
+        const uint32_t b = log_bin(v) >> 1;
+        if (ck_ok(b, kHistWords, bad)) atomicAdd(&hist[b], 1u);
+    });
+    __syncthreads();
+    find_rank_bin([&](int b) { return hist[b]; }, kHistWords, rank, S.pick, S.wsum);
+    const int b = (int)S.pick[0];
+    const int64_t before = (int64_t)S.pick[1];
+    __syncthreads();
+    if (b > 0 && b < kHistWords - 1) {
+        const int64_t lo = bin_floor(2 * b);
+        return radix_rank(src, n, rank - before, lo, bits_of((uint64_t)(bin_floor(2 * b + 2) - lo - 1)), hist, S CTR_CK_FLAG_ARG);
+    }
+    int64_t mn = INT64_MAX, mx = INT64_MIN;
+    for_each_value(src, n, [&](int64_t v) {
+        mn = v < mn ? v : mn;
+        mx = v > mx ? v : mx;
+    });
+    mn = block_reduce<int64_t>(mn, INT64_MAX, [](int64_t a, int64_t b) { return a < b ? a : b; }, S.red64);
+    mx = block_reduce<int64_t>(mx, INT64_MIN, [](int64_t a, int64_t b) { return a > b ? a : b; }, S.red64);
+    return radix_rank(src, n, rank, mn, bits_of((uint64_t)mx - (uint64_t)mn), hist, S CTR_CK_FLAG_ARG);
 }
 
 // the nearest rank of the P99 among m values, 0-based
 __device__ __forceinline__ int64_t p99_rank(int64_t m) { return (99 * m + 99) / 100 - 1; }
 
+// The request of sample i: all of a row of up to 2^log2, else evenly spaced groups of four neighbours.
+__device__ __forceinline__ int64_t sample_at(int i, int64_t n, int log2)
+{
+    return n <= (int64_t(1) << log2) ? i : ((((int64_t)(i >> 2) * n) >> (log2 - 2)) & ~int64_t(3)) + (i & 3);
+}
+// The sampled TTFTs, read again (they are in the L2); the sampled TPOTs, whose division is not repeated, are kept.
+struct SampledTtfts {
+    RowValues<false> row;
+    int log2;
+    using Raw = RowValues<false>::Raw;
+    __device__ __forceinline__ Raw load(int64_t i) const { return row.load(sample_at((int)i, row.n, log2)); }
+    __device__ __forceinline__ bool value(const Raw& r, int64_t& v) const { return row.value(r, v); }
+};
+
+// Within bin B (neither the first nor the last), which holds in_bin of src's `taken` samples, the floor of the part that
+// holds their want-th largest, by the next 8 bits; the floor of the part above where that leaves more than `most` of
+// them.  Block-collective.
+template <typename Src>
+__device__ __noinline__ int64_t finer_threshold(const Src src, int taken, uint32_t B, int32_t in_bin, int32_t want,
+                                                int32_t most, uint32_t* hist, SelScratch& S CTR_CK_FLAG_PARAM)
+{
+#if !CTR_BOUNDS_CHECK
+    bool bad = false;
+#endif
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int i = tid; i < kSubBins; i += nt) hist[i] = 0;
+    __syncthreads();
+    for_each_value(src, taken, [&](int64_t v) {
+        if (log_bin(v) != B) return;
+        const uint32_t sub = (__float_as_uint(__uint2float_rz((uint32_t)v)) >> 9) & (kSubBins - 1);
+        if (ck_ok(sub, kSubBins, bad)) atomicAdd(&hist[sub], 1u);
+    });
+    __syncthreads();
+    find_rank_bin([&](int b) { return hist[b]; }, kSubBins, want < in_bin ? in_bin - want : 0, S.pick, S.wsum);
+    uint32_t bits = ((B + (126u << 6)) << 17) + (S.pick[0] << 9);
+    if (in_bin - (int32_t)S.pick[1] > most) bits += 1u << 9;
+    __syncthreads();  // pick and wsum are free again
+    return (int64_t)ceilf(__uint_as_float(bits));
+}
+
 // A threshold that at least the top m - p99_rank(m) of about m values reach, from the histogram of `taken`
 // samples of them: the floor of the bin of the sample's j-th largest, j six standard deviations above the
-// expected count (neighbours are alike; exactly the count when every value is in the sample).
-// Block-collective.
-__device__ int64_t threshold(const uint32_t* hist, int64_t taken, int64_t m, SelScratch& S)
+// expected count (neighbours are alike; exactly the count when every value is in the sample).  Where that bin holds so
+// many that the kept values could outgrow their room (a fifth of a row's TPOTs may lie within 1 %), a finer one: of 352
+// simulated rows of 10,000 and 40,000 none needs the radix select with this at 0.6 of the room, five do at 0.9 and 170
+// without.  Equal values that are still too many are left out, as the radix select would be sure with them.  src: n_src
+// values, the samples among them.  Block-collective.
+template <typename Src>
+__device__ __forceinline__ int64_t threshold(uint32_t* hist, int32_t taken, int64_t m, uint32_t room, const Src& src, int n_src,
+                                             SelScratch& S CTR_CK_FLAG_PARAM)
 {
     if (taken <= 0) return INT64_MAX;
     const int64_t top = m - p99_rank(m);
-    int64_t j = top;
+    int32_t j = (int32_t)top;
     if (taken < m) {
         const float e = (float)taken * ((float)top / (float)m);
-        j = (int64_t)(e + 6.0f * sqrtf(e)) + 2;
+        j = (int32_t)(e + 6.0f * sqrtf(e)) + 2;
     }
     find_rank_bin([&](int b) { return at16(hist, b); }, kLogBins, j < taken ? taken - j : 0, S.pick, S.wsum);
-    const int64_t t = bin_floor(S.pick[0]);
-    __syncthreads();  // pick and wsum are free again
-    return t;
+    const uint32_t B = S.pick[0];
+    const int32_t reach = taken - (int32_t)S.pick[1], in_bin = (int32_t)at16(hist, (int)B);
+    __syncthreads();  // pick and wsum are free again, and hist is
+    if (10 * reach * m <= 6 * (int64_t)taken * room || B == 0 || B == kLogBins - 1) return bin_floor(B);
+    const int32_t above = reach - in_bin;
+    return finer_threshold<Src>(src, n_src, B, in_bin, j - above, (int32_t)(9 * (int64_t)taken * room / (10 * m)) - above, hist,
+                                S CTR_CK_FLAG_ARG);
 }
 
 // entries i and i + 1 as one load (bounds-checked builds also check its alignment)
@@ -247,8 +379,9 @@ __device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t
     __syncthreads();
     const int m = (int)S.n_few;
     if (m > kFew) {
-        auto val = [&](int64_t i, int64_t& v) { v = cand[i]; return true; };
-        return radix_rank(val, c, rank, hist, S CTR_CK_FLAG_ARG);
+        const int64_t lo = B == 0 ? 0 : bin_floor(B);
+        return radix_rank(KeptValues{cand}, c, r_in, lo, B == 0 ? 0 : bits_of((uint64_t)(bin_floor(B + 1) - lo - 1)), hist,
+                          S CTR_CK_FLAG_ARG);
     }
     for (int i = tid; i < m; i += nt) {  // the member whose position in (value, slot) order is the rank
         const uint32_t v = S.few[i];
@@ -265,9 +398,13 @@ __device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t
 // Bound by the pass: about 110 warp-instructions for 32 requests (64-bit times,
 // the SLO tables, one kept value in 30) and the bytes in flight.  Eight blocks
 // of 128 threads an SM overlap one row's sample and selection with the others'
-// passes.  4,096 rows x 20,000: 459 us with the P99 TPOT, 322 us without; 873 and
+// passes.  4,096 rows x 20,000: 445 us with the P99 TPOT, 305 us without; 873 and
 // 400 us when every request's logarithmic bin was counted and staged in shared
-// memory and the TPOT took two more passes of its own.
+// memory and the TPOT took two more passes of its own.  Those TPOTs are spread out;
+// 2,048 simulated rows x 10,000, whose TPOTs crowd within a few percent, take 139 to
+// 154 us with the P99 TPOT (mixed lengths, loads 0.1 to 0.85; 262 to 395 with the two
+// passes, 403 to 575 while crowded bins outgrew the room of the kept values), and 383
+// where most rows have thousands of equal times (502 with the two passes).
 template <bool kHash, bool kTpot, bool kLater>
 __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputParams P)
 {
@@ -275,7 +412,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
     __shared__ SelScratch S;
     __shared__ uint32_t n_cand[2];
     // kept TTFTs, then TPOTs (with kLater decode times, then output lengths less 1), cap each; before the pass the
-    // TPOTs' histogram.  Little shared memory leaves the pass more L1 for its loads in flight.
+    // TPOTs' histogram, then the sampled TPOTs.  Little shared memory leaves the pass more L1 for its loads in flight.
     extern __shared__ uint32_t cand_s[];
     uint32_t* const hist[2] = {hist_s, cand_s};
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -295,6 +432,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
         if (tid < 2) n_cand[tid] = 0;
         const int sample = 1 << P.sample_log2;
         const int taken = n < sample ? (int)n : sample;
+        uint32_t* const tpot_s = cand_s + kHistWords;
         int32_t taken_many = 0;
         __syncthreads();
         constexpr int kBatch = 4;  // samples a thread loads before it uses any
@@ -304,7 +442,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 const int i = i0 + j * nt < taken ? i0 + j * nt : i0;
-                const int64_t k = n <= sample ? i : ((((int64_t)(i >> 2) * n) >> (P.sample_log2 - 2)) & ~int64_t(3)) + (i & 3);
+                const int64_t k = sample_at(i, n, P.sample_log2);
                 const int64_t tf = ck_ldg(P.t_first, ob + k, out_len, bad);
                 ttft[j] = tf - ck_ldg(P.trace.arrival_us, tb + k, trace_len, bad);
                 if (kTpot) {
@@ -316,11 +454,14 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
             for (int j = 0; j < kBatch; ++j) {
                 if (i0 + j * nt >= taken) continue;
                 count16(hist[0], log_bin(ttft[j]), bad);
-                if (kTpot && o[j] >= 2) {
-                    ++taken_many;
-                    count16(hist[1], log_bin((uint64_t)dec[j] < (uint64_t(1) << 32)
-                                                 ? (int64_t)((uint32_t)dec[j] / (uint32_t)(o[j] - 1))
-                                                 : dec[j] / (o[j] - 1)), bad);
+                if (kTpot) {
+                    const int64_t v = o[j] >= 2 ? tpot_value(dec[j], o[j]) : 0;
+                    // (in the first and the last bin, which have no finer threshold, values may be cut and others be among them)
+                    ck_st(tpot_s, i0 + j * nt, sample, v <= 0 ? 0u : v >> 32 ? ~0u : (uint32_t)v, bad);
+                    if (o[j] >= 2) {
+                        ++taken_many;
+                        count16(hist[1], log_bin(v), bad);
+                    }
                 }
             }
         }
@@ -328,10 +469,13 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
                                                       reinterpret_cast<int32_t*>(S.red64));
         else
             __syncthreads();
-        const int64_t t_ttft = threshold(hist[0], taken, n, S);
+        const SampledTtfts again = {{P.t_first + ob, P.trace.arrival_us + tb, nullptr, n, bad}, P.sample_log2};
+        const int64_t t_ttft = threshold(hist[0], taken, n, cap, again, taken, S CTR_CK_FLAG_ARG);
         uint32_t t_tpot = 0;  // 0: none
         if (kTpot && taken_many > 0) {
-            const int64_t t = threshold(hist[1], taken_many, n <= sample ? taken_many : ((int64_t)taken_many * n) >> P.sample_log2, S);
+            const int64_t t = threshold(hist[1], taken_many,
+                                        n <= sample ? taken_many : ((int64_t)taken_many * n) >> P.sample_log2, cap,
+                                        KeptValues{tpot_s}, taken, S CTR_CK_FLAG_ARG);
             t_tpot = t > 0 ? (uint32_t)t : 0;  // below 2^32
         }
 
@@ -427,11 +571,7 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
             if (n_cand[0] <= cap && rank >= below && packs) {
                 p99 = kept_rank(cand_s, (int)n_cand[0], rank - below, hist[0], S CTR_CK_FLAG_ARG);
             } else {
-                auto ttft_of = [&](int64_t k, int64_t& v) {
-                    v = ck_ld(P.t_first, ob + k, out_len, bad) - ck_ld(P.trace.arrival_us, tb + k, trace_len, bad);
-                    return true;
-                };
-                p99 = radix_rank(ttft_of, n, rank, hist[0], S CTR_CK_FLAG_ARG);
+                p99 = row_rank<false>(P.t_first + ob, P.trace.arrival_us + tb, nullptr, n, rank, hist[0], S CTR_CK_FLAG_ARG);
             }
         }
         if (kTpot && many > 0) {
@@ -442,13 +582,8 @@ __global__ void __launch_bounds__(kMaxThreads, 2) goodput_kernel(const GoodputPa
                 // (its barriers order the divided values)
                 p99_tpot = kept_rank(cand_s + cap, (int)n_cand[1], rank - below, hist[0], S CTR_CK_FLAG_ARG);
             } else {
-                auto tpot_of = [&](int64_t k, int64_t& v) {
-                    const int32_t ok = ck_ld(P.trace.true_out, tb + k, trace_len, bad);
-                    if (ok < 2) return false;
-                    v = (ck_ld(P.t_done, ob + k, out_len, bad) - ck_ld(P.t_first, ob + k, out_len, bad)) / (int64_t)(ok - 1);
-                    return true;
-                };
-                p99_tpot = radix_rank(tpot_of, n, rank, hist[0], S CTR_CK_FLAG_ARG);
+                p99_tpot = row_rank<true>(P.t_done + ob, P.t_first + ob, P.trace.true_out + tb, n, rank, hist[0],
+                                    S CTR_CK_FLAG_ARG);
             }
         }
 #if CTR_BOUNDS_CHECK
@@ -507,7 +642,8 @@ cudaError_t launch_rows(const GoodputParams& p, int sms, cudaStream_t stream)
     const bool later = kTpot && (kMaxThreads * 2 / threads) * (block_bytes + (size_t)p.cand_cap * 12) <= 196 * 1024;
     const auto k = later ? goodput_kernel<kHash, kTpot, kTpot> : goodput_kernel<kHash, kTpot, false>;
     size_t dyn_bytes = (size_t)p.cand_cap * 4 * (later ? 3 : kTpot ? 2 : 1);
-    if (kTpot && dyn_bytes < kHistWords * 4) dyn_bytes = kHistWords * 4;
+    const size_t sampled = (kHistWords + (size_t(1) << p.sample_log2)) * 4;
+    if (kTpot && dyn_bytes < sampled) dyn_bytes = sampled;
     cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxCand * 12);
     if (err != cudaSuccess) return err;
     int per_sm = 0;

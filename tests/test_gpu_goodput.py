@@ -56,11 +56,11 @@ def test_goodput_adversarial_times(orc):
             assert (met[r], p99[r]) == orc.goodput(sc, row, tf[r], td[r]), (N, r)
 
 
-@pytest.mark.parametrize("crowd", [1, 511, 512, 513, 3000])
+@pytest.mark.parametrize("crowd", [1, 127, 128, 129, 511, 512, 513, 3000])
 def test_goodput_crowded_p99_bin(orc, crowd):
     """The P99's rank falls among `crowd` requests whose TTFTs share one
-    logarithmic bin: up to 512 of them are counted out exactly in shared
-    memory, more go to the radix select; TTFTs at 0 and 2^32 - 1 (the ends of
+    logarithmic bin: up to 128 of the kept ones are counted out in shared
+    memory, more are selected by their digits; TTFTs at 0 and 2^32 - 1 (the ends of
     the binned range) and a row with one TTFT of 2^32 (outside it) ride along."""
     ctr = need_gpu()
     rng = np.random.default_rng(crowd)
@@ -297,3 +297,34 @@ def test_longest_row_meeting_every_slo(N, slow):
         ctr.ctr_simulate(sc, [W.CALIBRATED], [W.POLICY_RR], tr, 1, N, tf, td, out[0], st,
                          ctr.simulate_workspace(sc, 1, N, "cuda"), met_count=out[1], p99_ttft_us=out[2])
         assert (int(st), int(out[1])) == (0, N)
+
+
+@pytest.mark.parametrize("N", [600, 1500, 9_001, 10_000, 70_002])
+@pytest.mark.parametrize("shape", ["narrow", "tie_below", "tie_at", "ties", "two_ties", "small", "wide_bins", "end_bin"])
+def test_crowded_thresholds(orc, N, shape):
+    """Rows whose values crowd where the threshold falls (narrow: a third within 1 %), with equal values below the P99, at
+    it or everywhere, in the bins of single integers, in those of 2^24 and more, and in the last one: counted again by
+    finer parts, left out, or selected from memory."""
+    ctr = need_gpu()
+    rng = np.random.default_rng(N + len(shape))
+    R = 3
+    u = rng.random((R, N))
+    v = {"narrow": np.floor(15_500 * np.exp(0.008 * rng.standard_normal((R, N)))),
+         "tie_below": np.where(u < 0.88, rng.integers(14_000, 15_000, (R, N)), np.where(u < 0.975, 15_204, rng.integers(15_204, 15_300, (R, N)))),
+         "tie_at": np.where(u < 0.9, rng.integers(14_000, 15_204, (R, N)), np.where(u < 0.995, 15_204, 15_205)),
+         "ties": np.full((R, N), 15_204), "two_ties": np.where(u < 0.985, 15_203, 15_204), "small": rng.integers(0, 40, (R, N)),
+         "wide_bins": 3_000_000_000 + rng.integers(0, 20_000_000, (R, N)),
+         "end_bin": (1 << 32) - 1 - rng.integers(0, 1 << 20, (R, N))}[shape].astype(np.int64)
+    o = rng.integers(1, 400, (R, N))
+    arr = np.sort(rng.integers(0, 10**9, (R, N)), axis=1)
+    tf = arr + v
+    td = tf + rng.permutation(v.T).T * np.maximum(o - 1, 0)
+    trh = {"arrival_us": arr, "prompt_len": np.ones((R, N)), "true_out": o, "pred_out": np.ones((R, N)),
+           "slo_class": rng.integers(0, 2, (R, N))}
+    tr, tfd, tdd = to_dev(trh), torch.from_numpy(tf).cuda(), torch.from_numpy(td).cuda()
+    met, p99 = _goodput(ctr, W.SimCfg(), tr, R, 1, N, tfd, tdd)
+    tpot = _p99_tpot(ctr, W.SimCfg(), tr, R, 1, N, tfd, tdd)
+    for r in range(R):
+        row = {k: a[r] for k, a in trh.items()}
+        assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), row, tf[r], td[r]), r
+        assert tpot[r] == orc.p99_tpot({"true_out": o[r]}, tf[r], td[r]), r
