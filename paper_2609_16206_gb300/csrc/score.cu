@@ -238,11 +238,13 @@ __device__ void warp_envelope(Smem& sm, const ScoreParams& P, int s, int n_inst,
 // The same walk for pools of 65 to 256 instances, one line to a thread and eight
 // warps (a named barrier of their own) to a class.  A step is each warp's argmin,
 // one barrier, and the argmin over the eight warps' candidates, which every warp
-// takes for itself.  Bound by that chain, about 0.3 us a segment: 2^20 requests x
-// 256 random instances take 5.3 us, 56 us when the block compared all pairs (a
-// Pareto test, intervals and ranks) before the first request; 6 M x 200: 53.5 ->
-// 18.9 us.  An envelope of every line, which states seen in practice have none
-// of, takes 24 / 41 / 76 us at 65 / 128 / 256 instances (18 / 29 / 92 before).
+// takes for itself.  The crossings there only order the lines; the left ends are
+// divided once per segment afterwards, correctly rounded and off the chain.  Bound
+// by that chain, about 0.25 us a segment: 6,001 requests x 256 random instances
+// take 5.1 us, 52 us when the block compared all pairs (a Pareto test, intervals and
+// ranks) before the first request.  An envelope of every line, which states seen in
+// practice have none of, takes 21 / 36 / 67 us at 65 / 128 / 256 instances
+// (17 / 28 / 90 before; 32 / 58 / 100 with a correctly rounded division a step).
 __device__ void group_envelope(Smem& sm, const ScoreParams& P, int n_inst, int tid)
 {
     const float inf = __int_as_float(0x7f800000);
@@ -255,7 +257,6 @@ __device__ void group_envelope(Smem& sm, const ScoreParams& P, int n_inst, int t
     sm.la[s][j] = a;
     sm.lm[s][j] = m;
     // the line of least (x, j) over the class's threads, -1 when none has one; also publishes la and lm
-    uint32_t gx = 0;  // the key of its x
     auto group_argmin = [&](bool has, float x, int buf) {
         const uint32_t kx = has ? fkey(x) : 0xffffffffu;
         const uint32_t mx = __reduce_min_sync(0xffffffffu, kx);
@@ -263,34 +264,37 @@ __device__ void group_envelope(Smem& sm, const ScoreParams& P, int n_inst, int t
         if (lane == 0) sm.cand[s][buf][w] = make_uint2(mx, mj);
         asm volatile("bar.sync %0, 256;" ::"r"(s + 1) : "memory");
         const uint2 c = lane < 8 ? sm.cand[s][buf][lane] : make_uint2(0xffffffffu, 0xffffffffu);
-        gx = __reduce_min_sync(0xffffffffu, c.x);
+        const uint32_t gx = __reduce_min_sync(0xffffffffu, c.x);
         return (int)__reduce_min_sync(0xffffffffu, c.x == gx ? c.y : 0xffffffffu);
     };
     int ci = group_argmin(live, a, 0);
     bool more = ci >= 0;
     if (!more) ci = 0;  // no finite line at all (outside the input contract): line 0
-    if (j == 0) {
-        sm.seg_lo[s][0] = 0.0f;
-        sm.seg_id[s][0] = ci;
-    }
-    float ca = sm.la[s][ci], cm = sm.lm[s][ci], x_cur = 0.0f;
+    if (j == 0) sm.seg_id[s][0] = ci;
+    float ca = sm.la[s][ci], cm = sm.lm[s][ci];
     int nseg = 1;
     while (more && nseg < n_inst) {  // the same for all threads of the class
-        const float x = __fdividef(a - ca, cm - m);
+        // a crossing good to 2 ulp, for the order only; scaled, as __fdividef gives 0 for denominators above 2^126
+        const float x = __fdividef(0.25f * (a - ca), 0.25f * (cm - m));
         const int bi = group_argmin(live && m < cm && x == x, x, nseg & 1);
         if (bi < 0) break;  // no line of smaller slope is left
         ca = sm.la[s][bi];
         cm = sm.lm[s][bi];
-        x_cur = fmaxf(__uint_as_float((gx & 0x80000000u) ? gx ^ 0x80000000u : ~gx), x_cur);  // fkey undone
-        if (j == 0) {
-            sm.seg_lo[s][nseg] = x_cur;
-            sm.seg_id[s][nseg] = bi;
-        }
+        if (j == 0) sm.seg_id[s][nseg] = bi;
         ++nseg;
     }
+    // the left ends, correctly rounded and kept non-decreasing against rounding: a maximum over the segments before
     asm volatile("bar.sync %0, 256;" ::"r"(s + 1) : "memory");
-    if (j < nseg) sm.seg_e[s][j] = seg_entry(sm, P, s, sm.seg_id[s][j]);
-    if (j >= 1 && j <= 8) reinterpret_cast<float*>(&sm.brk[s][0])[j - 1] = j < nseg ? sm.seg_lo[s][j] : inf;
+    const int id = j < nseg ? sm.seg_id[s][j] : 0, before = j > 0 && j < nseg ? sm.seg_id[s][j - 1] : id;
+    float lo = j > 0 && j < nseg ? (sm.la[s][id] - sm.la[s][before]) / (sm.lm[s][before] - sm.lm[s][id]) : 0.0f;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) lo = fmaxf(lo, __shfl_up_sync(0xffffffffu, lo, off));
+    if (lane == 31) sm.cand[s][0][w].x = __float_as_uint(lo);  // (every warp has read the last candidates: the barrier above)
+    asm volatile("bar.sync %0, 256;" ::"r"(s + 1) : "memory");
+    for (int v = 0; v < w; ++v) lo = fmaxf(lo, __uint_as_float(sm.cand[s][0][v].x));
+    if (j < nseg) sm.seg_lo[s][j] = lo;
+    if (j < nseg) sm.seg_e[s][j] = seg_entry(sm, P, s, id);
+    if (j >= 1 && j <= 8) reinterpret_cast<float*>(&sm.brk[s][0])[j - 1] = j < nseg ? lo : inf;
     if (j == 0) sm.nseg[s] = nseg;
 }
 

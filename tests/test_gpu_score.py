@@ -244,3 +244,22 @@ def test_chained_launches_read_completed_outputs():
         torch.cuda.synchronize()
         assert not torch.isnan(c1).any() and not torch.isnan(c2).any(), it
         assert torch.equal(am2, ref_am) and torch.equal(c2, ref_c), it
+
+
+@pytest.mark.parametrize("n_inst", [65, 200, 256])
+def test_wide_pool_slopes_past_2_to_126(n_inst):
+    """Slopes so far apart that a division which flushes the reciprocals of denominators above 2^126 puts the crossing of
+    the first two lines at 0 (the cost is 1e37 against 2e36 there)."""
+    ctr = need_gpu()
+    consts = np.array([1, 1, 0, 1, 0, 1, 1, 0, 0, 1, 0.5, 1, 1], np.float32)
+    Q, kap = np.full(n_inst, 2e38, np.float32), np.zeros(n_inst, np.float32)
+    i, j = n_inst // 3, n_inst - 2
+    Q[i], kap[i], Q[j], kap[j] = 0, 2e38, 1e37, 1e37
+    oh = np.linspace(0, 0.2, 4_001, dtype=np.float32)
+    p, A, cls = np.ones_like(oh), np.zeros(n_inst, np.float32), (np.arange(oh.size) % 4).astype(np.uint8)
+    am, cost = _run(ctr, p, oh, cls, Q, A, kap, consts)
+    c64 = Q.astype(np.float64)[None] + p[:, None] + oh[:, None].astype(np.float64) * (1 + kap.astype(np.float64)[None])
+    c64 *= np.where(cls == 1, 0.5, 1.0)[:, None]
+    best = c64.min(1)
+    assert np.all(c64[np.arange(oh.size), am] <= best * (1 + 1e-6))  # a tie within fp32 roundings may go either way
+    assert np.max(np.abs(cost - best) / best) <= 2e-6
