@@ -423,71 +423,56 @@ __global__ void __launch_bounds__(kWalkWarps * 32, 7) trace_kernel(const TracePa
     }
 }
 
-// A cluster of blocks per replica, each block a contiguous range of its chunks.
-// Pass 1 writes every request's lengths, and its work within the chunk into its
-// arrival's place; a block scan of the chunks' totals and the totals of the
-// cluster's blocks before it (read from their shared memory) give each chunk
-// its start; pass 2 turns the work into arrival times, each thread reading back
-// what it wrote itself.  Bound by the chain of a chunk (Philox, quantile,
-// logarithm) and the two cluster barriers: 1 x 10,000 requests take 8.3 us
-// (Poisson) and 11.5 us (MMPP: every warp steps over the windows before its
-// chunks), 408 and 459 us with one warp.
+// A cluster of blocks per replica, each warp a contiguous run of its chunks.
+// Pass 1 writes every request's lengths, and its work within the run into its
+// arrival's place; the totals of the runs before it, of its block's warps and of
+// the cluster's blocks (read from their shared memory), give each run its start;
+// pass 2 turns the work into arrival times, each thread reading back what it
+// wrote itself.  Bound by the chain of a chunk (Philox, quantile, logarithm) and
+// the two cluster barriers: 1 x 10,000 requests take 7.9 us (Poisson) and 12.2 us
+// (MMPP: every warp steps over the windows before its run), 356 and 430 us with
+// one warp.  Nothing but the totals is shared: with every chunk's total in shared
+// memory (8 bytes each, 128 KB for the longest) 650 x 450,000 took 13.6 ms, 10.3 now.
 constexpr int kSplitWarps = 8;
 constexpr int kMaxCluster = 16;
-constexpr int64_t kMaxChunks = 16384;  // of one block: 2^23 requests over a full cluster
 __global__ void __launch_bounds__(kSplitWarps * 32) trace_split_kernel(const TraceParams P)
 {
     __shared__ uint32_t queue[kSplitWarps][96];
     __shared__ uint64_t warp_sum[kSplitWarps];
     __shared__ uint64_t block_sum;
-    extern __shared__ uint64_t chunk[];  // work of each chunk, then the block's work before it
     cg::cluster_group cluster = cg::this_cluster();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t blocks = (int64_t)cluster.num_blocks(), rank = (int64_t)cluster.block_rank();
     const int64_t r = blockIdx.x / blocks;
-    const int64_t n_chunks = (P.n_req + 31) / 32;
-    const int64_t c0 = n_chunks * rank / blocks, c1 = n_chunks * (rank + 1) / blocks;
+    const int64_t n_chunks = (P.n_req + 31) / 32, runs = blocks * kSplitWarps, run = rank * kSplitWarps + wid;
+    const int64_t c0 = n_chunks * run / runs, c1 = n_chunks * (run + 1) / runs;
     const Stream S = stream_of(P, r);
     const int64_t row = r * P.n_req;
 
-    for (int64_t c = c0 + wid; c < c1; c += kSplitWarps) {
+    uint64_t work = 0;  // of the run so far
+    for (int64_t c = c0; c < c1; ++c) {
         const int64_t k = c * 32 + lane;
-        const uint64_t lam = scan32((uint64_t)request(P, S, row, k, queue[wid], lane), lane);
+        const uint64_t lam = work + scan32((uint64_t)request(P, S, row, k, queue[wid], lane), lane);
         if (k < P.n_req) P.out.arrival_us[row + k] = (int64_t)lam;
-        if (lane == 31) chunk[c - c0] = lam;
+        work = __shfl_sync(0xffffffffu, lam, 31);
     }
+    if (lane == 0) warp_sum[wid] = work;
     __syncthreads();
-    // exclusive scan of the chunks' work: a run of chunks per thread, then over the block's threads
-    const int64_t m = c1 - c0, per = (m + blockDim.x - 1) / blockDim.x;
-    const int64_t b = threadIdx.x * per, e = b + per < m ? b + per : m;
-    uint64_t sum = 0;
-    for (int64_t i = b; i < e; ++i) sum += chunk[i];
-    const uint64_t incl = scan32(sum, lane);
-    if (lane == 31) warp_sum[wid] = incl;
-    __syncthreads();
-    uint64_t before = incl - sum;
-    for (int w = 0; w < wid; ++w) before += warp_sum[w];
-    for (int64_t i = b; i < e; ++i) {
-        const uint64_t v = chunk[i];
-        chunk[i] = before;
-        before += v;
-    }
-    if (threadIdx.x == 0) {
-        uint64_t all = 0;
-        for (int w = 0; w < kSplitWarps; ++w) all += warp_sum[w];
-        block_sum = all;
-    }
-    cluster.sync();  // every block's sum is there (and this block's chunks)
-    uint64_t offset = lane < rank ? *cluster.map_shared_rank(&block_sum, lane) : 0;
+    uint64_t offset = 0;
+    for (int w = 0; w < wid; ++w) offset += warp_sum[w];
+    if (wid == kSplitWarps - 1 && lane == 0) block_sum = offset + work;
+    cluster.sync();  // every block's sum is there
+    uint64_t others = lane < rank ? *cluster.map_shared_rank(&block_sum, lane) : 0;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) offset += __shfl_xor_sync(0xffffffffu, offset, off);
+    for (int off = 16; off > 0; off >>= 1) others += __shfl_xor_sync(0xffffffffu, others, off);
+    offset += others;
 
     Arrivals arr;
     arr.start(P, S, lane);
-    for (int64_t c = c0 + wid; c < c1; c += kSplitWarps) {
+    for (int64_t c = c0; c < c1; ++c) {
         const int64_t k = c * 32 + lane;
         const bool live = k < P.n_req;
-        const uint64_t lam = live ? offset + chunk[c - c0] + (uint64_t)P.out.arrival_us[row + k] : 0;
+        const uint64_t lam = live ? offset + (uint64_t)P.out.arrival_us[row + k] : 0;
         const int64_t t = arr.time(P, S, lam, live, lane);
         if (live) P.out.arrival_us[row + k] = t;
     }
@@ -504,13 +489,14 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream)
     if (err != cudaSuccess) return err;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    // Split replicas while a warp each leaves the GPU idle or waiting on one warp's chain (1.5 us a chunk
-    // against 2 us for the 8 of a block): 1 x 10,000 requests 459 -> 11.5 us, 64 x 10,000 469 -> 34,
-    // 1,024 x 5,000 271 -> 167, 3,000 x 5,000 457 -> 441.  Short traces leave a block's warps idle and stay
-    // with one warp a replica unless there are very few of them: 1,000 x 64 takes 6.3 us there, 13 us split.
-    // The fewer its chunks, the fewer replicas pay for a block's barriers and uneven last chunks (MMPP, split / whole:
-    // 512 requests 1,520 replicas 36 / 37 us, 1,824 41 / 37, 3,040 64 / 51; 1,000 requests 2,128 78 / 80, 2,432 88 / 80;
-    // 2,500 requests 2,736 217 / 228, 3,040 240 / 228; 4,000 requests 3,040 371 / 421).
+    // Split replicas while a warp each leaves the GPU idle or waiting on one warp's chain (1.4 us a chunk): 64 x 10,000
+    // requests 446 -> 35 us.  Short traces leave a block's warps idle and stay with one warp a replica unless there are
+    // very few of them: 1,000 x 64 takes 6.8 us there, 6.9 split; 152 x 128 9.0 and 6.1.  The fewer its chunks, the fewer
+    // replicas pay for a block's barriers and uneven runs (MMPP, split / whole: 512 requests 1,520 replicas 32 / 36 us,
+    // 1,824 38 / 36, 3,040 59 / 49; 1,000 requests 2,280 77 / 79, 2,432 81 / 79; 2,500 requests 2,736 200 / 226, 3,040
+    // 221 / 227; 4,000 requests 3,040 339 / 355, 3,344 371 / 416; 20,000 requests 3,040 1,632 / 1,744, 4,096 2,180 /
+    // 2,354): the lines of the longer traces are where the split crossed with its chunks' totals in shared memory, and
+    // on the safe side of where it would now.
     const int64_t n_chunks = (p.n_req + 31) / 32;
     const int64_t most = (int64_t)sms * (n_chunks < 32 ? 10 : n_chunks < 64 ? 15 : n_chunks < 100 ? 18 : 20);
     if (p.n_replicas <= most && n_chunks >= (p.n_replicas <= sms ? 4 : 16)) {
@@ -518,20 +504,14 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream)
         // replicas, as they are slow to place (16 x 10,000: 19.6 us with 8 blocks, 16.8 with 16; 64 x 10,000: 34 us
         // with 4 or 8, 40 with 16)
         int cluster = 1;
-        while (cluster < kMaxCluster &&
-               ((p.n_replicas * cluster * 2 <= (cluster < 8 ? sms * 8 : sms * 2) && n_chunks >= cluster * 4) ||
-                n_chunks > (int64_t)cluster * kMaxChunks))
+        while (cluster < kMaxCluster && p.n_replicas * cluster * 2 <= (cluster < 8 ? sms * 8 : sms * 2) &&
+               n_chunks >= cluster * 4)
             cluster *= 2;
-        const size_t smem = (size_t)((n_chunks + cluster - 1) / cluster) * 8;
-        err = cudaFuncSetAttribute(trace_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(kMaxChunks * sizeof(uint64_t)));
-        if (err != cudaSuccess) return err;
         err = cudaFuncSetAttribute(trace_split_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (err != cudaSuccess) return err;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(p.n_replicas * cluster));
         cfg.blockDim = dim3(kSplitWarps * 32);
-        cfg.dynamicSmemBytes = smem;
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -539,6 +519,12 @@ cudaError_t launch_trace(const TraceParams& p, cudaStream_t stream)
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+        int fit = 1;
+        if (cluster > 8 && (cudaOccupancyMaxActiveClusters(&fit, trace_split_kernel, &cfg) != cudaSuccess || fit < 1)) {
+            (void)cudaGetLastError();  // more than the portable 8 blocks: not on every device (the query takes 0.2 us)
+            cfg.gridDim.x = (unsigned)(p.n_replicas * 8);
+            attr[0].val.clusterDim.x = 8;
+        }
         err = cudaLaunchKernelEx(&cfg, trace_split_kernel, p);
         if (err != cudaSuccess) return err;
         return cudaGetLastError();

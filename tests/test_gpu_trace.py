@@ -48,6 +48,14 @@ def test_split_replicas_bit_identical(orc, tc, R, N):
     _compare(orc, tc, tr, R, N, 5, rows=sorted({0, 1, R // 2, R - 1} & set(range(R))))
 
 
+@pytest.mark.parametrize("R,N", [(1, 1 << 23), (1, (1 << 23) - 31), (9, 600_001), (650, 200_000)])
+def test_long_split_replicas(orc, R, N):
+    """The longest traces: runs of hundreds to thousands of chunks a warp, in clusters of 16, 8 and 1."""
+    ctr = need_gpu()
+    tc = W.replica_sweep().trace
+    _compare(orc, tc, gen(ctr, tc, R, N, 3), R, N, 3, rows=sorted({0, R - 1}))
+
+
 def test_empty_sizes(orc):
     ctr = need_gpu()
     gen(ctr, W.TraceCfg(), 0, 100)
