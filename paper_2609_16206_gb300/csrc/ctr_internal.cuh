@@ -115,8 +115,7 @@ struct TraceParams {
     int32_t arrival_kind;
     int64_t rate[2];
     uint64_t rate_recip[2];     // floor((2^64 - 1) / rate)
-    int64_t dwell_mean_us;
-    float dwell_mean_f;         // dwell_mean_us rounded once to fp32
+    float dwell_mean_f;         // the mean dwell in us, rounded once to fp32
     float prompt_mu, prompt_sigma, short_mu, short_sigma, long_mu, long_sigma, noise_sigma;
     struct Clip {
         int32_t lo, hi;

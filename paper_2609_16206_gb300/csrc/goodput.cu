@@ -676,7 +676,7 @@ cudaError_t launch_goodput(const GoodputParams& given, cudaStream_t stream)
     if (err != cudaSuccess) return err;
     GoodputParams p = given;
     p.pairs = p.n_req % 2 == 0 &&
-              ((uintptr_t)p.trace.arrival_us | (uintptr_t)p.t_first | (uintptr_t)p.t_done | (uintptr_t)p.kmix) % 16 == 0 &&
+              ((uintptr_t)p.trace.arrival_us | (uintptr_t)p.t_first | (uintptr_t)p.t_done) % 16 == 0 &&
               (uintptr_t)p.trace.true_out % 8 == 0 && (uintptr_t)p.trace.slo_class % 2 == 0;
     // one request in 32 to 64 of a long row, so that the kept values, 3 % of a row at 1,024 samples, still have room:
     // 1,200 rows of 200,000: 1,093 us, 3,980 with 1,024 samples (past kMaxCand a row takes the radix select)

@@ -1365,12 +1365,12 @@ namespace {
 
 // The instantiation with the most registers at which all of the launch's
 // persistent warps are resident at once (its launch bound promises that many
-// blocks an SM): 4 blocks / 128 registers for launches of up to 16 warps an SM,
-// which wait on their own chains and not for issue slots, so spills and
-// constants re-read from the parameter bank cost time (against 7 blocks, 1,500
-// requests: 2,048 document rows 4.8 -> 4.3 ms, 2,080 learned rows 4.5 -> 4.2);
-// 7 blocks / 72 registers for one wave of up to 28; else 8 / 64, where more
-// warps hide more latency.
+// blocks an SM): 4 blocks / up to 128 registers (90 to 105 are used) for launches
+// of up to 16 warps an SM, which wait on their own chains and not for issue slots,
+// so spills and constants re-read from the parameter bank cost time (against 7
+// blocks, 1,500 requests: 2,048 document rows 4.8 -> 4.3 ms, 2,080 learned rows
+// 4.5 -> 4.2); 7 blocks / 72 registers for one wave of up to 28; else 8 / 64,
+// where more warps hide more latency.
 template <int G, int kMode>
 cudaError_t launch_width(const SimParams& p, int blocks, cudaStream_t stream)
 {

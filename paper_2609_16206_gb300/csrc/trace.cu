@@ -398,7 +398,8 @@ struct Arrivals {
 
 // One warp per replica.  Bound by instruction issue (Philox, the fp32 variates): 4,096 x 20,000 MMPP requests took
 // 2.95 ms (980 warp-instructions a chunk of 32) with a tail path per variate, scalar polynomials and one dwell at a
-// time, and take 2.26 ms (804, 0.68 of the issue slots); 21 B a request are 0.76 TB/s of stores.  72 registers keep the 27 warps an SM of that size in one wave.
+// time, and take 2.26 ms (804, 0.72 of the issue slots); 21 B a request are 0.76 TB/s of stores.  At 64 registers the
+// 27 warps an SM of that size are one wave.
 constexpr int kWalkWarps = 4;
 __global__ void __launch_bounds__(kWalkWarps * 32, 7) trace_kernel(const TraceParams P)
 {
