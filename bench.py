@@ -611,17 +611,17 @@ def run_ours(args, rank, world, local_rank):
 # request, keyed by a hash of the simulator's code: a stale entry
 # (the kernel changed since the counters were taken) reports null.
 SIM_SLICE_COUNTERS: dict = {
-    "64afa14802b7ece5": {"warp_inst_per_routed": 22899474615 / 81_920_000,
-                         "thread_inst_per_warp_inst": 184476552804 / 22899474615,
-                         "dram_bytes_per_routed": (1615253504 + 2389551616) / 81_920_000,
+    "40cbb605b87f83fd": {"warp_inst_per_routed": 23234051072 / 81_920_000,
+                         "thread_inst_per_warp_inst": 185820114766 / 23234051072,
+                         "dram_bytes_per_routed": (1615846656 + 2390868224) / 81_920_000,
                          "slice": "ncu on one launch of 2,560 replicas x 8,000 requests x 4 policies "
-                                  "(81.92 M routed requests): 2.290e10 warp-instructions, 1.845e11 thread-"
-                                  "instructions, 1.615 GB DRAM read + 2.390 GB written"},
+                                  "(81.92 M routed requests): 2.323e10 warp-instructions, 1.858e11 thread-"
+                                  "instructions, 1.616 GB DRAM read + 2.391 GB written"},
 }
 
 # DRAM bytes of one scorer launch (2^20 requests x 64 instances) inside the step.
 SCORE_DRAM_PER_LAUNCH: dict = {
-    "44c805c02eec218b": {"read": 9467648.0, "write": 0.0},
+    "7d38351f9f4172da": {"read": 9470464.0, "write": 0.0},
 }
 
 

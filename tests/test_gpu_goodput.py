@@ -20,7 +20,7 @@ def _goodput(ctr, sc, tr, R, rows_per, N, tf, td):
 
 @pytest.mark.parametrize("wl,R,N", [(W.single_replica(), 1, 2000), (W.replica_sweep(), 8, 5000),
                                     (W.large_pool(rate_mreq=34_000), 2, 3000), (W.replica_sweep(), 3, 37),
-                                    (W.replica_sweep(), 1, 45_000)])  # rows past the shared-memory staging
+                                    (W.replica_sweep(), 1, 45_000)])  # long rows: wider blocks
 def test_goodput_matches_oracle(orc, wl, R, N):
     ctr = need_gpu()
     tr = gen(ctr, wl.trace, R, N)
