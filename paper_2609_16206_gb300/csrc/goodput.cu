@@ -379,6 +379,7 @@ __device__ int64_t kept_rank(const uint32_t* cand, int c, int64_t rank, uint32_t
     __syncthreads();
     const int m = (int)S.n_few;
     if (m > kFew) {
+        __syncthreads();  // n_few has been read (a bin of a single value has no digits to select by, so no barrier there)
         const int64_t lo = B == 0 ? 0 : bin_floor(B);
         return radix_rank(KeptValues{cand}, c, r_in, lo, B == 0 ? 0 : bits_of((uint64_t)(bin_floor(B + 1) - lo - 1)), hist,
                           S CTR_CK_FLAG_ARG);

@@ -26,6 +26,7 @@ std::vector<Fiber> fibers;
 std::vector<std::vector<uint64_t>> out;  // of each warp's last exchange
 char* stacks = nullptr;
 size_t stacks_bytes = 0;
+std::vector<char> shared;  // dynamic, of the block that runs
 ucontext_t scheduler;
 int current = -1;
 uint64_t block_value = 0;
@@ -120,8 +121,11 @@ uint64_t block_or(uint64_t v)
     return block_value;
 }
 
-void launch(int64_t blocks, int threads, const std::function<void()>& thread)
+void* dynamic_shared() { return shared.data(); }
+
+void launch(int64_t blocks, int threads, size_t dynamic_bytes, const std::function<void()>& thread)
 {
+    shared.assign(dynamic_bytes, 0);
     body = &thread;
     gridDim = dim3((unsigned)blocks);
     blockDim = dim3((unsigned)threads);

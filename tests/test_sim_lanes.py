@@ -1,4 +1,4 @@
-"""The simulator's kernels on the CPU (simlanes), the lanes of a warp as far
+"""The kernels of the simulator and of the goodput pass on the CPU (simlanes), the lanes of a warp as far
 apart as its barriers allow: every row the oracle's, and no access to shared
 structures that only a lockstep warp would keep in order."""
 import numpy as np
@@ -113,3 +113,27 @@ def test_failure_inside_a_run_of_steps(orc, lanes, name, sc, rows, status, ws_ro
     assert (res["status"] == status).all(), res["status"]
     sc = sc.replace(prefill_batch_tokens=1)
     check(orc, lanes, sc, [W.CALIBRATED], [W.POLICY_RR, W.POLICY_LEARNED], [tr], 0, ws_rows=ws_rows)
+
+
+@pytest.mark.parametrize("order", [0, 1, 7])
+@pytest.mark.parametrize("N", [1, 130, 1500, 3001])
+@pytest.mark.parametrize("shape", ["spread", "narrow", "tie_below", "equal", "small", "negative", "wide"])
+def test_goodput(orc, lanes, shape, N, order):
+    """The goodput pass with both P99s: thresholds of spread, crowded and equal values, bins of a single value with more
+    members than are counted out (small), and rows that are selected from memory."""
+    rng = np.random.default_rng(N)
+    R, u = 2, rng.random((2, N))
+    v = {"spread": rng.integers(1, 10**7, (R, N)), "narrow": np.floor(15_500 * np.exp(0.008 * rng.standard_normal((R, N)))),
+         "tie_below": np.where(u < 0.88, rng.integers(14_000, 15_000, (R, N)), np.where(u < 0.975, 15_204, 15_290)),
+         "equal": np.full((R, N), 15_204), "small": rng.integers(1, 9, (R, N)), "negative": rng.integers(-500, 3, (R, N)),
+         "wide": (1 << 33) + rng.integers(0, 1000, (R, N))}[shape].astype(np.int64)
+    o = rng.integers(1, 400, (R, N))
+    tr = {"arrival_us": np.sort(rng.integers(0, 10**9, (R, N)), axis=1), "prompt_len": np.ones((R, N)), "true_out": o,
+          "pred_out": np.ones((R, N)), "slo_class": rng.integers(0, 2, (R, N))}
+    tf = tr["arrival_us"] + v
+    td = tf + rng.permutation(v.T).T * np.maximum(o - 1, 0)
+    (met, p99, tpot), races, stuck = simlanes.goodput(lanes, W.SimCfg(), tr, tf, td, order)
+    assert (races, stuck) == (0, 0)
+    for r in range(R):
+        assert (met[r], p99[r]) == orc.goodput(W.SimCfg(), {k: x[r] for k, x in tr.items()}, tf[r], td[r])
+        assert tpot[r] == orc.p99_tpot({"true_out": o[r]}, tf[r], td[r])
